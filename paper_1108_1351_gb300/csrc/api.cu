@@ -177,24 +177,6 @@ int DeviceScratch::alloc(void** p, size_t bytes, cudaStream_t s)
 
 // ---------------------------------------------------------------- stage plumbing
 
-__global__ void fill_f32_kernel(float* p, long long count, float v)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x)
-        p[i] = v;
-}
-
-int fill_f32(float* p, long long count, float v, cudaStream_t s)
-{
-    if (count <= 0) return KMEANS2_OK;
-    int grid = (int)((count + 255) / 256);
-    if (grid > 1024) grid = 1024;
-    ++g_launches;
-    fill_f32_kernel<<<grid, 256, 0, s>>>(p, count, v);
-    KM2_CUDA(cudaGetLastError());
-    return KMEANS2_OK;
-}
-
 // True if p is memory the current device addresses as device memory.
 bool is_device_ptr(const void* p)
 {
@@ -220,8 +202,7 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
     KM2_TRY(ws.alloc((void**)&w.c.c64, kd * sizeof(double), s));
     KM2_TRY(ws.alloc((void**)&w.c.c32, kd * sizeof(float), s));
     KM2_TRY(ws.alloc((void**)&w.c.c32t, (size_t)w.c.dpad * w.c.kpad * sizeof(float), s));
-    const long long cn_len = std::max((long long)w.c.kpad, (long long)(k + 255) / 256 * 256);
-    KM2_TRY(ws.alloc((void**)&w.c.cnorm, (size_t)cn_len * sizeof(float), s));
+    KM2_TRY(ws.alloc((void**)&w.c.cnorm, (size_t)center_norm_len(k, w.c.kpad) * sizeof(float), s));
     KM2_TRY(ws.alloc((void**)&w.acc.s_lo, kd * 8, s));
     KM2_TRY(ws.alloc((void**)&w.acc.s_hi, kd * 8, s));
     KM2_TRY(ws.alloc((void**)&w.acc.cnt, (size_t)k * 8, s));
@@ -230,10 +211,6 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
     KM2_TRY(ws.alloc((void**)&w.clus, (size_t)kClusSlots * k * sizeof(double), s));
     KM2_TRY(ws.alloc((void**)&w.traj_J, (size_t)max_iter * sizeof(double), s));
     KM2_TRY(ws.alloc((void**)&w.traj_shift, (size_t)max_iter * sizeof(double), s));
-    KM2_CUDA(cudaMemsetAsync(w.c.c32t, 0, (size_t)w.c.dpad * w.c.kpad * sizeof(float), s));
-    // padding centers: the largest finite key, so that packing an index into
-    // its low mantissa bits never makes a NaN and it never wins or ties
-    KM2_TRY(fill_f32(w.c.cnorm, cn_len, FLT_MAX, s));
     // (the split layout: a fit may switch from FP16 to split BF16 between stages)
     if (tc16_form(w.form)) KM2_TRY(ws.alloc((void**)&w.cb, bf16_cb_bytes(d, k, 0), s));
     return KMEANS2_OK;
@@ -466,12 +443,7 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
               int64_t* traj_n_host = nullptr, bool probe16 = false)
 {
     NvtxRange stage_range(name);
-    size_t kd = (size_t)w.c.k * d;
-    KM2_CUDA(cudaMemsetAsync(w.acc.s_lo, 0, kd * 8, s));
-    KM2_CUDA(cudaMemsetAsync(w.acc.s_hi, 0, kd * 8, s));
-    KM2_CUDA(cudaMemsetAsync(w.acc.cnt, 0, (size_t)w.c.k * 8, s));
-    KM2_TRY(launch_center_prep(w.c, w.st, s));
-    KM2_TRY(launch_stage_init(w.st, d, tol, max_iter, s));
+    KM2_TRY(launch_stage_begin(w.c, w.acc, w.st, tol, max_iter, s));
     KM2_TRY(launch_qsum(X, n, d, w.st, s, sm_count));
     KM2_TRY(prepare_stage_points(X, n, d, w, *w.ws, s));
     bool finished = false;
@@ -1162,11 +1134,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
     KM2_TRY(stream_pass(cs, s, [&](long long, const float* Xc, long long rows) {
         return launch_maxabs(Xc, rows, d, w.st, s, ws.sm_count);
     }));
-    KM2_CUDA(cudaMemsetAsync(w.acc.s_lo, 0, kd * 8, s));
-    KM2_CUDA(cudaMemsetAsync(w.acc.s_hi, 0, kd * 8, s));
-    KM2_CUDA(cudaMemsetAsync(w.acc.cnt, 0, (size_t)k * 8, s));
-    KM2_TRY(launch_center_prep(w.c, w.st, s));
-    KM2_TRY(launch_stage_init(w.st, d, tol, max_iter, s));
+    KM2_TRY(launch_stage_begin(w.c, w.acc, w.st, tol, max_iter, s));
     StageState ss;
     std::memset(&ss, 0, sizeof(ss));
     for (int it = 0; it < max_iter; ++it) {

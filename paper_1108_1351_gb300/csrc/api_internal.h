@@ -95,9 +95,16 @@ int launch_gather(const float* X, int d, const long long* subset, long long m, f
                   StageState* st, cudaStream_t s, int sm_count);
 int launch_init_centers(const float* Xs, int d, const long long* pos, int k, double* c64,
                         cudaStream_t s);
-int launch_center_prep(const Centers& c, StageState* st, cudaStream_t s);
-int launch_stage_init(StageState* st, int d, double tol, int max_iter, cudaStream_t s);
-// clus: kClusSlots*k doubles of scratch; tr: the stage's optional per-iteration records.
+// Floats of Centers::cnorm (padding included).
+inline long long center_norm_len(int k, int kpad)
+{
+    const long long r = (long long)(k + 255) / 256 * 256;
+    return r > kpad ? r : kpad;
+}
+// Loop state, scales, zero sums, the centers' copies (st zeroed, max |x| recorded).
+int launch_stage_begin(const Centers& c, const Accum& acc, StageState* st, double tol,
+                       int max_iter, cudaStream_t s);
+// clus: kClusSlots*k 8-byte words of scratch; tr: the stage's optional per-iteration records.
 int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const TrajDev& tr,
                     double* clus, unsigned long long cond_handle, int use_cond, cudaStream_t s);
 int launch_recheck(const float* X, int d, const Centers& c, int* labels, const int* list,

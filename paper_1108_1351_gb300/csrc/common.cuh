@@ -55,10 +55,12 @@ struct StageState {
     unsigned long long q[4];
     // single-pass FP16 form: rows its bound left undecided, summed over the stage
     long long undecided16_total;
+    // finalize: CTAs done with their centers (the last one reduces and resets it)
+    unsigned int ticket;
 };
 
-// Per-center scratch of finalize, in doubles per center (finalize_center_warp).
-constexpr int kClusSlots = 7;
+// Per-center scratch of finalize, in 8-byte words per center (finalize_center_warp).
+constexpr int kClusSlots = 6;
 
 constexpr int kErrNonFinite = 1;
 constexpr int kErrRange = 2;       // max|x| >= 2^50

@@ -4,11 +4,13 @@
 //               (the integer that J is formed from, Eq. 3)
 //   gather      X_s = rows of X at the subset indices (Algorithm: the per% subset)
 //   init        initial centers = chosen points of X_s (Algorithm: random initial centers)
-//   center_prep FP32 / transposed copies of the FP64 centers and ||c||^2
-//   stage_init  fixed-point scales and loop state of one stage
+//   stage_begin fixed-point scales and loop state of one stage, zero sums, FP32 /
+//               transposed copies of the FP64 centers and ||c||^2
 //   finalize    new centers = cluster means (Lloyd's method, Section 4.1), the
 //               largest movement (stop test, Sections 5-6), J (Eq. 3)
 //   recheck     FP64 re-evaluation of near-tie points (ties -> lowest index)
+#include <algorithm>
+#include <cfloat>
 #include <cstdint>
 
 #include "api_internal.h"
@@ -29,6 +31,20 @@ __device__ __forceinline__ unsigned int warp_max_u32(unsigned int v)
     return v;
 }
 
+// Block-wide maximum into st->maxabs_bits: one atomic per block.
+__device__ __forceinline__ void block_max_to(unsigned int m, StageState* st)
+{
+    __shared__ unsigned int wm[32];
+    m = warp_max_u32(m);
+    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : 0u;
+        m = warp_max_u32(m);
+        if (threadIdx.x == 0 && m) atomicMax(&st->maxabs_bits, m);
+    }
+}
+
 __global__ void maxabs_kernel(const float* __restrict__ X, long long count, int vec4,
                               StageState* st)
 {
@@ -39,6 +55,7 @@ __global__ void maxabs_kernel(const float* __restrict__ X, long long count, int 
     if (vec4) {
         const float4* X4 = reinterpret_cast<const float4*>(X);
         long long n4 = count >> 2;
+#pragma unroll 4
         for (long long i = tid; i < n4; i += stride) {
             float4 v = __ldg(X4 + i);
             m = max(m, max(max(abs_bits(v.x), abs_bits(v.y)), max(abs_bits(v.z), abs_bits(v.w))));
@@ -46,35 +63,82 @@ __global__ void maxabs_kernel(const float* __restrict__ X, long long count, int 
         done = n4 << 2;
     }
     for (long long i = done + tid; i < count; i += stride) m = max(m, abs_bits(__ldg(X + i)));
-    m = warp_max_u32(m);
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(&st->maxabs_bits, m);
+    block_max_to(m, st);
 }
 
-// Exact sum of s^2 over count coordinates, s = to_fixed(x, 2^F) (the same
-// integers the cluster sums add), into st->q.  Each thread sums < 2^26
-// squares below 2^92 in 128 bits; one wide_add4 per warp.
+// Partial sum of s^2 over coordinates, s = to_fixed(x, 2^F) = a 2^24 + b with |a| <=
+// 2^22, |b| <= 2^23: three 64-bit sums (wide multiply-adds), folded into 128
+// bits every 2^16 coordinates at most (each term is below 2^47).
+struct QSum {
+    unsigned __int128 total = 0;
+    unsigned long long aa = 0, bb = 0;
+    long long ab = 0;
+    __device__ __forceinline__ void add(float x, float scale)
+    {
+        const float t = x * scale;                                   // |t| < 2^46, exact
+        const float v = fmaf(t, 5.9604644775390625e-8f, 12582912.0f);   // 1.5 2^23 + rint(t 2^-24)
+        const int a = __float_as_int(v) - 0x4b400000;
+        const int b = __float2int_rn(fmaf(v - 12582912.0f, -16777216.0f, t));
+        aa += (unsigned long long)((long long)a * a);
+        ab += (long long)a * b;
+        bb += (unsigned long long)((long long)b * b);
+    }
+    __device__ __forceinline__ void fold()
+    {
+        total += ((unsigned __int128)aa << 48) + bb + (unsigned __int128)((__int128)ab * ((__int128)1 << 25));
+        aa = bb = 0;
+        ab = 0;
+    }
+};
+
+// Exact sum of s^2 over count coordinates (the same integers the cluster sums
+// add), into st->q.  Memory-bound: ~9 instructions per coordinate (one 128-bit
+// product and sum per coordinate took 2.5x the time of reading X; n = 5e5, d =
+// 128: 125 us).
 __global__ void qsum_kernel(const float* __restrict__ X, long long count, int vec4,
                             StageState* st)
 {
+    __shared__ unsigned long long wl[8], wh[8];
     if (st->error) return;
     const float scale = st->scaleF;
-    unsigned __int128 a = 0;
+    QSum q;
     long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long stride = (long long)gridDim.x * blockDim.x;
     long long done = 0;
     if (vec4) {
         const float4* X4 = reinterpret_cast<const float4*>(X);
         long long n4 = count >> 2;
-        for (long long i = tid; i < n4; i += stride) {
-            float4 v = __ldg(X4 + i);
-            a += sq_fixed(v.x, scale) + sq_fixed(v.y, scale) + sq_fixed(v.z, scale) +
-                 sq_fixed(v.w, scale);
+        for (long long i = tid; i < n4;) {
+            const long long end = min(n4, i + stride * (1 << 14));   // 2^16 coordinates
+#pragma unroll 4
+            for (; i < end; i += stride) {
+                const float4 v = __ldg(X4 + i);
+                q.add(v.x, scale);
+                q.add(v.y, scale);
+                q.add(v.z, scale);
+                q.add(v.w, scale);
+            }
+            q.fold();
         }
         done = n4 << 2;
     }
-    for (long long i = done + tid; i < count; i += stride) a += sq_fixed(__ldg(X + i), scale);
-    a = warp_sum_u128(a);
-    if ((threadIdx.x & 31) == 0 && a) wide_add4(st->q, a);
+    int left = 1 << 16;
+    for (long long i = done + tid; i < count; i += stride) {
+        q.add(__ldg(X + i), scale);
+        if (--left == 0) { q.fold(); left = 1 << 16; }
+    }
+    q.fold();
+    unsigned __int128 a = warp_sum_u128(q.total);
+    if ((threadIdx.x & 31) == 0) {
+        wl[threadIdx.x >> 5] = (unsigned long long)a;
+        wh[threadIdx.x >> 5] = (unsigned long long)(a >> 64);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += ((unsigned __int128)wh[w] << 64) | wl[w];
+        if (a) wide_add4(st->q, a);
+    }
 }
 
 __global__ void gather_kernel(const float* __restrict__ X, int d,
@@ -91,8 +155,7 @@ __global__ void gather_kernel(const float* __restrict__ X, int d,
         Xs[e] = v;
         mx = max(mx, abs_bits(v));
     }
-    mx = warp_max_u32(mx);
-    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&st->maxabs_bits, mx);
+    block_max_to(mx, st);
 }
 
 __global__ void init_centers_kernel(const float* __restrict__ Xs, int d,
@@ -108,63 +171,79 @@ __global__ void init_centers_kernel(const float* __restrict__ Xs, int d,
     }
 }
 
-// One CTA: FP32 copies and ||c_j||^2 of every center.
-__global__ void center_prep_kernel(Centers c, StageState* st)
+// Start of a stage (st zeroed, maxabs_bits set): loop state and scales, zero
+// sums and counts, the centers' FP32 copies (padding: zeros in c32t, the largest
+// finite float in cnorm, so that packing an index into its low mantissa bits
+// never makes a NaN and it never wins or ties), ||c_j||^2 and their maximum,
+// rounded up.  One warp per center over many CTAs (one CTA for all centers took
+// 149 us at k = 1024, d = 128), and one launch where three memsets, two fills and
+// two kernels did it.
+__global__ void __launch_bounds__(256) stage_begin_kernel(Centers c, Accum acc, StageState* st,
+                                                          double tol, int max_iter, long long cn_len)
 {
-    __shared__ double red[1024];
-    center_prep_block(c, st, red);
+    const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    if (gt == 0) stage_init_dev(st, c.d, tol, max_iter);
+    const long long kd = (long long)c.k * c.d;
+    for (long long e = gt; e < kd; e += stride) { acc.s_lo[e] = 0; acc.s_hi[e] = 0; }
+    for (long long e = gt; e < c.k; e += stride) acc.cnt[e] = 0;
+    for (long long e = c.k + gt; e < cn_len; e += stride) c.cnorm[e] = FLT_MAX;
+    const long long tot = (long long)c.dpad * c.kpad;
+    for (long long e = gt; e < tot; e += stride) {
+        const int t = (int)(e / c.kpad), j = (int)(e - (long long)t * c.kpad);
+        if (t >= c.d || j >= c.k) c.c32t[e] = 0.0f;
+    }
+    const int lane = threadIdx.x & 31;
+    double mx = 0.0;
+    for (long long j = gt >> 5; j < c.k; j += stride >> 5) {
+        double nn = 0.0;
+        for (int t = lane; t < c.d; t += 32) {
+            const double v = c.c64[j * c.d + t];
+            nn = fma(v, v, nn);
+            c.c32[j * c.d + t] = (float)v;
+            c.c32t[(long long)t * c.kpad + j] = (float)v;
+        }
+        nn = warp_sum_f64(nn);
+        if (lane == 0) c.cnorm[j] = (float)nn;
+        mx = fmax(mx, nn);
+    }
+    // non-negative floats order as their bits; rounding up keeps the order
+    if (lane == 0 && mx > 0.0)
+        atomicMax(reinterpret_cast<unsigned int*>(&st->cmax2), __float_as_uint(__double2float_ru(mx)));
 }
 
-__global__ void stage_init_kernel(StageState* st, int d, double tol, int max_iter)
-{
-    stage_init_dev(st, d, tol, max_iter);
-}
-
-// One CTA.  New centers, movement, J; loop control for the next iteration.
-__global__ void __launch_bounds__(1024) finalize_kernel(Accum acc, Centers c, StageState* st,
-                                                        TrajDev tr, double* clus,
-                                                        unsigned long long handle, int use_cond)
+// New centers (one warp each, many CTAs), then, in the CTA that finishes last,
+// movement, J and loop control for the next iteration.
+__global__ void __launch_bounds__(256) finalize_kernel(Accum acc, Centers c, StageState* st,
+                                                       TrajDev tr, double* clus,
+                                                       unsigned long long handle, int use_cond)
 {
     __shared__ FinalizeSmem sm;
+    __shared__ int last;
     if (st->error) {
-        if (threadIdx.x == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
             st->done = 1;
             if (use_cond) cudaGraphSetConditional(handle, 0u);
         }
         return;
     }
-    finalize_block(acc, c, st, tr, clus, sm);
-    if (threadIdx.x == 0 && use_cond) cudaGraphSetConditional(handle, st->done ? 0u : 1u);
-}
-
-// Many CTAs: the new centers, one warp per center (large k * d).
-__global__ void __launch_bounds__(256) finalize_centers_kernel(Accum acc, Centers c,
-                                                               StageState* st, TrajDev tr,
-                                                               double* clus)
-{
-    if (st->error) return;
     const double inv = st->inv_scaleF;
     const int it = st->iter;
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int j = gw; j < c.k; j += nw) finalize_center_warp(acc, c, inv, j, clus, tr, it);
-}
-
-// One CTA after finalize_centers_kernel: movement, J, loop control.
-__global__ void __launch_bounds__(1024) finalize_reduce_kernel(int k, StageState* st,
-                                                               TrajDev tr, const double* clus,
-                                                               unsigned long long handle,
-                                                               int use_cond)
-{
-    __shared__ FinalizeSmem sm;
-    if (st->error) {
-        if (threadIdx.x == 0) {
-            st->done = 1;
-            if (use_cond) cudaGraphSetConditional(handle, 0u);
-        }
-        return;
+    for (int j = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); j < c.k;
+         j += (int)((gridDim.x * blockDim.x) >> 5))
+        finalize_center_warp(acc, c, inv, j, clus, tr, it);
+    if (gridDim.x > 1) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) st->ticket = 0;
+    } else {
+        __syncthreads();
     }
-    finalize_reduce_block(k, st, tr, clus, sm);
+    finalize_reduce_block(c.k, acc.cnt, st, tr, clus, sm);
     if (threadIdx.x == 0 && use_cond) cudaGraphSetConditional(handle, st->done ? 0u : 1u);
 }
 
@@ -251,42 +330,24 @@ int launch_init_centers(const float* Xs, int d, const long long* pos, int k, dou
     return KMEANS2_OK;
 }
 
-int launch_center_prep(const Centers& c, StageState* st, cudaStream_t s)
+int launch_stage_begin(const Centers& c, const Accum& acc, StageState* st, double tol,
+                       int max_iter, cudaStream_t s)
 {
+    const long long cn_len = center_norm_len(c.k, c.kpad);
+    const long long work = std::max((long long)c.k * 32, (long long)c.dpad * c.kpad / 4);
     ++g_launches;
-    center_prep_kernel<<<1, 1024, 0, s>>>(c, st);
+    stage_begin_kernel<<<(int)std::min(1024ll, (work + 255) / 256), 256, 0, s>>>(c, acc, st, tol,
+                                                                               max_iter, cn_len);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }
-
-int launch_stage_init(StageState* st, int d, double tol, int max_iter, cudaStream_t s)
-{
-    ++g_launches;
-    stage_init_kernel<<<1, 1, 0, s>>>(st, d, tol, max_iter);
-    KM2_CUDA(cudaGetLastError());
-    return KMEANS2_OK;
-}
-
-// k * d from which the center updates run on many CTAs instead of one.
-constexpr long long kSplitFinalizeWork = 16384;
 
 int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const TrajDev& tr,
                     double* clus, unsigned long long cond_handle, int use_cond, cudaStream_t s)
 {
-    if ((long long)c.k * c.d >= kSplitFinalizeWork) {
-        // spread the k center updates over the GPU, then reduce in one CTA
-        // (the same per-center arithmetic and reduction order as one CTA)
-        int blocks = (c.k + 7) / 8;
-        if (blocks > 1024) blocks = 1024;
-        g_launches += 2;
-        finalize_centers_kernel<<<blocks, 256, 0, s>>>(acc, c, st, tr, clus);
-        KM2_CUDA(cudaGetLastError());
-        finalize_reduce_kernel<<<1, 1024, 0, s>>>(c.k, st, tr, clus, cond_handle, use_cond);
-        KM2_CUDA(cudaGetLastError());
-        return KMEANS2_OK;
-    }
     ++g_launches;
-    finalize_kernel<<<1, 1024, 0, s>>>(acc, c, st, tr, clus, cond_handle, use_cond);
+    finalize_kernel<<<std::min(1024, (c.k + 7) / 8), 256, 0, s>>>(acc, c, st, tr, clus, cond_handle,
+                                                                 use_cond);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }

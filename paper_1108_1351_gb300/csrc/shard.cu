@@ -265,16 +265,11 @@ int run_local_pass(kmeans2_shard* sh, kmeans2_exchange* next)
 int resume_maxabs(kmeans2_shard* sh, kmeans2_exchange* next)
 {
     cudaStream_t s = sh->s;
-    const size_t kd = (size_t)sh->k * sh->d;
     ++g_launches;
     maxabs_xchg_kernel<<<1, 1, 0, s>>>(sh->w.st, sh->x, 0);
     KM2_CUDA(cudaGetLastError());
-    KM2_CUDA(cudaMemsetAsync(sh->w.acc.s_lo, 0, kd * 8, s));
-    KM2_CUDA(cudaMemsetAsync(sh->w.acc.s_hi, 0, kd * 8, s));
-    KM2_CUDA(cudaMemsetAsync(sh->w.acc.cnt, 0, (size_t)sh->k * 8, s));
-    KM2_TRY(launch_center_prep(sh->w.c, sh->w.st, s));
-    KM2_TRY(launch_stage_init(sh->w.st, sh->d, sh->stage == 0 ? sh->tol_fast : sh->tol,
-                              sh->max_iter, s));
+    KM2_TRY(launch_stage_begin(sh->w.c, sh->w.acc, sh->w.st, sh->stage == 0 ? sh->tol_fast : sh->tol,
+                               sh->max_iter, s));
     StageState st;
     KM2_CUDA(cudaMemcpyAsync(&st, sh->w.st, sizeof(st), cudaMemcpyDeviceToHost, s));
     KM2_CUDA(cudaStreamSynchronize(s));

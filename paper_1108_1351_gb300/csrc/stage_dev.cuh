@@ -22,7 +22,7 @@ __device__ __forceinline__ double warp_sum_f64(double v)
 }
 
 // FP32 copies and ||c_j||^2 of every center; st->cmax2 = max_j ||c_j||^2 rounded
-// up.  Whole block; warps stride over centers; fixed reduction order.
+// up.  Whole block; warps stride over centers.
 // red: blockDim.x doubles of shared memory.
 static __device__ void center_prep_block(Centers c, StageState* st, double* red)
 {
@@ -180,16 +180,13 @@ __device__ __forceinline__ double u256_to_double(U256 a)
 
 // One warp: the new center j (its cluster mean; an empty cluster keeps its
 // center) with its FP32 copies and ||c_j||^2, and center j's terms of the
-// movement, of J and of the empty count in clus (kClusSlots k doubles):
+// movement and of J in clus (kClusSlots k words):
 //   clus[j]          ||c_j' - c_j||^2
-//   clus[k + j]      N_j ||c_j - mu_j||^2 - frac(T_j / N_j) 2^-2F
+//   clus[k + j]      sum_t (N_j c_jt - s_jt 2^-F)^2 = N_j^2 ||c_j - mu_j||^2
 //   clus[2k + j]     ||c_j'||^2
-//   clus[3k + j]     1 if the cluster is empty
-//   clus[4k + 3j..]  floor(T_j / N_j) as three 64-bit limbs
+//   clus[3k + 3j..]  T_j as three 64-bit limbs
 // where s_jt = the exact integer sum of the cluster's fixed-point coordinates,
-// mu_j = s_j 2^-F / N_j its mean and T_j = ||s_j||^2, so that over all clusters
-// J = (sum s^2 - sum_j T_j / N_j) 2^-2F + sum_j N_j ||c_j - mu_j||^2
-//   = sum_j sum_{i in j} ||x_i - c_j||^2   (Eq. 3, on the fixed-point values).
+// mu_j = s_j 2^-F / N_j its mean and T_j = ||s_j||^2; finalize_reduce_block divides.
 // Iteration it's records of center j go to tr.centers / tr.counts when those are set.
 static __device__ __forceinline__ void finalize_center_warp(const Accum& acc, const Centers& c,
                                                             double inv, int j, double* clus,
@@ -207,7 +204,8 @@ static __device__ __forceinline__ void finalize_center_warp(const Accum& acc, co
         long long e = (long long)j * d + t;
         const unsigned long long lo = acc.s_lo[e], hi = acc.s_hi[e];
         const __int128 v = (__int128)(long long)hi * (__int128)4294967296LL + (__int128)lo;
-        double S = (double)v * inv;
+        // v to FP64 in one rounding: |v >> 32| < 2^50, both halves exact
+        const double S = fma((double)(long long)(v >> 32), 4294967296.0, (double)(unsigned)v) * inv;
         // carry the low word's upper half into the high word (same value):
         // every pass adds at most 2 n < 2^32 low parts below 2^32 each, so
         // the low word cannot wrap however many delta passes follow
@@ -239,125 +237,183 @@ static __device__ __forceinline__ void finalize_center_warp(const Accum& acc, co
     t_lo = warp_sum_u128(t_lo);
     t_hi = warp_sum_u128(t_hi);
     if (lane == 0) {
-        unsigned long long* qw = reinterpret_cast<unsigned long long*>(clus + 4 * k) + 3ll * j;
-        double v = 0.0;
-        unsigned __int128 q_hi = 0;
-        unsigned long long q_lo = 0;
-        if (N > 0) {
-            // floor(T / N) and T mod N by long division (N < 2^63)
-            t_hi += t_lo >> 64;
-            const unsigned long long un = (unsigned long long)N;
-            q_hi = t_hi / un;
-            const unsigned __int128 x = ((t_hi % un) << 64) | (unsigned long long)t_lo;
-            q_lo = (unsigned long long)(x / un);
-            const unsigned long long rem = (unsigned long long)(x % un);
-            v = dev2 / Nd - ((double)rem / Nd) * (inv * inv);
-        }
-        qw[0] = q_lo;
-        qw[1] = (unsigned long long)q_hi;
-        qw[2] = (unsigned long long)(q_hi >> 64);
+        t_hi += t_lo >> 64;
+        unsigned long long* qw = reinterpret_cast<unsigned long long*>(clus + 3 * k) + 3ll * j;
+        qw[0] = (unsigned long long)t_lo;
+        qw[1] = (unsigned long long)t_hi;
+        qw[2] = (unsigned long long)(t_hi >> 64);
         clus[j] = diff2;
-        clus[k + j] = v;
+        clus[k + j] = dev2;
         clus[2 * k + j] = nn;
-        clus[3 * k + j] = (N == 0) ? 1.0 : 0.0;
         c.cnorm[j] = (float)nn;
         if (tr.counts) tr.counts[(long long)it * k + j] = N;
     }
 }
 
+// floor(T / N) of a 192-bit T (three limbs, in place) for 0 < N < 2^32, and T mod
+// N: long division by 32-bit digits, each quotient digit from an FP64 product
+// with 1 / N (off by at most one: the digit is below 2^32 and the product's
+// relative error below 2^-51) and corrected exactly.
+__device__ __forceinline__ unsigned long long div192(unsigned long long (&T)[3], unsigned long long N)
+{
+    const double inv = 1.0 / (double)N;
+    unsigned long long rem = 0, Q[3] = {0ull, 0ull, 0ull};
+#pragma unroll
+    for (int i = 5; i >= 0; --i) {
+        const unsigned long long digit = (T[i >> 1] >> (32 * (i & 1))) & 0xffffffffull;
+        const unsigned long long x = (rem << 32) | digit;          // < N 2^32
+        unsigned long long q = 0;
+        if (x >= N) {
+            q = (unsigned long long)((double)x * inv);
+            long long r = (long long)(x - q * N);
+            if (r < 0) { --q; r += (long long)N; }
+            if (r >= (long long)N) { ++q; r -= (long long)N; }
+            rem = (unsigned long long)r;
+        } else {
+            rem = x;
+        }
+        Q[i >> 1] |= q << (32 * (i & 1));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) T[i] = Q[i];
+    return rem;
+}
+
 struct FinalizeSmem {
-    double r_shift[1024];
-    double r_J[1024];
-    double r_nn[1024];
-    int r_empty[1024];
+    double r_shift[32];
+    double r_J[256];
+    double r_nn[32];
+    int r_empty[32];
     unsigned __int128 r_q[32][3];
 };
 
-// Whole block (blockDim.x <= 1024, a power of two), after every center's
-// finalize_center_warp: movement, J and loop control from clus, in a fixed
-// order (thread 0 updates st).  The integer part of J, sum s^2 - sum_j
-// floor(T_j / N_j), is exact (256-bit); it is rounded to FP64 once and added
-// to the sum of the per-center remainders.  Ends with the block synchronised.
-static __device__ void finalize_reduce_block(int k, StageState* st, const TrajDev& tr,
-                                             const double* clus, FinalizeSmem& sm)
+// Whole block of 256 threads, after every center's finalize_center_warp:
+// movement, J and loop control from clus (thread 0 updates st).  J's floating
+// terms are added in one fixed order, the one of a tree over 1024 threads that
+// stride over the centers.  The integer part of J, sum s^2 - sum_j floor(T_j /
+// N_j), is exact (256-bit); it is rounded to FP64 once and added to the sum of the
+// per-center remainders:
+//   J = (sum s^2 - sum_j T_j / N_j) 2^-2F + sum_j N_j ||c_j - mu_j||^2
+//     = sum_j sum_{i in j} ||x_i - c_j||^2   (Eq. 3, on the fixed-point values).
+// A thread per center divides, so the divisions of all centers overlap (one
+// lane per warp did them before, one center after the other, with the
+// compiler's 128-bit division: 51 us for k = 50, d = 5, 134 us for k = 100, d = 37
+// in all of finalize).  Ends with the block synchronised.
+static __device__ void finalize_reduce_block(int k, const unsigned long long* cnt, StageState* st,
+                                             const TrajDev& tr, const double* clus, FinalizeSmem& sm)
 {
+    constexpr int B = 256;
     double* traj_J = tr.J;
     double* traj_shift = tr.shift;
-    const unsigned long long* qw = reinterpret_cast<const unsigned long long*>(clus + 4 * k);
-    double sh = 0.0, jj = 0.0, mx = 0.0;
+    const unsigned long long* qw = reinterpret_cast<const unsigned long long*>(clus + 3 * k);
+    const double inv = st->inv_scaleF;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double sh = 0.0, mx = 0.0;
+    double jj[4] = {0.0, 0.0, 0.0, 0.0};         // threads tid, tid + 256, .. of the 1024
     int em = 0;
     unsigned __int128 a0 = 0, a1 = 0, a2 = 0;    // sums of the limbs of floor(T_j / N_j)
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
-        sh = fmax(sh, clus[j]);
-        jj += clus[k + j];
-        mx = fmax(mx, clus[2 * k + j]);
-        em += (int)clus[3 * k + j];
-        a0 += qw[3ll * j];
-        a1 += qw[3ll * j + 1];
-        a2 += qw[3ll * j + 2];
+    for (int j0 = 0; j0 < k; j0 += 1024) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int j = j0 + B * v + tid;
+            if (j >= k) break;
+            sh = fmax(sh, __ldcg(clus + j));
+            mx = fmax(mx, __ldcg(clus + 2 * k + j));
+            const unsigned long long N = __ldcg(cnt + j);
+            double term = 0.0;
+            if ((long long)N > 0) {
+                unsigned long long T[3] = {__ldcg(qw + 3ll * j), __ldcg(qw + 3ll * j + 1),
+                                           __ldcg(qw + 3ll * j + 2)};
+                const unsigned long long rem = div192(T, N);
+                const double Nd = (double)N;
+                term = __ldcg(clus + k + j) / Nd - ((double)rem / Nd) * (inv * inv);
+                a0 += T[0];
+                a1 += T[1];
+                a2 += T[2];
+            }
+            jj[v] += term;
+            em += N == 0 ? 1 : 0;
+        }
     }
+    // the 1024-thread tree's first two levels, then 256 values
+    sm.r_J[tid] = (jj[0] + jj[2]) + (jj[1] + jj[3]);
     a0 = warp_sum_u128(a0);
     a1 = warp_sum_u128(a1);
     a2 = warp_sum_u128(a2);
-    if ((threadIdx.x & 31) == 0) {
-        sm.r_q[threadIdx.x >> 5][0] = a0;
-        sm.r_q[threadIdx.x >> 5][1] = a1;
-        sm.r_q[threadIdx.x >> 5][2] = a2;
+    for (int o = 16; o; o >>= 1) {
+        sh = fmax(sh, __shfl_xor_sync(0xffffffffu, sh, o));
+        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        em += __shfl_xor_sync(0xffffffffu, em, o);
     }
-    sm.r_shift[threadIdx.x] = sh;
-    sm.r_J[threadIdx.x] = jj;
-    sm.r_nn[threadIdx.x] = mx;
-    sm.r_empty[threadIdx.x] = em;
+    if (lane == 0) {
+        sm.r_shift[warp] = sh;
+        sm.r_nn[warp] = mx;
+        sm.r_empty[warp] = em;
+        sm.r_q[warp][0] = a0;
+        sm.r_q[warp][1] = a1;
+        sm.r_q[warp][2] = a2;
+    }
     __syncthreads();
-    for (int s = blockDim.x >> 1; s; s >>= 1) {
-        if ((int)threadIdx.x < s) {
-            sm.r_shift[threadIdx.x] = fmax(sm.r_shift[threadIdx.x], sm.r_shift[threadIdx.x + s]);
-            sm.r_J[threadIdx.x] += sm.r_J[threadIdx.x + s];
-            sm.r_nn[threadIdx.x] = fmax(sm.r_nn[threadIdx.x], sm.r_nn[threadIdx.x + s]);
-            sm.r_empty[threadIdx.x] += sm.r_empty[threadIdx.x + s];
+    if (warp == 0) {
+        double r[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) r[v] = sm.r_J[lane + 32 * v];
+        // levels 128, 64, 32 of the tree in this lane, 16 .. 1 across lanes
+        double J0 = ((r[0] + r[4]) + (r[2] + r[6])) + ((r[1] + r[5]) + (r[3] + r[7]));
+        for (int o = 16; o; o >>= 1) J0 += __shfl_down_sync(0xffffffffu, J0, o);
+        const bool in = lane < B / 32;
+        sh = in ? sm.r_shift[lane] : 0.0;
+        mx = in ? sm.r_nn[lane] : 0.0;
+        em = in ? sm.r_empty[lane] : 0;
+        a0 = in ? sm.r_q[lane][0] : (unsigned __int128)0;
+        a1 = in ? sm.r_q[lane][1] : (unsigned __int128)0;
+        a2 = in ? sm.r_q[lane][2] : (unsigned __int128)0;
+        a0 = warp_sum_u128(a0);
+        a1 = warp_sum_u128(a1);
+        a2 = warp_sum_u128(a2);
+        for (int o = 16; o; o >>= 1) {
+            sh = fmax(sh, __shfl_xor_sync(0xffffffffu, sh, o));
+            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            em += __shfl_xor_sync(0xffffffffu, em, o);
         }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        // D = sum s^2 - sum_j floor(T_j / N_j)  (>= 0: Cauchy-Schwarz per cluster)
-        U256 D = {{0ull, 0ull, 0ull, 0ull}};
-        U256 Tq = {{0ull, 0ull, 0ull, 0ull}};
-        u256_add_at(D, (unsigned __int128)st->q[0], 0);
-        u256_add_at(D, (unsigned __int128)st->q[1] << 32, 0);
-        u256_add_at(D, (unsigned __int128)st->q[2], 1);
-        u256_add_at(D, (unsigned __int128)st->q[3] << 32, 1);
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            u256_add_at(Tq, sm.r_q[w][0], 0);
-            u256_add_at(Tq, sm.r_q[w][1], 1);
-            u256_add_at(Tq, sm.r_q[w][2], 2);
+        if (lane == 0) {
+            // D = sum s^2 - sum_j floor(T_j / N_j)  (>= 0: Cauchy-Schwarz per cluster)
+            U256 D = {{0ull, 0ull, 0ull, 0ull}};
+            U256 Tq = {{0ull, 0ull, 0ull, 0ull}};
+            u256_add_at(D, (unsigned __int128)st->q[0], 0);
+            u256_add_at(D, (unsigned __int128)st->q[1] << 32, 0);
+            u256_add_at(D, (unsigned __int128)st->q[2], 1);
+            u256_add_at(D, (unsigned __int128)st->q[3] << 32, 1);
+            u256_add_at(Tq, a0, 0);
+            u256_add_at(Tq, a1, 1);
+            u256_add_at(Tq, a2, 2);
+            u256_neg(Tq);
+            for (int i = 0; i < 4; ++i) u256_add_at(D, (unsigned __int128)Tq.w[i], i);
+            double J = u256_to_double(D) * (inv * inv) + J0;
+            if (J < 0.0) J = 0.0;   // only rounding of an exactly zero objective can go below
+            double shift = sqrt(sh);
+            int it = st->iter;
+            if (traj_J) traj_J[it] = J;
+            if (traj_shift) traj_shift[it] = shift;
+            st->J = J;
+            st->shift = shift;
+            st->empty = em;
+            st->cmax2 = __double2float_ru(mx);
+            st->iter = it + 1;
+            int conv = shift <= st->tol;
+            st->converged = conv;
+            st->done = conv || (it + 1 >= st->max_iter);
+            st->mode = kModeDelta;
+            st->rechecked_total += st->recheck_count;
+            st->recheck_count = 0;
         }
-        u256_neg(Tq);
-        for (int i = 0; i < 4; ++i) u256_add_at(D, (unsigned __int128)Tq.w[i], i);
-        const double inv = st->inv_scaleF;
-        double J = u256_to_double(D) * (inv * inv) + sm.r_J[0];
-        if (J < 0.0) J = 0.0;   // only rounding of an exactly zero objective can go below
-        double shift = sqrt(sm.r_shift[0]);
-        int it = st->iter;
-        if (traj_J) traj_J[it] = J;
-        if (traj_shift) traj_shift[it] = shift;
-        st->J = J;
-        st->shift = shift;
-        st->empty = sm.r_empty[0];
-        st->cmax2 = __double2float_ru(sm.r_nn[0]);
-        st->iter = it + 1;
-        int conv = shift <= st->tol;
-        st->converged = conv;
-        st->done = conv || (it + 1 >= st->max_iter);
-        st->mode = kModeDelta;
-        st->rechecked_total += st->recheck_count;
-        st->recheck_count = 0;
     }
     __syncthreads();
 }
 
-// Whole block (blockDim.x <= 1024, a power of two).  New centers, movement,
-// J; loop control for the next iteration (thread 0 updates st).  clus: 4 k
-// doubles of scratch.  Ends with the block synchronised.
+// Whole block of 256 threads.  New centers, movement, J; loop control for the
+// next iteration (thread 0 updates st).  clus: kClusSlots k words of scratch.
+// Ends with the block synchronised.
 static __device__ void finalize_block(Accum acc, Centers c, StageState* st, TrajDev tr,
                                       double* clus, FinalizeSmem& sm)
 {
@@ -366,7 +422,7 @@ static __device__ void finalize_block(Accum acc, Centers c, StageState* st, Traj
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int j = warp; j < c.k; j += nw) finalize_center_warp(acc, c, inv, j, clus, tr, it);
     __syncthreads();
-    finalize_reduce_block(c.k, st, tr, clus, sm);
+    finalize_reduce_block(c.k, acc.cnt, st, tr, clus, sm);
 }
 
 // FP32 D_j = ||c_j||^2 - 2 x.c_j of one point against centers j0 + 32 i

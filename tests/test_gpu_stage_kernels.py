@@ -1,0 +1,58 @@
+"""The kernels that start and finish an iteration (GPU): the stage start (centers
+spread over warps and CTAs, padding), the exact sum of squares, and the update
+with its 192-by-32-bit divisions and its last-CTA reduction.  Center counts lie
+around 8 per CTA, 256 per reduction pass, 1024 per reduction round and the cap
+of 1024 CTAs; data reach the ends of the fixed-point range."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_helpers import assert_centers_close, assert_J_close, to_np
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import oracle  # noqa: E402
+import paper_1108_1351_gb300 as km  # noqa: E402
+
+
+def _check(X, C):
+    cn, lab, J, sh, em = km.step(torch.as_tensor(X, device="cuda"), torch.as_tensor(C, device="cuda"),
+                                 precision="fp32")
+    ocn, olab, oJ, osh, oem = oracle.lloyd_step(X, C)
+    assert np.array_equal(to_np(lab), olab)
+    assert_centers_close(to_np(cn), ocn, X)
+    assert_J_close(J, oJ, X)
+    assert abs(sh - osh) <= 1e-10 * max(osh, 1.0)
+    assert em == oem
+
+
+@pytest.mark.parametrize("k", [1, 7, 8, 9, 255, 256, 257, 1023, 1025, 2049, 8200])
+@pytest.mark.parametrize("d", [1, 5, 33])
+def test_center_counts(k, d):
+    rng = np.random.default_rng(k + d)
+    X = rng.normal(size=(2 * k + 37, d)).astype(np.float32) * 3.0
+    C = X[rng.choice(X.shape[0], size=k, replace=False)].astype(np.float64)
+    _check(X, C)
+
+
+@pytest.mark.parametrize("case", ["powers", "wide", "negative", "ties_of_the_grid", "constant"])
+def test_value_ranges(case):
+    rng = np.random.default_rng(3)
+    X = rng.normal(size=(5003, 6)).astype(np.float32)
+    if case == "powers":                      # at and next to powers of two, both signs
+        e = rng.integers(-3, 10, size=X.shape).astype(np.float64)
+        X = np.ldexp(1.0, e.astype(int)).astype(np.float32) * np.sign(X)
+        X[0, 0] = np.nextafter(np.float32(1024.0), np.float32(0))
+    elif case == "wide":                      # within the 2^23 below the largest value
+        X = (X * np.exp(rng.uniform(-8, 6, size=X.shape))).astype(np.float32)
+    elif case == "negative":
+        X = (-np.abs(X) - 100.0).astype(np.float32)
+    elif case == "ties_of_the_grid":          # halves of the low part's unit
+        X = (rng.integers(-2 ** 22, 2 ** 22, size=X.shape) + 0.5).astype(np.float32)
+    else:
+        X[:] = np.float32(0.1)
+    C = X[rng.choice(X.shape[0], size=11, replace=False)].astype(np.float64)
+    _check(X, C)
