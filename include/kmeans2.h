@@ -97,7 +97,11 @@ extern "C" {
                                          more than 10 % of the rows undecided; the slow
                                          stage runs FP16 if the fast stage left at most
                                          5 % per iteration, else BF16 (the other entry
-                                         points take BF16 there); FP32 otherwise */
+                                         points take BF16 there); FP32 otherwise, with a
+                                         tensor-core screen for 8 <= d <= 16: split-FP16
+                                         products decide the rows outside their error
+                                         bound, the FP32 chain the others (same labels,
+                                         centers and J; reported as FP32) */
 #define KMEANS2_PRECISION_TF32X3 3    /* cross term on the tensor cores as three TF32
                                          products of the exact hi/lo split of the FP32
                                          operands; d in {4, 8, 16, 32}, k <= 256 */
@@ -226,7 +230,7 @@ KMEANS2_API int kmeans2_fit(const float* X, int64_t n, int32_t d, int32_t k, dou
  *                is, over the CPU-GPU link (NVLink-C2C on GB300), with no
  *                staging copies and no chunk loop (same results; on GB300 the
  *                staged chunks measured faster), otherwise 2^26-row chunks.
- *  opt           precision must be FP32 or AUTO (the CUDA-core form);
+ *  opt           precision must be FP32 or AUTO (the FP32 form, screened under AUTO);
  *                use_graph is ignored (the slow stage is host-driven).
  * Errors as kmeans2_fit; KMEANS2_ERR_INVALID if X is device memory,
  * KMEANS2_ERR_UNSUPPORTED for a tensor-core precision.
@@ -557,7 +561,7 @@ KMEANS2_API int kmeans_step(const float* X, int64_t n, int32_t d, int32_t k, con
  * device memory is entirely owned by its own caching allocator or memory pool,
  * where a stray allocation could fail or fragment that pool, or a latency-
  * critical loop that must not wait on the allocator.  This entry point runs
- * kmeans_step's CUDA-core FP32 form (the form whose scratch fits the array for
+ * kmeans_step's FP32 form as under AUTO (the form whose scratch fits the array for
  * every shape within the limits below; the tensor-core forms would need a copy
  * of X) and takes its scratch from one fixed device array of 24 MiB compiled
  * into the library, which every GPU that loads the library holds until the

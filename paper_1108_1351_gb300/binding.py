@@ -442,7 +442,7 @@ def fit_streamed(X, k: int, subset_fraction: float, seed: int, tol: float, max_i
     _check_devices(X, C0, cen, lab)
     opt = Options()
     lib.kmeans2_default_options(ctypes.byref(opt))
-    opt.precision = PRECISION["fp32"]
+    opt.precision = PRECISION["auto"]
     opt.tol_fast = tol_fast
     opt.init_centers = _ptr(C0) if C0 is not None else None
     opt.start_stage = start_stage

@@ -255,6 +255,8 @@ int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels,
     if (tc16_form(w.form))
         return launch_assign_bf16(X, w.xt, w.xn2, w.cb, n, d, w.c, labels, w.st, w.acc, w.list,
                                   0, s, sm_count);
+    if (w.screen && assign_mma_supported(d, w.c.k, X))
+        return launch_assign_mma(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
     return launch_assign_fp32(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
 }
 
@@ -517,6 +519,7 @@ Resolved resolve_options(const kmeans2_options* opt)
     Resolved r;
     kmeans2_default_options(&r.opt);
     if (opt) r.opt = *opt;
+    r.screen = r.opt.precision == KMEANS2_PRECISION_AUTO;
     r.stream = static_cast<cudaStream_t>(r.opt.stream);
     if (!r.stream) {
         int dev = 0;
@@ -740,6 +743,7 @@ int kmeans_step(const float* X, int64_t n, int32_t d, int32_t k, const double* c
     KM2_TRY(device_view(X, (long long)n * d, &Xd, ws, s));
     Workspace w;
     KM2_TRY(choose_form(r.opt.precision, d, k, Xd, &w.form));
+    w.screen = r.screen;
     KM2_TRY(alloc_workspace(w, ws, n, k, d, 1, s));
     bool lab_dev = is_device_ptr(labels_out) && (reinterpret_cast<uintptr_t>(labels_out) & 3) == 0;
     int* labels = lab_dev ? labels_out : nullptr;
@@ -800,6 +804,7 @@ int kmeans_step_noalloc(const float* X, int64_t n, int32_t d, int32_t k,
     // labels, centers and J.
     Workspace w;
     w.form = KMEANS2_PRECISION_FP32;
+    w.screen = true;
     KM2_TRY(alloc_workspace(w, ws, n, k, d, 1, s));
     KM2_CUDA(cudaMemcpyAsync(w.c.c64, centers_in, sizeof(double) * (size_t)k * d,
                              cudaMemcpyDeviceToDevice, s));
@@ -842,6 +847,7 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
     const long long m = kmeans2_subset_size(n, k, subset_fraction);
     Workspace w;
     KM2_TRY(choose_form(o.precision, d, k, Xd, &w.form));
+    w.screen = r.screen;
     // AUTO on a 16-bit tensor-core shape: the fast stage runs the single-pass
     // FP16 form and the slow stage keeps it only if that left few rows
     // undecided there (on tie-heavy data its second pass and the FP64 recheck
@@ -1078,6 +1084,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
 
     Workspace w;
     w.form = KMEANS2_PRECISION_FP32;
+    w.screen = r.screen;
     KM2_TRY(alloc_workspace(w, ws, std::max(m, chunk), k, d, max_iter, s));
     bool lab_dev = is_device_ptr(labels_out) && (reinterpret_cast<uintptr_t>(labels_out) & 3) == 0;
     int* labels = lab_dev ? labels_out : nullptr;

@@ -159,10 +159,17 @@ int launch_assign_fp32(const float* X, long long n, int d, const Centers& c, int
                        StageState* st, const Accum& acc, int* list, cudaStream_t s,
                        int sm_count);
 
+// assign_mma.cu: the FP32 form with a tensor-core screen (split-FP16 products
+// decide the rows outside their bound, the FP32 chain the others)
+int assign_mma_supported(int d, int k, const float* X);
+int launch_assign_mma(const float* X, long long n, int d, const Centers& c, int* labels,
+                      StageState* st, const Accum& acc, int* list, cudaStream_t s, int sm_count);
+
 // ---------------------------------------------------------------- stage plumbing (api.cu)
 // Per-stage device state of one fit: centers, exact sums, loop state, near-tie list.
 struct Workspace {
     int form = KMEANS2_PRECISION_FP32;   // distance-kernel form used by this call
+    bool screen = false;                 // FP32 form: rows go through the tensor-core screen first
     Centers c{};
     Accum acc{};
     StageState* st = nullptr;
@@ -201,6 +208,7 @@ int device_view(const float* X, long long count, const float** out, DeviceScratc
 struct Resolved {
     cudaStream_t stream;
     kmeans2_options opt;
+    bool screen;       // precision AUTO: the FP32 form may screen rows on the tensor cores
 };
 Resolved resolve_options(const kmeans2_options* opt);
 

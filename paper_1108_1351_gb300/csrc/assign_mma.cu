@@ -1,0 +1,337 @@
+// assign_mma.cu -- the FP32 form's fused distance kernel with a tensor-core
+// screen: split-FP16 products (22 significant bits per operand, FP32
+// accumulation) on mma.sync decide every row whose best center is separated by
+// more than their bound; the rest are decided by the FP32 FMA chain in the same
+// warp, and what that leaves open by the FP64 recheck (mma_dev.cuh).  Labels,
+// sums and J equal those of the CUDA-core kernels (assign_fp32.cu) bit for bit.
+//
+// assign_mma_ring (8 <= d <= 16): a warp takes 64 rows at a time from its own ring
+// of cp.async stages in shared memory (rows as they lie in X, and the old labels);
+// the centers' fragments stay in shared memory for the whole launch.  Warps never
+// wait for one another except to flush the partial sums.
+//
+// What bounds it: instruction issue and register ports, not memory (at d = 8, k
+// = 32 it reads 3.1 TB/s).  Per converged pass against the CUDA-core kernel
+// (GB300; microseconds):
+//   n 2e7 d 8 k 32   325 -> 233      n 4e6 d 16 k 100   378 -> 197
+//   n 1e7 d 12 k 16  216 -> 141      n 1e6 d 16 k 1000  783 -> 360
+//   n 4e6 d 8 k 256  428 -> 272
+// Tried and dropped: 32 rows at a time (d 8, k 32: 250); work handed out to warps
+// dynamically (balance better, ~45 more instructions per 32 rows: 275); the
+// candidate test as saturated FFMAs (250); the same screen on tcgen05 with one
+// row per lane (296: 330 instructions per 32 rows against 274, and warpgroup
+// barriers); d < 8 (precision, see mma_dev.cuh).
+#include <algorithm>
+#include <cfloat>
+#include <climits>
+#include <cstdint>
+
+#include "api_internal.h"
+#include "mma_dev.cuh"
+
+namespace km2 {
+
+namespace {
+
+constexpr int kSmemCap = 224 * 1024;       // dynamic shared memory of an SM for these kernels
+constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
+
+// Ring stages per warp: about 40-55 KB in flight per SM.
+template <int DP>
+constexpr int kStages = DP <= 8 ? 3 : 2;
+
+__device__ __forceinline__ void cp_async16_zfill(unsigned sdst, const void* gsrc, int bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sdst), "l"(gsrc), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16_u32(unsigned sdst, const void* gsrc)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sdst), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async4_u32(unsigned sdst, const void* gsrc)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sdst), "l"(gsrc) : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// UNIT: rows a warp takes at a time (32 where n is too small to give every warp 64).
+template <int DP, int NT, bool SINGLE, bool FULL, int UNIT>
+__global__ void __launch_bounds__(kThreads, SINGLE ? 3 : 2)
+assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __restrict__ labels,
+                StageState* st, Accum acc, int* __restrict__ list, int ntiles, int use_sacc)
+{
+    constexpr int S = kStages<DP>;
+    constexpr int H = UNIT / 32;
+    constexpr int kFlushSteps = kFlushPoints / (kWarps * UNIT);   // steps per int64 partial
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (st->error) return;
+    const int k = c.k, d = FULL ? DP : c.d;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const unsigned stage_bytes = 4 * UNIT * (d + 1);       // rows, then labels
+    uint32_t* sb = reinterpret_cast<uint32_t*>(smem);
+    float* sn = reinterpret_cast<float*>(sb + (size_t)ntiles * MmaCfg<DP>::BW * 32);
+    unsigned char* ring = reinterpret_cast<unsigned char*>(sn + ntiles * 8) +
+                          (size_t)warp * S * stage_bytes;
+    long long* sacc = reinterpret_cast<long long*>(reinterpret_cast<unsigned char*>(sn + ntiles * 8) +
+                                                   (size_t)kWarps * S * stage_bytes);
+    int* scnt = reinterpret_cast<int*>(sacc + (size_t)k * d);
+    const bool delta = st->mode == kModeDelta;
+    const float scaleF = st->scaleF;
+    const float thr_base = 2.0f * st->cmax2;
+    const MmaScale ms = mma_scale(st, d, MmaCfg<DP>::KS);
+
+    // step i of this CTA: rows [T tile_rows, + tile_rows), T = blockIdx.x + i gridDim.x;
+    // the warp's unit starts UNIT * warp rows into it (n < 2^31)
+    constexpr int tile_rows = kWarps * UNIT;
+    const int steps = (int)((n + tile_rows - 1) / tile_rows);
+    constexpr int NQ = (UNIT * DP + 127) / 128;         // 16-byte copies per lane and stage, at most
+    const long long row_first = (long long)blockIdx.x * tile_rows + warp * UNIT;
+    const unsigned char* xsrc = reinterpret_cast<const unsigned char*>(X + row_first * d) + 16 * lane;
+    const int* lsrc = labels + row_first + lane;
+    const long long rstep = (long long)gridDim.x * tile_rows;
+    long long left_issue = n - row_first;                // rows from the next issue's first one on
+    const unsigned ring_u32 = smem_u32(ring);
+    // the next unit's rows and labels (in a full pass those are read and not
+    // used) -> the stage at byte offset `so` of the ring; rows past n are
+    // zero-filled
+    auto issue = [&](unsigned so) {
+        const unsigned dst = ring_u32 + so + 16 * lane, ldst = ring_u32 + so + 4 * UNIT * d + 4 * lane;
+        if (left_issue >= UNIT) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                if (lane + 32 * q < UNIT / 4 * d) cp_async16_u32(dst + 512 * q, xsrc + 512 * q);
+            cp_async4_u32(ldst, lsrc);
+            if (H == 2) cp_async4_u32(ldst + 128, lsrc + 32);
+        } else {
+            const int rows = (int)max(0ll, min(left_issue, (long long)UNIT));
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int have = min(16, max(0, rows * d * 4 - 16 * (lane + 32 * q)));
+                if (lane + 32 * q < UNIT / 4 * d)
+                    cp_async16_zfill(dst + 512 * q, have ? xsrc + 512 * q : reinterpret_cast<const unsigned char*>(X), have);
+            }
+            if (lane < rows) cp_async4_u32(ldst, lsrc);
+            if (H == 2 && lane + 32 < rows) cp_async4_u32(ldst + 128, lsrc + 32);
+        }
+        cp_async_commit();
+        xsrc += rstep * d * 4;
+        lsrc += rstep;
+        left_issue -= rstep;
+    };
+#pragma unroll
+    for (int s = 0; s < S - 1; ++s) issue(s * stage_bytes);
+
+    mma_load_centers<DP>(c, ntiles, ms, sb, sn);
+    if (use_sacc) {
+        for (int e = tid; e < k * d; e += kThreads) sacc[e] = 0;
+        for (int e = tid; e < k; e += kThreads) scnt[e] = 0;
+    }
+    __syncthreads();
+
+    unsigned so = 0;                                     // the current stage's offset
+    const unsigned ring_bytes = S * stage_bytes;
+    int to_flush = kFlushSteps;
+    for (int step = blockIdx.x; step < steps; step += gridDim.x) {
+        issue(so == 0 ? ring_bytes - stage_bytes : so - stage_bytes);
+        cp_async_wait_group<S - 1>();
+        __syncwarp();
+        const float* xr = reinterpret_cast<const float*>(ring + so);
+        const int* lr = reinterpret_cast<const int*>(ring + so + 4 * UNIT * d);
+        const long long row0 = (long long)step * tile_rows + warp * UNIT;
+        const int rows = (int)min((long long)UNIT, n - row0);   // may be <= 0 in the last step
+
+        // row of this lane in half h: 32 h + 8 t + g
+        int lab[2], old[2];
+        bool open[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h >= H) { lab[h] = old[h] = -1; open[h] = false; continue; }
+            uint32_t A[2][MmaCfg<DP>::AREG];
+            float xmax = 0.0f;
+            mma_load_rows<DP, FULL>(xr + 32 * h * d, d, g, t, 0, ms.sx, A[0], xmax);
+            mma_load_rows<DP, FULL>(xr + 32 * h * d, d, g, t, 1, ms.sx, A[1], xmax);
+            lab[h] = mma_decide<DP, NT, SINGLE>(A, sb, sn, ntiles, lane, mma_thr(ms, xmax), open[h]);
+            old[h] = delta ? lr[32 * h + 8 * t + g] : -1;
+            if (32 * h + 8 * t + g >= rows) { open[h] = false; lab[h] = old[h]; }
+        }
+        if (__any_sync(0xffffffffu, open[0] || open[1])) {
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                unsigned todo = __ballot_sync(0xffffffffu, open[h]);
+                bool listed = false;
+#pragma unroll 1
+                while (todo) {
+                    const int o = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    bool op;
+                    const int l = decide_fp32_row(X + (row0 + 32 * h + 8 * (o & 3) + (o >> 2)) * d, d, c,
+                                                  thr_base, op);
+                    if (lane == o) { lab[h] = l; listed = op; }
+                }
+                recheck_append(listed, (int)(row0 + 32 * h + 8 * t + g), list, &st->recheck_count);
+                if (listed) lab[h] = old[h];             // the recheck moves it
+            }
+        }
+        if (__any_sync(0xffffffffu, lab[0] != old[0] || lab[1] != old[1])) {
+            auto add = [&](int lo, int ol, int dim, float xv) {
+                const long long v = to_fixed(xv, scaleF);
+                if (use_sacc) {
+                    atomicAdd(reinterpret_cast<unsigned long long*>(sacc + lo * d + dim), (unsigned long long)v);
+                    if (ol >= 0)
+                        atomicAdd(reinterpret_cast<unsigned long long*>(sacc + ol * d + dim), (unsigned long long)(-v));
+                } else {
+                    split_add(acc.s_lo + (long long)lo * d + dim, acc.s_hi + (long long)lo * d + dim, v);
+                    if (ol >= 0)
+                        split_add(acc.s_lo + (long long)ol * d + dim, acc.s_hi + (long long)ol * d + dim, -v);
+                }
+            };
+            auto count = [&](int lo, int ol) {
+                if (use_sacc) {
+                    atomicAdd(scnt + lo, 1);
+                    if (ol >= 0) atomicAdd(scnt + ol, -1);
+                } else {
+                    atomicAdd(acc.cnt + lo, 1ull);
+                    if (ol >= 0) atomicAdd(acc.cnt + ol, ~0ull);
+                }
+            };
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const bool moved = lab[h] != old[h] && label_ok(lab[h], k, st) && old_label_ok(old[h], k, st);
+                unsigned mv = __ballot_sync(0xffffffffu, moved);
+                if (moved) {
+                    labels[row0 + 32 * h + 8 * t + g] = lab[h];
+                    count(lab[h], old[h]);
+                }
+                if (__popc(mv) >= 12) {
+                    // many moved rows (a stage's first passes): each lane its own row
+                    const float* xo = xr + (32 * h + 8 * t + g) * d;
+                    if (moved)
+                        for (int dim = 0; dim < d; ++dim) add(lab[h], old[h], dim, xo[dim]);
+                    __syncwarp();
+                    continue;
+                }
+                // few: 32 / DP rows at a time, DP lanes per row, a coordinate each
+                const int dim = lane % DP;
+#pragma unroll 1
+                while (mv) {
+                    int o = -1;
+#pragma unroll
+                    for (int q = 0; q < 32 / DP; ++q) {
+                        if (lane / DP == q) o = __ffs(mv) - 1;
+                        mv &= mv - 1;              // 0 stays 0
+                    }
+                    const int src = o < 0 ? 0 : o;
+                    const int lo = __shfl_sync(0xffffffffu, lab[h], src);
+                    const int ol = __shfl_sync(0xffffffffu, old[h], src);
+                    if (o >= 0 && dim < d) add(lo, ol, dim, xr[(32 * h + 8 * (o & 3) + (o >> 2)) * d + dim]);
+                    __syncwarp();
+                }
+            }
+        }
+        __syncwarp();   // every lane is done with the stage before it is refilled
+        so = so + stage_bytes == ring_bytes ? 0 : so + stage_bytes;
+
+        // static flush schedule: at most 2^16 rows per int64 partial
+        if (use_sacc && (--to_flush == 0 || step + (int)gridDim.x >= steps)) {
+            to_flush = kFlushSteps;
+            __syncthreads();
+            for (int e = tid; e < k * d; e += kThreads) {
+                const long long v = sacc[e];
+                if (v) {
+                    split_add(acc.s_lo + e, acc.s_hi + e, v);
+                    sacc[e] = 0;
+                }
+            }
+            for (int e = tid; e < k; e += kThreads) {
+                const int v = scnt[e];
+                if (v) {
+                    atomicAdd(acc.cnt + e, (unsigned long long)(long long)v);
+                    scnt[e] = 0;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    cp_async_wait_group<0>();
+}
+
+template <int DP, int UNIT>
+size_t ring_bytes(int d) { return (size_t)kWarps * kStages<DP> * 4 * UNIT * (d + 1); }
+
+template <int DP, int NT, bool SINGLE, bool FULL, int UNIT>
+int launch_ring_u(const float* X, long long n, const Centers& c, int* labels, StageState* st,
+                  const Accum& acc, int* list, int ntiles, cudaStream_t s, int sm_count)
+{
+    const size_t base = mma_center_bytes(DP, ntiles) + ring_bytes<DP, UNIT>(c.d);
+    const size_t sums = (size_t)c.k * c.d * 8 + (size_t)c.k * 4;
+    const int use_sacc = base + sums <= (size_t)kSmemCap;
+    const size_t sm = base + (use_sacc ? sums : 0);
+    const void* kfn = (const void*)assign_mma_ring<DP, NT, SINGLE, FULL, UNIT>;
+    KM2_TRY(set_max_dynamic_smem(kfn, kSmemCap));
+    int per_sm = 0;
+    KM2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kThreads, sm));
+    if (per_sm < 1) return KMEANS2_ERR_UNSUPPORTED;
+    const long long steps = (n + kWarps * UNIT - 1) / (kWarps * UNIT);
+    const int grid = (int)std::max(1ll, std::min((long long)sm_count * per_sm, steps));
+    ++g_launches;
+    assign_mma_ring<DP, NT, SINGLE, FULL, UNIT><<<grid, kThreads, sm, s>>>(X, n, c, labels, st, acc,
+                                                                           list, ntiles, use_sacc);
+    KM2_CUDA(cudaGetLastError());
+    return KMEANS2_OK;
+}
+
+template <int DP, int NT, bool SINGLE>
+int launch_ring(const float* X, long long n, const Centers& c, int* labels, StageState* st,
+                const Accum& acc, int* list, int ntiles, cudaStream_t s, int sm_count)
+{
+    // 64 rows per warp and step once every warp of two or three CTAs per SM gets
+    // some; below, 32 (too few warps otherwise)
+    const bool small = n < (long long)sm_count * (SINGLE ? 3 : 2) * kWarps * 64;
+#define KM2_RING(FULL_, UNIT_) \
+    return launch_ring_u<DP, NT, SINGLE, FULL_, UNIT_>(X, n, c, labels, st, acc, list, ntiles, s, sm_count)
+    if (c.d == DP) {
+        if (small) KM2_RING(true, 32);
+        KM2_RING(true, 64);
+    }
+    if constexpr (DP > 8) {
+        if (small) KM2_RING(false, 32);
+        KM2_RING(false, 64);
+    }
+#undef KM2_RING
+    return KMEANS2_ERR_UNSUPPORTED;
+}
+
+template <int DP>
+int launch_ring_k(const float* X, long long n, const Centers& c, int* labels, StageState* st,
+                  const Accum& acc, int* list, cudaStream_t s, int sm_count)
+{
+    if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, s, sm_count);
+    if (c.k <= 32) return launch_ring<DP, 4, true>(X, n, c, labels, st, acc, list, 4, s, sm_count);
+    return launch_ring<DP, 4, false>(X, n, c, labels, st, acc, list, (c.k + 31) / 32 * 4, s, sm_count);
+}
+
+}  // namespace
+
+// d from 8 on: see the precision figures in mma_dev.cuh.
+int assign_mma_supported(int d, int k, const float* X)
+{
+    if ((reinterpret_cast<uintptr_t>(X) & 15) != 0 || d < 8 || d > 16) return 0;
+    const size_t ring = d == 8 ? ring_bytes<8, 64>(d) : ring_bytes<16, 64>(d);
+    return mma_center_bytes(mma_dp(d), (k + 31) / 32 * 4) + ring <= (size_t)kSmemCap;
+}
+
+int launch_assign_mma(const float* X, long long n, int d, const Centers& c, int* labels,
+                      StageState* st, const Accum& acc, int* list, cudaStream_t s, int sm_count)
+{
+    if (d == 8) return launch_ring_k<8>(X, n, c, labels, st, acc, list, s, sm_count);
+    return launch_ring_k<16>(X, n, c, labels, st, acc, list, s, sm_count);
+}
+
+}  // namespace km2

@@ -339,6 +339,7 @@ int shard_setup(kmeans2_shard* sh, const float* X_local, double subset_fraction,
     // on every rank after device_view
     const float* aligned = reinterpret_cast<const float*>(static_cast<uintptr_t>(256));
     KM2_TRY(choose_form(sh->opt.precision, d, k, aligned, &sh->w.form));
+    sh->w.screen = sh->opt.precision == KMEANS2_PRECISION_AUTO;
     sh->m = kmeans2_subset_size(sh->n_total, k, subset_fraction);
     long long* subset = nullptr;
     long long* bnd = nullptr;
