@@ -446,14 +446,25 @@ static __device__ __forceinline__ void recheck_d4(const float* __restrict__ x, i
 }
 
 // One warp: re-decide point i.  Pass 1: FP32 D_j for every center on the CUDA
-// cores (recheck_d4) and their minimum b1.  Pass 2: every center with
-// D_j <= b1 + tie_kappa (2 C2 + X2) + tie_abs -- a set that provably holds the FP64
-// argmin -- is evaluated exactly in the oracle's form (sum_t fma(x_t - c_t,
-// x_t - c_t, acc), t ascending) and the smallest wins, lowest index on ties.
+// cores (recheck_d4) and their minimum b1.  Pass 2: the centers with D_j <= b1 +
+// tie_kappa (2 C2 + X2) + tie_abs -- a set that provably holds the FP64 argmin -- are
+// compared by their FP64 distances and the smallest wins, lowest index on ties,
+// as in the oracle's form (sum_t fma(x_t - c_t, x_t - c_t, acc), t ascending):
+//   one candidate   it is the argmin;
+//   few, d > 16     the lanes share a candidate's coordinates: 2 d / 32 + 5 FP64
+//                   instructions each, in another order of addition, which
+//                   decides when the best two differ by more than both orders'
+//                   rounding (d + 7 and d + 1 roundings of 2^-53 at most);
+//   otherwise       a lane per candidate in the oracle's order (2 d FP64
+//                   instructions).
+// An FP64 instruction holds the SM's FP64 pipe for 16 cycles whatever its active
+// lanes, so at d = 128 the second form takes 26 instead of 256 pipe slots for a
+// pair of candidates (recheck of 8,600 points, k = 32: 82 -> 39 us).
 // The point's new label and the sums follow (delta mode: from its old label).
 // cache: per-warp shared memory of cache_cap floats for the pass-1 values
-// (pass 2 recomputes them when kpad > cache_cap or cache is null).
-static __device__ __forceinline__ void recheck_point(const float* __restrict__ X, int d,
+// (pass 2 recomputes them when kpad > cache_cap or cache is null).  Returns
+// whether the point had a single candidate.
+static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X, int d,
                                                      const Centers& c, int* __restrict__ labels,
                                                      int i, StageState* st, const Accum& acc,
                                                      float* cache, int cache_cap)
@@ -472,49 +483,97 @@ static __device__ __forceinline__ void recheck_point(const float* __restrict__ X
     for (int t = lane; t < d; t += 32) { float v = __ldg(x + t); x2 = fmaf(v, v, x2); }
     for (int o = 16; o; o >>= 1) x2 += __shfl_xor_sync(0xffffffffu, x2, o);
     float b1 = INFINITY;
+    int b1j = k;
     for (int j0 = lane; j0 < k; j0 += 128) {
         float a[4];
         recheck_d4(x, d, c, j0, a);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            if (j0 + 32 * q < k) b1 = fminf(b1, a[q]);
+            if (j0 + 32 * q < k && a[q] < b1) { b1 = a[q]; b1j = j0 + 32 * q; }
             if (cached) cache[j0 + 32 * q] = a[q];
         }
     }
+    const float lane_b1 = b1;
     for (int o = 16; o; o >>= 1) b1 = fminf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
     const float lim = b1 + kap * (c2x2 + x2) * 1.0009765625f + tie_abs(d + 1);
-    double best = DBL_MAX;
-    int bj = INT_MAX;
-    for (int j0 = lane; j0 < k; j0 += 128) {
-        float a[4];
+    // candidates of this lane (a NaN or an infinite distance counts as one)
+    auto value = [&](int j0, float a[4]) {
         if (cached) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) a[q] = cache[j0 + 32 * q];
         } else {
             recheck_d4(x, d, c, j0, a);
         }
+    };
+    int ncand = 0;
+    for (int j0 = lane; j0 < k; j0 += 128) {
+        float a[4];
+        value(j0, a);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int j = j0 + 32 * q;
-            if (j < k && a[q] <= lim) {
-                const double* cj64 = c.c64 + (long long)j * d;
-                double a2 = 0.0;
-                for (int t = 0; t < d; ++t) {
-                    double e = (double)__ldg(x + t) - cj64[t];
-                    a2 = fma(e, e, a2);
+        for (int q = 0; q < 4; ++q) ncand += (j0 + 32 * q < k && a[q] <= lim) ? 1 : 0;
+    }
+    ncand = __reduce_add_sync(0xffffffffu, ncand);
+    int bj = INT_MAX;
+    bool decided = false;
+    const bool single = ncand == 1 && lim < FLT_MAX;
+    if (single) {
+        const unsigned m = __ballot_sync(0xffffffffu, lane_b1 == b1);
+        bj = __shfl_sync(0xffffffffu, b1j, __ffs(m) - 1);
+        decided = true;
+    } else if (d > 16 && ncand * (2 * ((d + 31) / 32) + 5) < 2 * d) {
+        double s1 = DBL_MAX, s2 = DBL_MAX;       // best two sums (the same on every lane)
+        for (int jb = 0; jb < k; jb += 128) {
+            float a[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+            if (jb + lane < k) value(jb + lane, a);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                unsigned m = __ballot_sync(0xffffffffu, jb + lane + 32 * q < k && a[q] <= lim);
+                while (m) {
+                    const int j = jb + 32 * q + __ffs(m) - 1;
+                    m &= m - 1;
+                    const double* cj64 = c.c64 + (long long)j * d;
+                    double p = 0.0;
+                    for (int t = lane; t < d; t += 32) {
+                        const double e = (double)__ldg(x + t) - cj64[t];
+                        p = fma(e, e, p);
+                    }
+                    p = warp_sum_f64(p);
+                    if (p < s1) { s2 = s1; s1 = p; bj = j; }
+                    else if (p < s2) s2 = p;
                 }
-                if (a2 < best || (a2 == best && j < bj)) { best = a2; bj = j; }
             }
         }
+        decided = s2 - s1 > (double)(2 * d + 16) * 1.1102230246251565e-16 * (s1 + s2);
     }
-    // lowest (distance, index) over the lanes; the FP64 sums of squares are
-    // non-negative, so their bit patterns order as the values do and the
-    // comparison stays off the (narrow) FP64 pipe
-    unsigned long long bb = (unsigned long long)__double_as_longlong(best);
-    for (int o = 16; o; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bb, o);
-        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-        if (ob < bb || (ob == bb && oj < bj)) { bb = ob; bj = oj; }
+    if (!decided) {
+        double best = DBL_MAX;
+        bj = INT_MAX;
+        for (int j0 = lane; j0 < k; j0 += 128) {
+            float a[4];
+            value(j0, a);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + 32 * q;
+                if (j < k && a[q] <= lim) {
+                    const double* cj64 = c.c64 + (long long)j * d;
+                    double a2 = 0.0;
+                    for (int t = 0; t < d; ++t) {
+                        double e = (double)__ldg(x + t) - cj64[t];
+                        a2 = fma(e, e, a2);
+                    }
+                    if (a2 < best || (a2 == best && j < bj)) { best = a2; bj = j; }
+                }
+            }
+        }
+        // lowest (distance, index) over the lanes; the FP64 sums of squares are
+        // non-negative, so their bit patterns order as the values do and the
+        // comparison stays off the (narrow) FP64 pipe
+        unsigned long long bb = (unsigned long long)__double_as_longlong(best);
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bb, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+            if (ob < bb || (ob == bb && oj < bj)) { bb = ob; bj = oj; }
+        }
     }
     __syncwarp();   // every lane has read the old label before lane 0 rewrites it
     if (bj != old && label_ok(bj, k, st) && old_label_ok(old, k, st)) {
@@ -530,6 +589,7 @@ static __device__ __forceinline__ void recheck_point(const float* __restrict__ X
             labels[i] = bj;
         }
     }
+    return single;
 }
 
 // One warp per listed point (recheck_point); warps w0, w0 + wstride, ... of

@@ -56,3 +56,19 @@ def test_value_ranges(case):
         X[:] = np.float32(0.1)
     C = X[rng.choice(X.shape[0], size=11, replace=False)].astype(np.float64)
     _check(X, C)
+
+
+@pytest.mark.parametrize("d", [16, 17, 32, 33, 64, 128, 300])
+@pytest.mark.parametrize("k", [2, 40, 130])
+def test_recheck_forms(d, k):
+    """Near ties of every kind: one, two and many candidates, exact ties and
+    pairs that only the oracle's order of addition can rank."""
+    rng = np.random.default_rng(d + k)
+    C = rng.normal(size=(k, d))
+    C[1] = C[0] + 1e-9 * rng.normal(size=d)
+    if k > 2:
+        C[2] = C[0]                                   # equal: lowest index
+        C[3:20] = C[3] + 1e-7 * rng.normal(size=(17, d))
+    X = np.concatenate([C[rng.integers(0, k, 600)], 0.5 * (C[0] + C[rng.integers(0, k, 600)])])
+    X = (X + 1e-3 * rng.normal(size=X.shape) * (rng.random((X.shape[0], 1)) < 0.5)).astype(np.float32)
+    _check(X, np.ascontiguousarray(C))
