@@ -98,7 +98,7 @@ extern "C" {
                                          stage runs FP16 if the fast stage left at most
                                          5 % per iteration, else BF16 (the other entry
                                          points take BF16 there); FP32 otherwise, with a
-                                         tensor-core screen for 8 <= d <= 16: split-FP16
+                                         tensor-core screen for 8 <= d <= 128: split-FP16
                                          products decide the rows outside their error
                                          bound, the FP32 chain the others (same labels,
                                          centers and J; reported as FP32) */

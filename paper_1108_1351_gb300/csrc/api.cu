@@ -241,6 +241,20 @@ int prepare_stage_points(const float* X, long long n, int d, Workspace& w, Devic
     return launch_convert_x_bf16(X, n, d, w.xt, w.xn2, w.st, single, s, ws.sm_count);
 }
 
+// Whether this pass goes through the tensor-core screen.
+static bool screened(const float* X, int d, const Workspace& w)
+{
+    return w.form == KMEANS2_PRECISION_FP32 && w.screen && assign_mma_supported(d, w.c.k, X);
+}
+
+int launch_stage_recheck(const float* X, int d, Workspace& w, int* labels, cudaStream_t s,
+                         int sm_count)
+{
+    // from d = 17 on the screen lists the rows it leaves open without an FP32 pass
+    const int settles = d > 16 && screened(X, d, w);
+    return launch_recheck(X, d, w.c, labels, w.list, w.st, w.acc, settles, s, sm_count);
+}
+
 // The fused distance kernel of the chosen form.
 int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels, cudaStream_t s,
                   int sm_count)
@@ -255,7 +269,7 @@ int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels,
     if (tc16_form(w.form))
         return launch_assign_bf16(X, w.xt, w.xn2, w.cb, n, d, w.c, labels, w.st, w.acc, w.list,
                                   0, s, sm_count);
-    if (w.screen && assign_mma_supported(d, w.c.k, X))
+    if (screened(X, d, w))
         return launch_assign_mma(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
     return launch_assign_fp32(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
 }
@@ -311,7 +325,7 @@ int launch_iteration(const float* X, long long n, int d, Workspace& w, int* labe
                      unsigned long long handle, int use_cond, cudaStream_t s, int sm_count)
 {
     KM2_TRY(launch_assign(X, n, d, w, labels, s, sm_count));
-    KM2_TRY(launch_recheck(X, d, w.c, labels, w.list, w.st, w.acc, s, sm_count));
+    KM2_TRY(launch_stage_recheck(X, d, w, labels, s, sm_count));
     KM2_TRY(launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, handle, use_cond,
                             s));
     return KMEANS2_OK;
@@ -388,7 +402,7 @@ int run_loop_host(const float* X, long long n, int d, Workspace& w, int* labels,
             rc = launch_assign(X, n, d, w, labels, s, sm_count);
             cudaEventRecord(ev1, s);
             if (rc == KMEANS2_OK)
-                rc = launch_recheck(X, d, w.c, labels, w.list, w.st, w.acc, s, sm_count);
+                rc = launch_stage_recheck(X, d, w, labels, s, sm_count);
             if (rc == KMEANS2_OK)
                 rc = launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, 0ull, 0, s);
         } else {
@@ -1150,7 +1164,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
             int* lab = labels + c * chunk;
             if (it == 0) KM2_TRY(launch_qsum(Xc, rows, d, w.st, s, ws.sm_count));
             KM2_TRY(launch_assign(Xc, rows, d, w, lab, s, ws.sm_count));
-            KM2_TRY(launch_recheck(Xc, d, w.c, lab, w.list, w.st, w.acc, s, ws.sm_count));
+            KM2_TRY(launch_stage_recheck(Xc, d, w, lab, s, ws.sm_count));
             return launch_recheck_reset(w.st, s);
         }));
         KM2_TRY(launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, 0ull, 0, s));

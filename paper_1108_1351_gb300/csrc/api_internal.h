@@ -108,7 +108,7 @@ int launch_stage_begin(const Centers& c, const Accum& acc, StageState* st, doubl
 int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const TrajDev& tr,
                     double* clus, unsigned long long cond_handle, int use_cond, cudaStream_t s);
 int launch_recheck(const float* X, int d, const Centers& c, int* labels, const int* list,
-                   StageState* st, const Accum& acc, cudaStream_t s, int sm_count);
+                   StageState* st, const Accum& acc, int settles, cudaStream_t s, int sm_count);
 // Folds this pass's recheck count into the stage total and empties the list
 // (between the chunks of a streamed pass, whose indices are chunk-relative).
 int launch_recheck_reset(StageState* st, cudaStream_t s);
@@ -197,6 +197,9 @@ int prepare_stage_points(const float* X, long long n, int d, Workspace& w, Devic
 // The fused distance kernel of w.form over n points.
 int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels, cudaStream_t s,
                   int sm_count);
+// The FP64 recheck of the rows that launch_assign listed.
+int launch_stage_recheck(const float* X, int d, Workspace& w, int* labels, cudaStream_t s,
+                         int sm_count);
 // Resolves a requested precision to the form this shape runs in.
 int choose_form(int requested, int d, int k, const float* X, int* form);
 int map_stage_error(int err);

@@ -5,22 +5,27 @@
 // warp, and what that leaves open by the FP64 recheck (mma_dev.cuh).  Labels,
 // sums and J equal those of the CUDA-core kernels (assign_fp32.cu) bit for bit.
 //
-// assign_mma_ring (8 <= d <= 16): a warp takes 64 rows at a time from its own ring
-// of cp.async stages in shared memory (rows as they lie in X, and the old labels);
-// the centers' fragments stay in shared memory for the whole launch.  Warps never
-// wait for one another except to flush the partial sums.
+// assign_mma_ring (8 <= d <= 128): a warp takes 32 or 64 rows at a time from its own
+// ring of cp.async stages in shared memory (rows as they lie in X, and the old
+// labels); the centers' fragments stay in shared memory for the whole launch.
+// Warps never wait for one another except to flush the partial sums.  Shapes
+// whose centers do not fit beside the rings go to the CUDA-core kernels.
 //
-// What bounds it: instruction issue and register ports, not memory (at d = 8, k
-// = 32 it reads 3.1 TB/s).  Per converged pass against the CUDA-core kernel
-// (GB300; microseconds):
-//   n 2e7 d 8 k 32   325 -> 233      n 4e6 d 16 k 100   378 -> 197
-//   n 1e7 d 12 k 16  216 -> 141      n 1e6 d 16 k 1000  783 -> 360
-//   n 4e6 d 8 k 256  428 -> 272
-// Tried and dropped: 32 rows at a time (d 8, k 32: 250); work handed out to warps
+// What bounds it: instruction issue and register ports for d <= 16 (at d = 8, k =
+// 32 it reads 3.1 TB/s), the legacy tensor rate (an MMA of 16 x 8 x 16 takes 8
+// cycles per SM sub-partition) for wider rows, DRAM for few centers (d = 128, k =
+// 32: 4.4 TB/s).  Per converged pass against the CUDA-core kernels (GB300; us):
+//   n 2e7 d 8 k 32   325 -> 233      n 2e6 d 32 k 200   969 -> 237
+//   n 1e7 d 12 k 16  216 -> 140      n 1e6 d 37 k 100   343 -> 115
+//   n 4e6 d 8 k 256  428 -> 272      n 1e6 d 64 k 200   842 -> 210
+//   n 4e6 d 16 k 100 378 -> 200      n 1e6 d 128 k 32   835 -> 119
+//   n 1e6 d 16 k 1000 783 -> 360     n 5e5 d 128 k 100  423 -> 131
+// Tried and dropped: 32 rows at a time at d = 8 (250); work handed out to warps
 // dynamically (balance better, ~45 more instructions per 32 rows: 275); the
 // candidate test as saturated FFMAs (250); the same screen on tcgen05 with one
-// row per lane (296: 330 instructions per 32 rows against 274, and warpgroup
-// barriers); d < 8 (precision, see mma_dev.cuh).
+// row per lane (d 8 k 32: 296, with warpgroup barriers and 330 instructions per
+// 32 rows against 274; d 32 k 200: 321; d 64 k 200: 511); d < 8 (precision, see
+// mma_dev.cuh).
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -34,12 +39,19 @@ namespace km2 {
 namespace {
 
 constexpr int kSmemCap = 224 * 1024;       // dynamic shared memory of an SM for these kernels
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 
-// Ring stages per warp: about 40-55 KB in flight per SM.
-template <int DP>
-constexpr int kStages = DP <= 8 ? 3 : 2;
+// Kernel shape by padded dimension.  d <= 16: 8 warps, 2 or 3 CTAs per SM, rings of
+// 2 or 3 stages per warp.  Wider rows (WIDE): the A registers grow with d, so one
+// CTA of as many warps as the registers hold; one stage per warp, refilled as soon
+// as its rows are in registers (the MMAs of 32 rows take longer than the copy).
+template <int DP, bool SINGLE>
+struct RingCfg {
+    static constexpr bool WIDE = DP > 16;
+    static constexpr int W = DP <= 16 ? 8 : DP <= 32 ? 16 : DP <= 64 ? 12 : 8;   // warps
+    static constexpr int THREADS = 32 * W;
+    static constexpr int MINB = WIDE ? 1 : SINGLE ? 3 : 2;
+    static constexpr int S = DP <= 8 ? 3 : DP <= 16 ? 2 : 1;                     // stages
+};
 
 __device__ __forceinline__ void cp_async16_zfill(unsigned sdst, const void* gsrc, int bytes)
 {
@@ -63,12 +75,15 @@ __device__ __forceinline__ void cp_async_wait_group()
 
 // UNIT: rows a warp takes at a time (32 where n is too small to give every warp 64).
 template <int DP, int NT, bool SINGLE, bool FULL, int UNIT>
-__global__ void __launch_bounds__(kThreads, SINGLE ? 3 : 2)
+__global__ void __launch_bounds__((RingCfg<DP, SINGLE>::THREADS), (RingCfg<DP, SINGLE>::MINB))
 assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __restrict__ labels,
                 StageState* st, Accum acc, int* __restrict__ list, int ntiles, int use_sacc)
 {
-    constexpr int S = kStages<DP>;
+    using R = RingCfg<DP, SINGLE>;
+    constexpr int S = R::S, kWarps = R::W, kThreads = R::THREADS;
+    constexpr bool WIDE = R::WIDE;
     constexpr int H = UNIT / 32;
+    static_assert(!WIDE || UNIT == 32, "wide rows: one 32-row block per warp and step");
     constexpr int kFlushSteps = kFlushPoints / (kWarps * UNIT);   // steps per int64 partial
     extern __shared__ __align__(16) unsigned char smem[];
     if (st->error) return;
@@ -125,8 +140,9 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
         lsrc += rstep;
         left_issue -= rstep;
     };
+    // WIDE: the first unit now, each next one once the stage's rows are in registers
 #pragma unroll
-    for (int s = 0; s < S - 1; ++s) issue(s * stage_bytes);
+    for (int s = 0; s < (WIDE ? 1 : S - 1); ++s) issue(s * stage_bytes);
 
     mma_load_centers<DP>(c, ntiles, ms, sb, sn);
     if (use_sacc) {
@@ -139,7 +155,7 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
     const unsigned ring_bytes = S * stage_bytes;
     int to_flush = kFlushSteps;
     for (int step = blockIdx.x; step < steps; step += gridDim.x) {
-        issue(so == 0 ? ring_bytes - stage_bytes : so - stage_bytes);
+        if (!WIDE) issue(so == 0 ? ring_bytes - stage_bytes : so - stage_bytes);
         cp_async_wait_group<S - 1>();
         __syncwarp();
         const float* xr = reinterpret_cast<const float*>(ring + so);
@@ -157,11 +173,20 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
             float xmax = 0.0f;
             mma_load_rows<DP, FULL>(xr + 32 * h * d, d, g, t, 0, ms.sx, A[0], xmax);
             mma_load_rows<DP, FULL>(xr + 32 * h * d, d, g, t, 1, ms.sx, A[1], xmax);
-            lab[h] = mma_decide<DP, NT, SINGLE>(A, sb, sn, ntiles, lane, mma_thr(ms, xmax), open[h]);
             old[h] = delta ? lr[32 * h + 8 * t + g] : -1;
+            if (WIDE) {
+                __syncwarp();            // every lane has read the stage
+                issue(0);
+            }
+            lab[h] = mma_decide<DP, NT, SINGLE>(A, sb, sn, ntiles, lane, mma_thr(ms, xmax), open[h]);
             if (32 * h + 8 * t + g >= rows) { open[h] = false; lab[h] = old[h]; }
         }
-        if (__any_sync(0xffffffffu, open[0] || open[1])) {
+        if (WIDE) {
+            // the recheck kernel decides the open rows: its FP32 pass over k d center
+            // values finds them in L1, which shared memory leaves little of here
+            recheck_append(open[0], (int)(row0 + 8 * t + g), list, &st->recheck_count);
+            if (open[0]) lab[0] = old[0];
+        } else if (__any_sync(0xffffffffu, open[0] || open[1])) {
 #pragma unroll
             for (int h = 0; h < H; ++h) {
                 unsigned todo = __ballot_sync(0xffffffffu, open[h]);
@@ -209,23 +234,31 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
                     labels[row0 + 32 * h + 8 * t + g] = lab[h];
                     count(lab[h], old[h]);
                 }
-                // 32 / DP moved rows at a time, DP lanes per row, a coordinate each: at most
-                // 32 / DP lanes meet on one word (a lane per row is slower in full
+                // 32 / LPR moved rows at a time, LPR lanes per row, a coordinate each: at most
+                // 32 / LPR lanes meet on one word (a lane per row is slower in full
                 // passes: 8.2 against 3.8 ms for n = 1e8, d = 8, k = 32, where a few large
                 // clusters take most rows)
-                const int dim = lane % DP;
+                constexpr int LPR = DP < 32 ? DP : 32;
 #pragma unroll 1
                 while (mv) {
                     int o = -1;
 #pragma unroll
-                    for (int q = 0; q < 32 / DP; ++q) {
-                        if (lane / DP == q) o = __ffs(mv) - 1;
+                    for (int q = 0; q < 32 / LPR; ++q) {
+                        if (lane / LPR == q) o = __ffs(mv) - 1;
                         mv &= mv - 1;              // 0 stays 0
                     }
                     const int src = o < 0 ? 0 : o;
                     const int lo = __shfl_sync(0xffffffffu, lab[h], src);
                     const int ol = __shfl_sync(0xffffffffu, old[h], src);
-                    if (o >= 0 && dim < d) add(lo, ol, dim, xr[(32 * h + 8 * (o & 3) + (o >> 2)) * d + dim]);
+                    if (o >= 0) {
+                        const int r = 32 * h + 8 * (o & 3) + (o >> 2);
+                        if (WIDE) {                // the stage holds other rows by now
+                            const float* xg = X + (row0 + r) * d;
+                            for (int dim = lane; dim < d; dim += 32) add(lo, ol, dim, __ldg(xg + dim));
+                        } else if (lane % LPR < d) {
+                            add(lo, ol, lane % LPR, xr[r * d + lane % LPR]);
+                        }
+                    }
                     __syncwarp();
                 }
             }
@@ -257,26 +290,27 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
     cp_async_wait_group<0>();
 }
 
-template <int DP, int UNIT>
-size_t ring_bytes(int d) { return (size_t)kWarps * kStages<DP> * 4 * UNIT * (d + 1); }
+template <int DP, bool SINGLE, int UNIT>
+size_t ring_bytes(int d) { return (size_t)RingCfg<DP, SINGLE>::W * RingCfg<DP, SINGLE>::S * 4 * UNIT * (d + 1); }
 
 template <int DP, int NT, bool SINGLE, bool FULL, int UNIT>
 int launch_ring_u(const float* X, long long n, const Centers& c, int* labels, StageState* st,
                   const Accum& acc, int* list, int ntiles, cudaStream_t s, int sm_count)
 {
-    const size_t base = mma_center_bytes(DP, ntiles) + ring_bytes<DP, UNIT>(c.d);
+    using R = RingCfg<DP, SINGLE>;
+    const size_t base = mma_center_bytes(DP, ntiles) + ring_bytes<DP, SINGLE, UNIT>(c.d);
     const size_t sums = (size_t)c.k * c.d * 8 + (size_t)c.k * 4;
     const int use_sacc = base + sums <= (size_t)kSmemCap;
     const size_t sm = base + (use_sacc ? sums : 0);
     const void* kfn = (const void*)assign_mma_ring<DP, NT, SINGLE, FULL, UNIT>;
     KM2_TRY(set_max_dynamic_smem(kfn, kSmemCap));
     int per_sm = 0;
-    KM2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kThreads, sm));
+    KM2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, R::THREADS, sm));
     if (per_sm < 1) return KMEANS2_ERR_UNSUPPORTED;
-    const long long steps = (n + kWarps * UNIT - 1) / (kWarps * UNIT);
+    const long long steps = (n + R::W * UNIT - 1) / (R::W * UNIT);
     const int grid = (int)std::max(1ll, std::min((long long)sm_count * per_sm, steps));
     ++g_launches;
-    assign_mma_ring<DP, NT, SINGLE, FULL, UNIT><<<grid, kThreads, sm, s>>>(X, n, c, labels, st, acc,
+    assign_mma_ring<DP, NT, SINGLE, FULL, UNIT><<<grid, R::THREADS, sm, s>>>(X, n, c, labels, st, acc,
                                                                            list, ntiles, use_sacc);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
@@ -288,14 +322,15 @@ int launch_ring(const float* X, long long n, const Centers& c, int* labels, Stag
 {
     // 64 rows per warp and step once every warp of two or three CTAs per SM gets
     // some; below, 32 (too few warps otherwise)
-    const bool small = n < (long long)sm_count * (SINGLE ? 3 : 2) * kWarps * 64;
+    const bool small = n < (long long)sm_count * RingCfg<DP, SINGLE>::MINB * RingCfg<DP, SINGLE>::W * 64;
 #define KM2_RING(FULL_, UNIT_) \
     return launch_ring_u<DP, NT, SINGLE, FULL_, UNIT_>(X, n, c, labels, st, acc, list, ntiles, s, sm_count)
-    if (c.d == DP) {
+    if constexpr (DP > 16) KM2_RING(false, 32);
+    if constexpr (DP <= 16) if (c.d == DP) {
         if (small) KM2_RING(true, 32);
         KM2_RING(true, 64);
     }
-    if constexpr (DP > 8) {
+    if constexpr (DP == 16) {
         if (small) KM2_RING(false, 32);
         KM2_RING(false, 64);
     }
@@ -307,26 +342,44 @@ template <int DP>
 int launch_ring_k(const float* X, long long n, const Centers& c, int* labels, StageState* st,
                   const Accum& acc, int* list, cudaStream_t s, int sm_count)
 {
-    if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, s, sm_count);
-    if (c.k <= 32) return launch_ring<DP, 4, true>(X, n, c, labels, st, acc, list, 4, s, sm_count);
-    return launch_ring<DP, 4, false>(X, n, c, labels, st, acc, list, (c.k + 31) / 32 * 4, s, sm_count);
+    if constexpr (DP > 64) {
+        // two accumulators per block (mma_chunk): chunks of 16 centers
+        if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, s, sm_count);
+        return launch_ring<DP, 2, false>(X, n, c, labels, st, acc, list, (c.k + 15) / 16 * 2, s, sm_count);
+    } else {
+        if constexpr (DP <= 16)
+            if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, s, sm_count);
+        if (c.k <= 32) return launch_ring<DP, 4, true>(X, n, c, labels, st, acc, list, 4, s, sm_count);
+        return launch_ring<DP, 4, false>(X, n, c, labels, st, acc, list, (c.k + 31) / 32 * 4, s, sm_count);
+    }
 }
+
+#define KM2_RING_DPS(X) X(8) X(16) X(32) X(48) X(64) X(96) X(128)
 
 }  // namespace
 
 // d from 8 on: see the precision figures in mma_dev.cuh.
 int assign_mma_supported(int d, int k, const float* X)
 {
-    if ((reinterpret_cast<uintptr_t>(X) & 15) != 0 || d < 8 || d > 16) return 0;
-    const size_t ring = d == 8 ? ring_bytes<8, 64>(d) : ring_bytes<16, 64>(d);
-    return mma_center_bytes(mma_dp(d), (k + 31) / 32 * 4) + ring <= (size_t)kSmemCap;
+    if ((reinterpret_cast<uintptr_t>(X) & 15) != 0 || d < 8 || d > 128) return 0;
+    switch (mma_dp(d)) {
+#define KM2_CASE(DD) case DD: return mma_center_bytes(DD, (k + 31) / 32 * 4) + \
+        ring_bytes<DD, false, (DD > 16 ? 32 : 64)>(d) <= (size_t)kSmemCap;
+        KM2_RING_DPS(KM2_CASE)
+#undef KM2_CASE
+        default: return 0;
+    }
 }
 
 int launch_assign_mma(const float* X, long long n, int d, const Centers& c, int* labels,
                       StageState* st, const Accum& acc, int* list, cudaStream_t s, int sm_count)
 {
-    if (d == 8) return launch_ring_k<8>(X, n, c, labels, st, acc, list, s, sm_count);
-    return launch_ring_k<16>(X, n, c, labels, st, acc, list, s, sm_count);
+    switch (mma_dp(d)) {
+#define KM2_CASE(DD) case DD: return launch_ring_k<DD>(X, n, c, labels, st, acc, list, s, sm_count);
+        KM2_RING_DPS(KM2_CASE)
+#undef KM2_CASE
+        default: return KMEANS2_ERR_UNSUPPORTED;
+    }
 }
 
 }  // namespace km2

@@ -17,7 +17,8 @@
 // Keys are no less precise than the FP32 chain's from d = 8 on.  Error against
 // FP64, rms / largest, in 2^-24 (||x||^2 + 2 C^2), isotropic and anisotropic
 // mixtures of 50 components: d = 8 0.26 / 1.9 (chain 0.27 / 2.1), d = 12 0.27 / 1.9
-// (0.33 / 2.9), d = 16 0.25 / 1.7 (0.39 / 3.0); largest error 0.02 of the bound.
+// (0.33 / 2.9), d = 16 0.25 / 1.7 (0.39 / 3.0), d = 32 0.26 / 2.5 (0.56 / 3.5), d = 64 0.37
+// / 4.4 (0.80 / 4.9), d = 128 0.34 / 4.1 (1.19 / 6.1); largest error 0.02 of the bound.
 // Below, two parts are less precise (d = 4 0.35, chain 0.24) and a third part costs
 // what the MMAs save (n = 1e7, d = 4, k = 20: 135 us against 121), so d < 8 stays on
 // the CUDA cores.
@@ -66,7 +67,7 @@ __host__ __device__ inline size_t mma_center_bytes(int dp, int ntiles)
 }
 __host__ __device__ inline int mma_dp(int d)
 {
-    return d <= 8 ? 8 : (d + 15) / 16 * 16;
+    return d <= 8 ? 8 : d <= 16 ? 16 : d <= 32 ? 32 : d <= 48 ? 48 : d <= 64 ? 64 : d <= 96 ? 96 : 128;
 }
 
 // Scales and bound of one pass, derived from the stage state by every CTA.
@@ -251,6 +252,11 @@ __device__ __forceinline__ void mma_chunk(const uint32_t (&A)[2][MmaCfg<DP>::ARE
             }
         }
         if constexpr (KS > 1) {
+            // from six K-steps on the hi products go to two accumulators, added in
+            // FP32: half the truncations at half the magnitude (d = 128: largest key
+            // error 7.7 in one accumulator, 6.4 for the FP32 chain)
+            constexpr bool TWO = KS > 4;
+            float acc2[2][TWO ? NT : 1][4];
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks) {
 #pragma unroll
@@ -259,9 +265,19 @@ __device__ __forceinline__ void mma_chunk(const uint32_t (&A)[2][MmaCfg<DP>::ARE
 #pragma unroll
                     for (int b = 0; b < 2; ++b) {
                         const uint32_t* a = A[b] + 8 * ks;
-                        mma16816(acc[b][q], a[0], a[1], a[2], a[3], h.x, h.y);
+                        if (TWO && ks == 0) mma16816z(acc2[b][q], a[0], a[1], a[2], a[3], h.x, h.y);
+                        else if (TWO && ks < KS / 2) mma16816(acc2[b][q], a[0], a[1], a[2], a[3], h.x, h.y);
+                        else mma16816(acc[b][q], a[0], a[1], a[2], a[3], h.x, h.y);
                     }
                 }
+            }
+            if constexpr (TWO) {
+#pragma unroll
+                for (int b = 0; b < 2; ++b)
+#pragma unroll
+                    for (int q = 0; q < NT; ++q)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[b][q][e] += acc2[b][q][e];
             }
         }
     } else {

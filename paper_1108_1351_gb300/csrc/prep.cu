@@ -253,13 +253,14 @@ constexpr int kRecheckCache = 1024;     // pass-1 values kept per warp (k <= 102
 // Warps of the grid share the listed points (see recheck_warps).
 __global__ void __launch_bounds__(kRecheckThreads) recheck_kernel(const float* __restrict__ X, int d, Centers c,
                                int* __restrict__ labels, const int* __restrict__ list,
-                               StageState* st, Accum acc)
+                               StageState* st, Accum acc, int settles)
 {
     __shared__ float cache[kRecheckThreads / 32][kRecheckCache];
     if (st->error) return;
     long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    recheck_warps(X, d, c, labels, list, st, acc, gw, nw, cache[threadIdx.x >> 5], kRecheckCache);
+    recheck_warps(X, d, c, labels, list, st, acc, gw, nw, cache[threadIdx.x >> 5], kRecheckCache,
+                  settles);
 }
 
 }  // namespace
@@ -353,10 +354,10 @@ int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const Tr
 }
 
 int launch_recheck(const float* X, int d, const Centers& c, int* labels, const int* list,
-                   StageState* st, const Accum& acc, cudaStream_t s, int sm_count)
+                   StageState* st, const Accum& acc, int settles, cudaStream_t s, int sm_count)
 {
     ++g_launches;
-    recheck_kernel<<<sm_count * 4, kRecheckThreads, 0, s>>>(X, d, c, labels, list, st, acc);
+    recheck_kernel<<<sm_count * 4, kRecheckThreads, 0, s>>>(X, d, c, labels, list, st, acc, settles);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }

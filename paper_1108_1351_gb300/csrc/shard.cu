@@ -246,8 +246,8 @@ int run_local_pass(kmeans2_shard* sh, kmeans2_exchange* next)
     if (rows > 0) {
         KM2_TRY(launch_assign(sh->stage_X(), rows, sh->d, sh->w, sh->stage_labels(), s,
                               sh->ws->sm_count));
-        KM2_TRY(launch_recheck(sh->stage_X(), sh->d, sh->w.c, sh->stage_labels(), sh->w.list,
-                               sh->w.st, sh->w.acc, s, sh->ws->sm_count));
+        KM2_TRY(launch_stage_recheck(sh->stage_X(), sh->d, sh->w, sh->stage_labels(), s,
+                                     sh->ws->sm_count));
     }
     const long long count = partials_count(sh->k, sh->d);
     ++g_launches;

@@ -594,14 +594,20 @@ static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X
 
 // One warp per listed point (recheck_point); warps w0, w0 + wstride, ... of
 // the caller each take the listed points.
+// settles: the list comes from a screen that leaves rows to the FP32 pass here;
+// those it decides alone do not count as rechecked in FP64.
 static __device__ void recheck_warps(const float* __restrict__ X, int d, Centers c,
                                      int* __restrict__ labels, const int* __restrict__ list,
                                      StageState* st, Accum acc, long long gw, long long nw,
-                                     float* cache, int cache_cap)
+                                     float* cache, int cache_cap, int settles)
 {
     const int count = st->recheck_count;
+    long long settled = 0;
     for (long long w = gw; w < count; w += nw)
-        recheck_point(X, d, c, labels, list[w], st, acc, cache, cache_cap);
+        settled += recheck_point(X, d, c, labels, list[w], st, acc, cache, cache_cap) ? 1 : 0;
+    if (settles && settled && (threadIdx.x & 31) == 0)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&st->rechecked_total),
+                  (unsigned long long)(-settled));
 }
 
 

@@ -1,11 +1,11 @@
-"""The tensor-core screen of the FP32 form (precision AUTO, 8 <= d <= 16; GPU).
+"""The tensor-core screen of the FP32 form (precision AUTO, 8 <= d <= 128; GPU).
 
 The screen decides a row only outside its bound and leaves the others to the
 FP32 chain and the FP64 recheck, so labels, centers, J and iteration counts
 must equal the oracle's (labels exactly; centers and J within the helpers'
 derived tolerances) and the plain FP32 form's bit for bit.  Sizes lie around
-the edges of its tiles: 32 / 64 rows per warp and 512 per step, 8 centers per
-block, 16 / 32 per chunk, d at, between and outside the padded sizes 8 and 16."""
+the edges of its tiles: 32 / 64 rows per warp and 256 to 512 per step, 8 centers per
+block, 16 / 32 per chunk, d at, between and outside the padded sizes 8 .. 128."""
 import numpy as np
 import pytest
 import torch
@@ -36,9 +36,9 @@ def _check_step(X, C):
     assert a[4] == oem
 
 
-@pytest.mark.parametrize("d", [7, 8, 9, 11, 12, 16, 17])
+@pytest.mark.parametrize("d", [7, 8, 9, 12, 16, 17, 32, 33, 48, 50, 64, 65, 96, 100, 128, 129])
 @pytest.mark.parametrize("n,k", [(1, 1), (31, 7), (64, 8), (65, 9), (511, 16), (513, 17),
-                                 (2000, 32), (2000, 33), (4099, 64), (5000, 257), (3000, 1000), (170_003, 20)])
+                                 (2000, 33), (5000, 257), (3000, 1000), (170_003, 20)])
 def test_step_sizes(n, k, d):
     X = synth.iso_gaussian_mixture(n, d, max(1, k // 2), 100 * d + k).numpy()
     rng = np.random.default_rng(n + k)
@@ -46,14 +46,16 @@ def test_step_sizes(n, k, d):
     _check_step(X, C)
 
 
+@pytest.mark.parametrize("d", [8, 40])
 @pytest.mark.parametrize("scale,shift", [(1e-20, 0.0), (1e-12, 0.0), (1e6, 0.0), (1.0, 1e4)])
-def test_step_ranges(scale, shift):
-    X = (synth.iso_gaussian_mixture(3001, 8, 9, 5).numpy() * scale + shift).astype(np.float32)
+def test_step_ranges(scale, shift, d):
+    X = (synth.iso_gaussian_mixture(3001, d, 9, 5).numpy() * scale + shift).astype(np.float32)
     _check_step(X, X[:20].astype(np.float64))
 
 
-def test_step_centers_outside_the_scaled_range_and_duplicates():
-    X = synth.iso_gaussian_mixture(1500, 8, 5, 6).numpy()
+@pytest.mark.parametrize("d", [8, 16, 24, 100])
+def test_step_centers_outside_the_scaled_range_and_duplicates(d):
+    X = synth.iso_gaussian_mixture(1500, d, 5, 6).numpy()
     C = X[:40].astype(np.float64)
     C[3] *= 1e14                       # far beyond the FP16 scaling: every row goes to the FP32 chain
     _check_step(X, C)
@@ -62,7 +64,8 @@ def test_step_centers_outside_the_scaled_range_and_duplicates():
     _check_step(np.ascontiguousarray(np.repeat(X[:50], 30, axis=0)), X[:33].astype(np.float64))
 
 
-@pytest.mark.parametrize("n,d,k", [(20_011, 9, 4), (60_001, 8, 32), (30_003, 12, 50)])
+@pytest.mark.parametrize("n,d,k", [(20_011, 9, 4), (60_001, 8, 32), (30_003, 12, 50),
+                                   (20_003, 31, 70), (9_001, 100, 20)])
 def test_fits_and_other_entry_points(n, d, k):
     X = synth.aniso_gaussian_noise(n, d, k, d).numpy()
     Xd = torch.as_tensor(X, device=DEV)
