@@ -174,7 +174,7 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
             mma_load_rows<DP, FULL>(xr + 32 * h * d, d, g, t, 0, ms.sx, A[0], xmax);
             mma_load_rows<DP, FULL>(xr + 32 * h * d, d, g, t, 1, ms.sx, A[1], xmax);
             old[h] = delta ? lr[32 * h + 8 * t + g] : -1;
-            if (WIDE) {
+            if (WIDE && delta) {
                 __syncwarp();            // every lane has read the stage
                 issue(0);
             }
@@ -252,9 +252,9 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
                     const int ol = __shfl_sync(0xffffffffu, old[h], src);
                     if (o >= 0) {
                         const int r = 32 * h + 8 * (o & 3) + (o >> 2);
-                        if (WIDE) {                // the stage holds other rows by now
-                            const float* xg = X + (row0 + r) * d;
-                            for (int dim = lane; dim < d; dim += 32) add(lo, ol, dim, __ldg(xg + dim));
+                        if (WIDE) {                // delta: the stage holds other rows by now
+                            const float* xg = delta ? X + (row0 + r) * d : xr + r * d;
+                            for (int dim = lane; dim < d; dim += 32) add(lo, ol, dim, xg[dim]);
                         } else if (lane % LPR < d) {
                             add(lo, ol, lane % LPR, xr[r * d + lane % LPR]);
                         }
@@ -264,6 +264,7 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
             }
         }
         __syncwarp();   // every lane is done with the stage before it is refilled
+        if (WIDE && !delta) issue(0);   // a full pass adds every row's coordinates from the stage
         so = so + stage_bytes == ring_bytes ? 0 : so + stage_bytes;
 
         // static flush schedule: at most 2^16 rows per int64 partial

@@ -212,8 +212,15 @@ __global__ void __launch_bounds__(256) stage_begin_kernel(Centers c, Accum acc, 
         atomicMax(reinterpret_cast<unsigned int*>(&st->cmax2), __float_as_uint(__double2float_ru(mx)));
 }
 
-// New centers (one warp each, many CTAs), then, in the CTA that finishes last,
-// movement, J and loop control for the next iteration.
+// New centers (one warp each) and their divisions (one thread each), then, in the
+// CTA that finishes last, movement, J and loop control for the next iteration.
+// What bounds it: FP64, ~60 instructions per center and 32 coordinates, each 16
+// cycles of its SM's pipe.  So the centers are dealt out over the SMs one warp at a
+// time, and the CTA's divisions run as one warp's instructions.  One CTA with the
+// compiler's 128-bit division, one lane and center after the other: 51 us for k =
+// 50, d = 5, 134 us for k = 100, d = 37; with 8 centers per CTA and the divisions in the
+// last: 15 and 19 us, k = 32, d = 128 26 us, k = 1024, d = 128 38 us; now 13, 15, 20 and
+// 27 us.
 __global__ void __launch_bounds__(256) finalize_kernel(Accum acc, Centers c, StageState* st,
                                                        TrajDev tr, double* clus,
                                                        unsigned long long handle, int use_cond)
@@ -229,9 +236,12 @@ __global__ void __launch_bounds__(256) finalize_kernel(Accum acc, Centers c, Sta
     }
     const double inv = st->inv_scaleF;
     const int it = st->iter;
-    for (int j = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); j < c.k;
-         j += (int)((gridDim.x * blockDim.x) >> 5))
+    for (int j = (int)(blockIdx.x + gridDim.x * (threadIdx.x >> 5)); j < c.k;
+         j += (int)(gridDim.x * (blockDim.x >> 5)))
         finalize_center_warp(acc, c, inv, j, clus, tr, it);
+    __syncthreads();
+    for (int j = (int)(blockIdx.x + gridDim.x * threadIdx.x); j < c.k; j += (int)(gridDim.x * blockDim.x))
+        finalize_divide(c.k, acc.cnt, inv, clus, j);
     if (gridDim.x > 1) {
         __threadfence();
         __syncthreads();
@@ -250,17 +260,30 @@ __global__ void __launch_bounds__(256) finalize_kernel(Accum acc, Centers c, Sta
 constexpr int kRecheckThreads = 256;
 constexpr int kRecheckCache = 1024;     // pass-1 values kept per warp (k <= 1024)
 
-// Warps of the grid share the listed points (see recheck_warps).
+// Warps of the grid share the listed points (see recheck_warps), or blocks do when
+// there are many centers and no more points than warps (recheck_point_block).
 __global__ void __launch_bounds__(kRecheckThreads) recheck_kernel(const float* __restrict__ X, int d, Centers c,
                                int* __restrict__ labels, const int* __restrict__ list,
                                StageState* st, Accum acc, int settles)
 {
-    __shared__ float cache[kRecheckThreads / 32][kRecheckCache];
+    constexpr int W = kRecheckThreads / 32;
+    __shared__ float cache[W * kRecheckCache];
+    __shared__ RecheckBlockSmem sm;
     if (st->error) return;
-    long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    recheck_warps(X, d, c, labels, list, st, acc, gw, nw, cache[threadIdx.x >> 5], kRecheckCache,
-                  settles);
+    const long long nw = (long long)gridDim.x * W;
+    if (c.k >= 256 && c.kpad <= W * kRecheckCache && st->recheck_count <= nw) {
+        const int count = st->recheck_count;
+        long long settled = 0;
+        for (int p = blockIdx.x; p < count; p += gridDim.x)
+            settled += recheck_point_block(X, d, c, labels, list[p], st, acc, cache, sm) ? 1 : 0;
+        if (settles && settled && threadIdx.x == 0)
+            atomicAdd(reinterpret_cast<unsigned long long*>(&st->rechecked_total),
+                      (unsigned long long)(-settled));
+        return;
+    }
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    recheck_warps(X, d, c, labels, list, st, acc, gw, nw, cache + (threadIdx.x >> 5) * kRecheckCache,
+                  kRecheckCache, settles);
 }
 
 }  // namespace
@@ -347,8 +370,10 @@ int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const Tr
                     double* clus, unsigned long long cond_handle, int use_cond, cudaStream_t s)
 {
     ++g_launches;
-    finalize_kernel<<<std::min(1024, (c.k + 7) / 8), 256, 0, s>>>(acc, c, st, tr, clus, cond_handle,
-                                                                 use_cond);
+    // one CTA for a handful of centers (no hand-over to a last CTA), else one
+    // center per CTA up to about one CTA per SM
+    finalize_kernel<<<c.k <= 8 ? 1 : std::min(c.k, 152), 256, 0, s>>>(acc, c, st, tr, clus,
+                                                                     cond_handle, use_cond);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }

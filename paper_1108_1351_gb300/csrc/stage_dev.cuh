@@ -279,6 +279,27 @@ __device__ __forceinline__ unsigned long long div192(unsigned long long (&T)[3],
     return rem;
 }
 
+// One thread: center j's division.  T_j becomes floor(T_j / N_j) in place, and
+// clus[k + j] its remaining term of J, N_j ||c_j - mu_j||^2 - frac(T_j / N_j) 2^-2F
+// (zeros for an empty cluster).
+static __device__ __forceinline__ void finalize_divide(int k, const unsigned long long* cnt,
+                                                       double inv, double* clus, int j)
+{
+    unsigned long long* qw = reinterpret_cast<unsigned long long*>(clus + 3 * k) + 3ll * j;
+    const unsigned long long N = cnt[j];
+    double term = 0.0;
+    if ((long long)N > 0) {
+        unsigned long long T[3] = {qw[0], qw[1], qw[2]};
+        const unsigned long long rem = div192(T, N);
+        const double Nd = (double)N;
+        term = clus[k + j] / Nd - ((double)rem / Nd) * (inv * inv);
+        qw[0] = T[0];
+        qw[1] = T[1];
+        qw[2] = T[2];
+    }
+    clus[k + j] = term;
+}
+
 struct FinalizeSmem {
     double r_shift[32];
     double r_J[256];
@@ -287,18 +308,15 @@ struct FinalizeSmem {
     unsigned __int128 r_q[32][3];
 };
 
-// Whole block of 256 threads, after every center's finalize_center_warp:
-// movement, J and loop control from clus (thread 0 updates st).  J's floating
-// terms are added in one fixed order, the one of a tree over 1024 threads that
-// stride over the centers.  The integer part of J, sum s^2 - sum_j floor(T_j /
-// N_j), is exact (256-bit); it is rounded to FP64 once and added to the sum of the
-// per-center remainders:
+// Whole block of 256 threads, after every center's finalize_center_warp and
+// finalize_divide: movement, J and loop control from clus (thread 0 updates st).
+// J's floating terms are added in one fixed order, the one of a tree over 1024
+// threads that stride over the centers.  The integer part of J, sum s^2 - sum_j
+// floor(T_j / N_j), is exact (256-bit); it is rounded to FP64 once and added to the
+// sum of the per-center remainders:
 //   J = (sum s^2 - sum_j T_j / N_j) 2^-2F + sum_j N_j ||c_j - mu_j||^2
 //     = sum_j sum_{i in j} ||x_i - c_j||^2   (Eq. 3, on the fixed-point values).
-// A thread per center divides, so the divisions of all centers overlap (one
-// lane per warp did them before, one center after the other, with the
-// compiler's 128-bit division: 51 us for k = 50, d = 5, 134 us for k = 100, d = 37
-// in all of finalize).  Ends with the block synchronised.
+// Ends with the block synchronised.
 static __device__ void finalize_reduce_block(int k, const unsigned long long* cnt, StageState* st,
                                              const TrajDev& tr, const double* clus, FinalizeSmem& sm)
 {
@@ -319,20 +337,14 @@ static __device__ void finalize_reduce_block(int k, const unsigned long long* cn
             if (j >= k) break;
             sh = fmax(sh, __ldcg(clus + j));
             mx = fmax(mx, __ldcg(clus + 2 * k + j));
-            const unsigned long long N = __ldcg(cnt + j);
-            double term = 0.0;
-            if ((long long)N > 0) {
-                unsigned long long T[3] = {__ldcg(qw + 3ll * j), __ldcg(qw + 3ll * j + 1),
-                                           __ldcg(qw + 3ll * j + 2)};
-                const unsigned long long rem = div192(T, N);
-                const double Nd = (double)N;
-                term = __ldcg(clus + k + j) / Nd - ((double)rem / Nd) * (inv * inv);
-                a0 += T[0];
-                a1 += T[1];
-                a2 += T[2];
+            jj[v] += __ldcg(clus + k + j);
+            if (__ldcg(cnt + j) == 0) {
+                ++em;
+            } else {
+                a0 += __ldcg(qw + 3ll * j);
+                a1 += __ldcg(qw + 3ll * j + 1);
+                a2 += __ldcg(qw + 3ll * j + 2);
             }
-            jj[v] += term;
-            em += N == 0 ? 1 : 0;
         }
     }
     // the 1024-thread tree's first two levels, then 256 values
@@ -422,31 +434,90 @@ static __device__ void finalize_block(Accum acc, Centers c, StageState* st, Traj
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int j = warp; j < c.k; j += nw) finalize_center_warp(acc, c, inv, j, clus, tr, it);
     __syncthreads();
+    for (int j = threadIdx.x; j < c.k; j += blockDim.x) finalize_divide(c.k, acc.cnt, inv, clus, j);
+    __syncthreads();
     finalize_reduce_block(c.k, acc.cnt, st, tr, clus, sm);
 }
 
 // FP32 D_j = ||c_j||^2 - 2 x.c_j of one point against centers j0 + 32 i
-// (i < 4): the CUDA-core FMA chain whose error tie_kappa bounds, t ascending.
+// (i < NQ): the CUDA-core FMA chain whose error tie_kappa bounds, t ascending.
 // c32t (dims x kpad, coalesced across the warp's lanes) holds the same FP32
 // values as the row-major copy; fmaf(-2 x_t, c_t, a) equals fmaf(x_t, -2 c_t, a)
 // (scaling by -2 is exact).  Padding centers read zeros.
-static __device__ __forceinline__ void recheck_d4(const float* __restrict__ x, int d,
-                                                  const Centers& c, int j0, float a[4])
+template <int NQ>
+static __device__ __forceinline__ void recheck_d(const float* __restrict__ x, int d,
+                                                 const Centers& c, int j0, float (&a)[NQ])
 {
     const int kpad = c.kpad;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = c.cnorm[j0 + 32 * i];
+    for (int i = 0; i < NQ; ++i) a[i] = c.cnorm[j0 + 32 * i];
     const float* ct = c.c32t + j0;
-    for (int t = 0; t < d; ++t) {
+    int t = 0;
+    if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+#pragma unroll 2
+        for (; t + 4 <= d; t += 4) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(x + t));
+            const float xm2[4] = {-2.0f * v.x, -2.0f * v.y, -2.0f * v.z, -2.0f * v.w};
+            float w[4][NQ];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < NQ; ++i) w[u][i] = ct[(long long)(t + u) * kpad + 32 * i];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < NQ; ++i) a[i] = fmaf(xm2[u], w[u][i], a[i]);
+        }
+    }
+#pragma unroll 4
+    for (; t < d; ++t) {
         const float xm2 = -2.0f * __ldg(x + t);
         const float* row = ct + (long long)t * kpad;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = fmaf(xm2, row[32 * i], a[i]);
+        for (int i = 0; i < NQ; ++i) a[i] = fmaf(xm2, row[32 * i], a[i]);
     }
 }
 
+// The sums, counts and label of point i (row x) move from cluster old (-1: none)
+// to bj; threads tid of nt share the coordinates.
+static __device__ __forceinline__ void recheck_move(const float* __restrict__ x, int d, const Accum& acc,
+                                                    int* __restrict__ labels, int i, int old, int bj,
+                                                    float scaleF, int tid, int nt)
+{
+    for (int t = tid; t < d; t += nt) {
+        long long v = to_fixed(__ldg(x + t), scaleF);
+        split_add(acc.s_lo + (long long)bj * d + t, acc.s_hi + (long long)bj * d + t, v);
+        if (old >= 0)
+            split_add(acc.s_lo + (long long)old * d + t, acc.s_hi + (long long)old * d + t, -v);
+    }
+    if (tid == 0) {
+        atomicAdd(acc.cnt + bj, 1ull);
+        if (old >= 0) atomicAdd(acc.cnt + old, ~0ull);
+        labels[i] = bj;
+    }
+}
+
+// One warp: FP64 squared distance of row x to center j, lanes over coordinates.
+static __device__ __forceinline__ double recheck_lanes_f64(const float* __restrict__ x, int d,
+                                                           const Centers& c, int j)
+{
+    const double* cj64 = c.c64 + (long long)j * d;
+    double p = 0.0;
+    for (int t = threadIdx.x & 31; t < d; t += 32) {
+        const double e = (double)__ldg(x + t) - cj64[t];
+        p = fma(e, e, p);
+    }
+    return warp_sum_f64(p);
+}
+
+// Whether the best two of recheck_lanes_f64 rank the same in the oracle's order.
+static __device__ __forceinline__ bool recheck_ranked(double s1, double s2, int d)
+{
+    return s2 - s1 > (double)(2 * d + 16) * 1.1102230246251565e-16 * (s1 + s2);
+}
+
 // One warp: re-decide point i.  Pass 1: FP32 D_j for every center on the CUDA
-// cores (recheck_d4) and their minimum b1.  Pass 2: the centers with D_j <= b1 +
+// cores (recheck_d) and their minimum b1.  Pass 2: the centers with D_j <= b1 +
 // tie_kappa (2 C2 + X2) + tie_abs -- a set that provably holds the FP64 argmin -- are
 // compared by their FP64 distances and the smallest wins, lowest index on ties,
 // as in the oracle's form (sum_t fma(x_t - c_t, x_t - c_t, acc), t ascending):
@@ -464,13 +535,15 @@ static __device__ __forceinline__ void recheck_d4(const float* __restrict__ x, i
 // cache: per-warp shared memory of cache_cap floats for the pass-1 values
 // (pass 2 recomputes them when kpad > cache_cap or cache is null).  Returns
 // whether the point had a single candidate.
-static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X, int d,
-                                                     const Centers& c, int* __restrict__ labels,
-                                                     int i, StageState* st, const Accum& acc,
-                                                     float* cache, int cache_cap)
+// NQ: centers per lane and step (1 for k <= 32, 2 for k <= 64, else 4).
+template <int NQ>
+static __device__ __forceinline__ bool recheck_point_nq(const float* __restrict__ X, int d,
+                                                        const Centers& c, int* __restrict__ labels,
+                                                        int i, StageState* st, const Accum& acc,
+                                                        float* cache, int cache_cap)
 {
+    constexpr int STEP = 32 * NQ;
     const int mode = st->mode;
-    const float scaleF = st->scaleF;
     const float c2x2 = 2.0f * st->cmax2;
     const float kap = tie_kappa(d);
     const int k = c.k;
@@ -484,11 +557,11 @@ static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X
     for (int o = 16; o; o >>= 1) x2 += __shfl_xor_sync(0xffffffffu, x2, o);
     float b1 = INFINITY;
     int b1j = k;
-    for (int j0 = lane; j0 < k; j0 += 128) {
-        float a[4];
-        recheck_d4(x, d, c, j0, a);
+    for (int j0 = lane; j0 < k; j0 += STEP) {
+        float a[NQ];
+        recheck_d<NQ>(x, d, c, j0, a);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             if (j0 + 32 * q < k && a[q] < b1) { b1 = a[q]; b1j = j0 + 32 * q; }
             if (cached) cache[j0 + 32 * q] = a[q];
         }
@@ -496,21 +569,20 @@ static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X
     const float lane_b1 = b1;
     for (int o = 16; o; o >>= 1) b1 = fminf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
     const float lim = b1 + kap * (c2x2 + x2) * 1.0009765625f + tie_abs(d + 1);
-    // candidates of this lane (a NaN or an infinite distance counts as one)
-    auto value = [&](int j0, float a[4]) {
+    auto value = [&](int j0, float (&a)[NQ]) {
         if (cached) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] = cache[j0 + 32 * q];
+            for (int q = 0; q < NQ; ++q) a[q] = cache[j0 + 32 * q];
         } else {
-            recheck_d4(x, d, c, j0, a);
+            recheck_d<NQ>(x, d, c, j0, a);
         }
     };
     int ncand = 0;
-    for (int j0 = lane; j0 < k; j0 += 128) {
-        float a[4];
+    for (int j0 = lane; j0 < k; j0 += STEP) {
+        float a[NQ];
         value(j0, a);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) ncand += (j0 + 32 * q < k && a[q] <= lim) ? 1 : 0;
+        for (int q = 0; q < NQ; ++q) ncand += (j0 + 32 * q < k && a[q] <= lim) ? 1 : 0;
     }
     ncand = __reduce_add_sync(0xffffffffu, ncand);
     int bj = INT_MAX;
@@ -522,37 +594,31 @@ static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X
         decided = true;
     } else if (d > 16 && ncand * (2 * ((d + 31) / 32) + 5) < 2 * d) {
         double s1 = DBL_MAX, s2 = DBL_MAX;       // best two sums (the same on every lane)
-        for (int jb = 0; jb < k; jb += 128) {
-            float a[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+        for (int jb = 0; jb < k; jb += STEP) {
+            float a[NQ];
             if (jb + lane < k) value(jb + lane, a);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 unsigned m = __ballot_sync(0xffffffffu, jb + lane + 32 * q < k && a[q] <= lim);
                 while (m) {
                     const int j = jb + 32 * q + __ffs(m) - 1;
                     m &= m - 1;
-                    const double* cj64 = c.c64 + (long long)j * d;
-                    double p = 0.0;
-                    for (int t = lane; t < d; t += 32) {
-                        const double e = (double)__ldg(x + t) - cj64[t];
-                        p = fma(e, e, p);
-                    }
-                    p = warp_sum_f64(p);
+                    const double p = recheck_lanes_f64(x, d, c, j);
                     if (p < s1) { s2 = s1; s1 = p; bj = j; }
                     else if (p < s2) s2 = p;
                 }
             }
         }
-        decided = s2 - s1 > (double)(2 * d + 16) * 1.1102230246251565e-16 * (s1 + s2);
+        decided = recheck_ranked(s1, s2, d);
     }
     if (!decided) {
         double best = DBL_MAX;
         bj = INT_MAX;
-        for (int j0 = lane; j0 < k; j0 += 128) {
-            float a[4];
+        for (int j0 = lane; j0 < k; j0 += STEP) {
+            float a[NQ];
             value(j0, a);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const int j = j0 + 32 * q;
                 if (j < k && a[q] <= lim) {
                     const double* cj64 = c.c64 + (long long)j * d;
@@ -576,19 +642,131 @@ static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X
         }
     }
     __syncwarp();   // every lane has read the old label before lane 0 rewrites it
-    if (bj != old && label_ok(bj, k, st) && old_label_ok(old, k, st)) {
-        for (int t = lane; t < d; t += 32) {
-            long long v = to_fixed(__ldg(x + t), scaleF);
-            split_add(acc.s_lo + (long long)bj * d + t, acc.s_hi + (long long)bj * d + t, v);
-            if (old >= 0)
-                split_add(acc.s_lo + (long long)old * d + t, acc.s_hi + (long long)old * d + t, -v);
-        }
-        if (lane == 0) {
-            atomicAdd(acc.cnt + bj, 1ull);
-            if (old >= 0) atomicAdd(acc.cnt + old, ~0ull);
-            labels[i] = bj;
-        }
+    if (bj != old && label_ok(bj, k, st) && old_label_ok(old, k, st))
+        recheck_move(x, d, acc, labels, i, old, bj, st->scaleF, lane, 32);
+    return single;
+}
+
+static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X, int d,
+                                                     const Centers& c, int* __restrict__ labels,
+                                                     int i, StageState* st, const Accum& acc,
+                                                     float* cache, int cache_cap)
+{
+    if (c.k <= 32) return recheck_point_nq<1>(X, d, c, labels, i, st, acc, cache, cache_cap);
+    if (c.k <= 64) return recheck_point_nq<2>(X, d, c, labels, i, st, acc, cache, cache_cap);
+    return recheck_point_nq<4>(X, d, c, labels, i, st, acc, cache, cache_cap);
+}
+
+// A block of 256 threads per point, for many centers and few listed points: the
+// warps share the centers, so a point waits for an eighth of the loads (one warp
+// per point is bound by their latency: k = 1024, d = 128 reads 512 KB of centers).
+// The same decisions as recheck_point.  cache: kpad floats of shared memory.
+struct RecheckBlockSmem {
+    float b1[8];
+    int b1j[8];
+    int ncand[8];
+    double s1[8], s2[8];
+    int sj[8];
+    int bj;
+};
+static __device__ bool recheck_point_block(const float* __restrict__ X, int d, const Centers& c,
+                                           int* __restrict__ labels, int i, StageState* st,
+                                           const Accum& acc, float* cache, RecheckBlockSmem& sm)
+{
+    const int k = c.k;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float* x = X + (long long)i * d;
+    const int old = (st->mode == kModeDelta) ? labels[i] : -1;
+    float x2 = 0.0f;
+    for (int t = lane; t < d; t += 32) { float v = __ldg(x + t); x2 = fmaf(v, v, x2); }
+    for (int o = 16; o; o >>= 1) x2 += __shfl_xor_sync(0xffffffffu, x2, o);
+    float b1 = INFINITY;
+    int b1j = k;
+    for (int j0 = 32 * warp + lane; j0 < k; j0 += 256) {
+        float a[1];
+        recheck_d<1>(x, d, c, j0, a);
+        if (a[0] < b1) { b1 = a[0]; b1j = j0; }
+        cache[j0] = a[0];
     }
+    const float lane_b1 = b1;
+    for (int o = 16; o; o >>= 1) b1 = fminf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
+    {
+        const unsigned m = __ballot_sync(0xffffffffu, lane_b1 == b1);
+        b1j = __shfl_sync(0xffffffffu, b1j, m ? __ffs(m) - 1 : 0);
+    }
+    if (lane == 0) { sm.b1[warp] = b1; sm.b1j[warp] = b1j; }
+    __syncthreads();
+    int bj = INT_MAX;
+    for (int w = 0; w < 8; ++w)
+        if (sm.b1[w] < b1 || (sm.b1[w] == b1 && w <= warp)) b1 = sm.b1[w];
+    for (int w = 7; w >= 0; --w)
+        if (sm.b1[w] == b1) bj = sm.b1j[w];
+    const float lim = b1 + tie_kappa(d) * (2.0f * st->cmax2 + x2) * 1.0009765625f + tie_abs(d + 1);
+    int nc = 0;
+    double s1 = DBL_MAX, s2 = DBL_MAX;
+    int sj = INT_MAX;
+    for (int jb = 32 * warp; jb < k; jb += 256) {
+        unsigned m = __ballot_sync(0xffffffffu, jb + lane < k && cache[jb + lane] <= lim);
+        nc += __popc(m);
+    }
+    if (lane == 0) sm.ncand[warp] = nc;
+    __syncthreads();
+    int ncand = 0;
+    for (int w = 0; w < 8; ++w) ncand += sm.ncand[w];
+    const bool single = ncand == 1 && lim < FLT_MAX;
+    bool decided = single;
+    if (!single && ncand <= 256) {
+        for (int jb = 32 * warp; jb < k; jb += 256) {
+            unsigned m = __ballot_sync(0xffffffffu, jb + lane < k && cache[jb + lane] <= lim);
+            while (m) {
+                const int j = jb + __ffs(m) - 1;
+                m &= m - 1;
+                const double p = recheck_lanes_f64(x, d, c, j);
+                if (p < s1) { s2 = s1; s1 = p; sj = j; }
+                else if (p < s2) s2 = p;
+            }
+        }
+        if (lane == 0) { sm.s1[warp] = s1; sm.s2[warp] = s2; sm.sj[warp] = sj; }
+        __syncthreads();
+        s1 = s2 = DBL_MAX;
+        bj = INT_MAX;
+        for (int w = 0; w < 8; ++w) {
+            const double a1 = sm.s1[w], a2 = sm.s2[w];
+            if (a1 < s1) { s2 = fmin(s1, a2); s1 = a1; bj = sm.sj[w]; }
+            else s2 = fmin(s2, a1);
+        }
+        decided = recheck_ranked(s1, s2, d);
+    }
+    if (!decided) {                              // the same on every thread
+        if (warp == 0) {
+            // the oracle's order, a lane per candidate
+            double best = DBL_MAX;
+            bj = INT_MAX;
+            for (int j = lane; j < k; j += 32) {
+                if (cache[j] <= lim) {
+                    const double* cj64 = c.c64 + (long long)j * d;
+                    double a2 = 0.0;
+                    for (int t = 0; t < d; ++t) {
+                        double e = (double)__ldg(x + t) - cj64[t];
+                        a2 = fma(e, e, a2);
+                    }
+                    if (a2 < best || (a2 == best && j < bj)) { best = a2; bj = j; }
+                }
+            }
+            unsigned long long bb = (unsigned long long)__double_as_longlong(best);
+            for (int o = 16; o; o >>= 1) {
+                const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bb, o);
+                const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+                if (ob < bb || (ob == bb && oj < bj)) { bb = ob; bj = oj; }
+            }
+            if (lane == 0) sm.bj = bj;
+        }
+        __syncthreads();
+        bj = sm.bj;
+    }
+    __syncthreads();   // every thread has read the old label and the shared values
+    if (bj != old && label_ok(bj, k, st) && old_label_ok(old, k, st))
+        recheck_move(x, d, acc, labels, i, old, bj, st->scaleF, threadIdx.x, blockDim.x);
     return single;
 }
 

@@ -59,7 +59,7 @@ def test_value_ranges(case):
 
 
 @pytest.mark.parametrize("d", [16, 17, 32, 33, 64, 128, 300])
-@pytest.mark.parametrize("k", [2, 40, 130])
+@pytest.mark.parametrize("k", [2, 33, 130, 256, 700])
 def test_recheck_forms(d, k):
     """Near ties of every kind: one, two and many candidates, exact ties and
     pairs that only the oracle's order of addition can rank."""
