@@ -842,7 +842,7 @@ def fit_batched(Xs, ks, subset_fraction, seeds, tol, max_iter, *, tol_fast: floa
     res = (Result * cnt)()
     opt = Options()
     lib.kmeans2_default_options(ctypes.byref(opt))
-    opt.precision = PRECISION["fp32"]
+    opt.precision = PRECISION["auto"]
     opt.tol_fast = tol_fast
     opt.stream = _stream_of(Xs[0], stream)
     opt.profile = ctypes.addressof(profile) if profile is not None else None

@@ -3,7 +3,7 @@
 // and convergence flag in a device descriptor; one iteration of the whole
 // batch is
 //   batch_assign<DC>  one launch per dimension class over a list of work items
-//                     (job, first 1024-point tile, tile count); items of jobs
+//   or batch_mma<DP>  (job, first 1024-point tile, tile count); items of jobs
 //                     that are done, or beyond the current stage's points, are
 //                     skipped
 //   batch_recheck     FP64 re-decision of the near ties of every running job
@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "mma_dev.cuh"
 #include "stage_dev.cuh"
 
 namespace km2 {
@@ -66,6 +67,7 @@ struct BatchInst {
     double tol_fast, tol_slow;
     int d, k, max_iter;
     int stage;               // 0 fast, 1 slow, 2 done
+    int settles;             // its distance kernel leaves open rows to the recheck's FP32 pass
     unsigned int maxabs_x;   // max |x| over X (scale of the slow stage)
     int iters_fast, conv_fast, error;
     double shift_fast;
@@ -85,6 +87,8 @@ __device__ __forceinline__ unsigned int abs_bits(float v)
 
 // ---------------------------------------------------------------- sampling
 
+constexpr int kSampleThreads = 1024;
+
 // Block-level exact radix select: ascending positions (relative to `off`) of
 // the `want` smallest keys splitmix64_at(seed, off + i), i in [0, count).
 __device__ void select_block(unsigned long long seed, unsigned long long off, long long count,
@@ -93,7 +97,7 @@ __device__ void select_block(unsigned long long seed, unsigned long long off, lo
     __shared__ unsigned int hist[256];
     __shared__ unsigned long long prefix;
     __shared__ long long need;
-    __shared__ long long scan[kThreads + 1];
+    __shared__ long long scan[kSampleThreads];
     if (threadIdx.x == 0) { prefix = 0; need = want; }
     __syncthreads();
     for (int pass = 0; pass < 8; ++pass) {
@@ -107,15 +111,23 @@ __device__ void select_block(unsigned long long seed, unsigned long long off, lo
             if (match) atomicAdd(&hist[(key >> shift) & 255ull], 1u);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            long long acc = 0, nd = need;
-            for (int b = 0; b < 256; ++b) {
-                if (nd <= acc + (long long)hist[b]) {
-                    prefix = pf | ((unsigned long long)b << shift);
-                    need = nd - acc;
-                    break;
-                }
-                acc += hist[b];
+        if (threadIdx.x < 32) {
+            // eight bins per lane: the lane whose range holds the need-th key
+            const long long nd = need;
+            const int lane = threadIdx.x;
+            long long sum = 0;
+            for (int b = 0; b < 8; ++b) sum += hist[8 * lane + b];
+            long long incl = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            long long acc = incl - sum;
+            if (nd > acc && nd <= incl) {
+                int b = 8 * lane;
+                while (nd > acc + (long long)hist[b]) acc += hist[b++];
+                prefix = pf | ((unsigned long long)b << shift);
+                need = nd - acc;
             }
         }
         __syncthreads();
@@ -127,9 +139,22 @@ __device__ void select_block(unsigned long long seed, unsigned long long off, lo
     for (long long i = i0; i < i1; ++i) c += splitmix64_at(seed, off + (unsigned long long)i) <= T;
     scan[threadIdx.x] = c;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        long long a = 0;
-        for (int t = 0; t < (int)blockDim.x; ++t) { const long long v = scan[t]; scan[t] = a; a += v; }
+    if (threadIdx.x < 32) {
+        // exclusive scan, 32 threads' counts per lane
+        long long sum = 0;
+        for (int t = 0; t < kSampleThreads / 32; ++t) sum += scan[threadIdx.x * (kSampleThreads / 32) + t];
+        long long a = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long v = __shfl_up_sync(0xffffffffu, a, o);
+            if ((int)threadIdx.x >= o) a += v;
+        }
+        a -= sum;
+        for (int t = 0; t < kSampleThreads / 32; ++t) {
+            const int e = threadIdx.x * (kSampleThreads / 32) + t;
+            const long long v = scan[e];
+            scan[e] = a;
+            a += v;
+        }
     }
     __syncthreads();
     long long o = scan[threadIdx.x];
@@ -138,7 +163,7 @@ __device__ void select_block(unsigned long long seed, unsigned long long off, lo
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kThreads) batch_sample_kernel(BatchInst* insts)
+__global__ void __launch_bounds__(kSampleThreads) batch_sample_kernel(BatchInst* insts)
 {
     BatchInst* I = insts + blockIdx.x;
     select_block(I->seed, 0ull, I->n, I->m, I->subset);
@@ -153,17 +178,21 @@ __global__ void __launch_bounds__(kThreads) batch_sample_kernel(BatchInst* insts
     }
 }
 
-// Gather X_s, its max |x|, the initial centers, and max |x| over X.
+// Gather X_s, its max |x|, the initial centers, and max |x| over X: gridDim.y CTAs
+// per job (one CTA per job took 70 of a 262 ms call of 64 instances, the time of
+// the largest job's 934,613 x 2 values and of the wide jobs beside it).
 __global__ void __launch_bounds__(kThreads) batch_gather_kernel(BatchInst* insts)
 {
     __shared__ unsigned int mx_s, mx_x;
     BatchInst* I = insts + blockIdx.x;
     const int d = I->d;
+    const long long g0 = (long long)blockIdx.y * blockDim.x + threadIdx.x;
+    const long long stride = (long long)gridDim.y * blockDim.x;
     if (threadIdx.x == 0) { mx_s = 0; mx_x = 0; }
     __syncthreads();
     unsigned int a = 0;
     const long long total = I->m * d;
-    for (long long e = threadIdx.x; e < total; e += blockDim.x) {
+    for (long long e = g0; e < total; e += stride) {
         const long long p = e / d;
         const int t = (int)(e - p * d);
         const float v = I->X[I->subset[p] * d + t];
@@ -172,18 +201,25 @@ __global__ void __launch_bounds__(kThreads) batch_gather_kernel(BatchInst* insts
     }
     atomicMax(&mx_s, a);
     unsigned int b = 0;
-    const long long all = I->n * d;
-    for (long long e = threadIdx.x; e < all; e += blockDim.x) b = max(b, abs_bits(__ldg(I->X + e)));
+    const long long all = I->n * d, all4 = all >> 2;       // X is 16-byte aligned
+    const float4* X4 = reinterpret_cast<const float4*>(I->X);
+#pragma unroll 4
+    for (long long e = g0; e < all4; e += stride) {
+        const float4 v = __ldg(X4 + e);
+        b = max(b, max(max(abs_bits(v.x), abs_bits(v.y)), max(abs_bits(v.z), abs_bits(v.w))));
+    }
+    for (long long e = 4 * all4 + g0; e < all; e += stride) b = max(b, abs_bits(__ldg(I->X + e)));
     atomicMax(&mx_x, b);
-    __syncthreads();
-    for (long long e = threadIdx.x; e < (long long)I->k * d; e += blockDim.x) {
+    for (long long e = g0; e < (long long)I->k * d; e += stride) {
         const long long j = e / d;
         const int t = (int)(e - j * d);
-        I->c.c64[e] = (double)I->Xs[I->pos[j] * d + t];
+        I->c.c64[e] = (double)I->X[I->subset[I->pos[j]] * d + t];
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        I->st.maxabs_bits = mx_s;
-        I->maxabs_x = mx_x;
+        // both zero in the descriptors the host sends
+        if (mx_s) atomicMax(&I->st.maxabs_bits, mx_s);
+        if (mx_x) atomicMax(&I->maxabs_x, mx_x);
     }
 }
 
@@ -226,6 +262,13 @@ __global__ void __launch_bounds__(kThreads) batch_mode_kernel(BatchInst* insts, 
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < count) insts[j].st.mode = mode;
+}
+
+// Jobs of dimension lo .. hi: the recheck's FP32 pass settles the screen's open rows.
+__global__ void __launch_bounds__(kThreads) batch_settles_kernel(BatchInst* insts, int count, int lo, int hi)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < count && insts[j].d >= lo && insts[j].d <= hi) insts[j].settles = 1;
 }
 
 // ---------------------------------------------------------------- assign
@@ -546,6 +589,210 @@ batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item
     }
 }
 
+// ---------------------------------------------------------------- assign, tensor-core screen
+
+// The screen of mma_dev.cuh over the same work items (precision AUTO, d >= 8): the
+// job's centers as FP16 fragments in shared memory, 32 rows per warp and step
+// through a stage of cp.async copies that is refilled while their MMAs run (after
+// the sums in a full pass, which reads every row's coordinates again).  Rows it
+// leaves open go to the FP32 chain in the same warp up to d = 16, else to the
+// recheck's FP32 pass.  The autotuner takes it where its passes are faster; in a
+// batch of 64 instances (n 1e3 .. 1e6, d 2 .. 64, k 2 .. 256) the d = 64 class went
+// from 45 % of the call to 0.2 ms an iteration, the call from 262 to 151 ms (with
+// the gather over many CTAs), and to 119 ms with the update over many CTAs.
+template <int DP>
+struct BMma {
+    static constexpr int W = DP <= 16 ? 8 : DP <= 32 ? 16 : 12;      // warps
+    static constexpr int THREADS = 32 * W;
+    static constexpr int MINB = DP <= 16 ? 2 : 1;
+    static constexpr bool SACC = DP <= 32;                           // per-CTA partial sums
+    static constexpr int STAGE = 128 * (DP + 1);                     // 32 rows and labels, at most
+};
+
+template <int DP>
+constexpr size_t batch_mma_smem()
+{
+    return (size_t)(kMaxK / 8) * (mma_bw(DP) * 128 + 32) + (size_t)BMma<DP>::W * BMma<DP>::STAGE +
+           (BMma<DP>::SACC ? (size_t)kMaxK * DP * 8 + (size_t)kMaxK * 4 : 0);
+}
+
+template <int DP>
+__global__ void __launch_bounds__(BMma<DP>::THREADS, BMma<DP>::MINB)
+batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
+{
+    using B = BMma<DP>;
+    constexpr int kT = B::THREADS, W = B::W;
+    extern __shared__ __align__(16) unsigned char smem_b[];
+    uint32_t* sb = reinterpret_cast<uint32_t*>(smem_b);
+    float* sn = reinterpret_cast<float*>(smem_b + (size_t)(kMaxK / 8) * mma_bw(DP) * 128);
+    unsigned char* stages = reinterpret_cast<unsigned char*>(sn + kMaxK);
+    long long* sacc = reinterpret_cast<long long*>(stages + W * B::STAGE);   // k x DP
+    int* scnt = reinterpret_cast<int*>(sacc + (size_t)kMaxK * DP);
+    __shared__ unsigned long long sq[4];     // this item's sum of s^2 (wide_add4 words)
+    __shared__ int s_item;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    unsigned char* stage_mem = stages + warp * B::STAGE;
+    const unsigned stage_u32 = smem_u32(stage_mem);
+    const float* xr = reinterpret_cast<const float*>(stage_mem);
+
+    for (;;) {
+        if (tid == 0) s_item = atomicAdd(next_item, 1);
+        __syncthreads();
+        const int it = s_item;
+        __syncthreads();   // every thread has read it before thread 0 claims the next
+        if (it >= nitems) break;
+        const WorkItem w = items[it];
+        BatchInst* I = insts + w.inst;
+        const int stage = I->stage;
+        if (stage >= 2) continue;
+        const long long npts = stage == 0 ? I->m : I->n;
+        const long long tiles = (npts + kTile - 1) / kTile;
+        if (w.tile0 >= tiles) continue;
+        const float* X = stage == 0 ? I->Xs : I->X;
+        int* labels = stage == 0 ? I->lab_fast : I->lab_slow;
+        StageState* st = &I->st;
+        const int d = I->d, k = I->k;
+        const Centers c = I->c;
+        const bool delta = st->mode == kModeDelta;
+        const float scaleF = st->scaleF;
+        const float thr_base = 2.0f * st->cmax2;
+        const MmaScale ms = mma_scale(st, d, MmaCfg<DP>::KS);
+        const int ntiles = (k + 31) / 32 * 4;
+        mma_load_centers<DP>(c, ntiles, ms, sb, sn);
+        if (B::SACC) {
+            for (int e = tid; e < k * DP; e += kT) sacc[e] = 0;
+            for (int e = tid; e < k; e += kT) scnt[e] = 0;
+        }
+        if (tid < 4) sq[tid] = 0;
+        __syncthreads();
+
+        const long long row_begin = (long long)w.tile0 * kTile;
+        const long long row_end = min(npts, row_begin + (long long)w.ntile * kTile);
+        // 32 rows from row0 on and their labels (read and not used in a full pass)
+        // -> the warp's stage; rows past the end are zero-filled
+        auto issue = [&](long long row0) {
+            if (row0 < row_end) {
+                const int rows = (int)min(32ll, row_end - row0);
+                const unsigned char* src = reinterpret_cast<const unsigned char*>(X + row0 * d);
+                for (int q = lane; q < 8 * d; q += 32) {
+                    const int have = min(16, max(0, rows * d * 4 - 16 * q));
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(stage_u32 + 16 * q),
+                                 "l"(have ? src + 16 * q : src), "r"(have) : "memory");
+                }
+                if (lane < rows) cp_async4(stage_mem + 128 * d + 4 * lane, labels + row0 + lane);
+            }
+            cp_async_commit();
+        };
+        issue(row_begin + 32 * warp);
+        QSum qs;
+        for (long long row0 = row_begin + 32 * warp; row0 < row_end; row0 += 32 * W) {
+            cp_async_wait_all();
+            __syncwarp();
+            const int rows = (int)min(32ll, row_end - row0);
+            uint32_t A[2][MmaCfg<DP>::AREG];
+            float xmax = 0.0f;
+            mma_load_rows<DP, DP == 8>(xr, d, g, t, 0, ms.sx, A[0], xmax);
+            mma_load_rows<DP, DP == 8>(xr, d, g, t, 1, ms.sx, A[1], xmax);
+            const int r = 8 * t + g;                       // this lane's row of the 32
+            const int old = delta ? reinterpret_cast<const int*>(stage_mem + 128 * d)[r] : -1;
+            if (delta) {
+                __syncwarp();                              // every lane has read the stage
+                issue(row0 + 32 * W);
+            }
+            bool open;
+            const float thr = mma_thr(ms, xmax);
+            int lab = k <= 32 ? mma_decide<DP, 4, true>(A, sb, sn, 4, lane, thr, open)
+                              : mma_decide<DP, 4, false>(A, sb, sn, ntiles, lane, thr, open);
+            if (r >= rows) { open = false; lab = old; }
+            unsigned todo = __ballot_sync(0xffffffffu, open);
+            if (todo) {
+                bool listed = open;
+                if (DP <= 16) {
+                    listed = false;
+#pragma unroll 1
+                    while (todo) {
+                        const int o = __ffs(todo) - 1;
+                        todo &= todo - 1;
+                        bool op;
+                        const int l = decide_fp32_row(X + (row0 + 8 * (o & 3) + (o >> 2)) * d, d, c, thr_base, op);
+                        if (lane == o) { lab = l; listed = op; }
+                    }
+                }
+                recheck_append(listed, (int)(row0 + r), I->list, &st->recheck_count);
+                if (listed) lab = old;                     // the recheck moves it
+            }
+            const bool moved = lab != old && label_ok(lab, k, st) && old_label_ok(old, k, st);
+            unsigned mv = __ballot_sync(0xffffffffu, moved);
+            if (mv) {
+                if (moved) {
+                    labels[row0 + r] = lab;
+                    if (B::SACC) {
+                        atomicAdd(scnt + lab, 1);
+                        if (old >= 0) atomicAdd(scnt + old, -1);
+                    } else {
+                        atomicAdd(I->acc.cnt + lab, 1ull);
+                        if (old >= 0) atomicAdd(I->acc.cnt + old, ~0ull);
+                    }
+                }
+                constexpr int LPR = DP < 32 ? DP : 32;     // lanes per moved row
+#pragma unroll 1
+                while (mv) {
+                    int o = -1;
+#pragma unroll
+                    for (int q = 0; q < 32 / LPR; ++q) {
+                        if (lane / LPR == q) o = __ffs(mv) - 1;
+                        mv &= mv - 1;                      // 0 stays 0
+                    }
+                    const int src = o < 0 ? 0 : o;
+                    const int lo = __shfl_sync(0xffffffffu, lab, src), ol = __shfl_sync(0xffffffffu, old, src);
+                    if (o >= 0) {
+                        const int ro = 8 * (o & 3) + (o >> 2);
+                        // delta: the stage holds other rows by now
+                        const float* xg = delta ? X + (row0 + ro) * d : xr + ro * d;
+                        for (int dim = lane % LPR; dim < d; dim += LPR) {
+                            const long long v = to_fixed(xg[dim], scaleF);
+                            if (B::SACC) {
+                                atomicAdd(reinterpret_cast<unsigned long long*>(sacc + lo * DP + dim), (unsigned long long)v);
+                                if (ol >= 0)
+                                    atomicAdd(reinterpret_cast<unsigned long long*>(sacc + ol * DP + dim), (unsigned long long)(-v));
+                            } else {
+                                split_add(I->acc.s_lo + (long long)lo * d + dim, I->acc.s_hi + (long long)lo * d + dim, v);
+                                if (ol >= 0)
+                                    split_add(I->acc.s_lo + (long long)ol * d + dim, I->acc.s_hi + (long long)ol * d + dim, -v);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                }
+            }
+            if (!delta) {
+                for (int e = lane; e < rows * d; e += 32) qs.add(xr[e], scaleF);
+                qs.fold();
+                __syncwarp();                              // done with the stage
+                issue(row0 + 32 * W);
+            }
+        }
+        cp_async_wait_all();
+        if (!delta) {
+            const unsigned __int128 q = warp_sum_u128(qs.total);
+            if (lane == 0 && q) wide_add4(sq, q);
+        }
+        __syncthreads();
+        if (B::SACC) {
+            for (int e = tid; e < k * DP; e += kT) {
+                const int j = e / DP, dim = e - j * DP;
+                const long long v = sacc[e];
+                if (v && dim < d)
+                    split_add(I->acc.s_lo + (long long)j * d + dim, I->acc.s_hi + (long long)j * d + dim, v);
+            }
+            for (int j = tid; j < k; j += kT)
+                if (scnt[j]) atomicAdd(I->acc.cnt + j, (unsigned long long)(long long)scnt[j]);
+        }
+        if (tid < 4 && sq[tid]) atomicAdd(&st->q[tid], sq[tid]);
+        __syncthreads();   // the next item reuses shared memory
+    }
+}
+
 // ---------------------------------------------------------------- recheck, finalize, control
 
 // The recheck of the whole batch as one flat list: prefix[j] = flagged points
@@ -597,23 +844,53 @@ __global__ void __launch_bounds__(kThreads) batch_recheck_flat_kernel(BatchInst*
         BatchInst* I = insts + lo;
         const float* X = I->stage == 0 ? I->Xs : I->X;
         int* labels = I->stage == 0 ? I->lab_fast : I->lab_slow;
-        recheck_point(X, I->d, I->c, labels, I->list[w - prefix[lo]], &I->st, I->acc,
-                      cache[threadIdx.x >> 5], 256);
+        const bool settled = recheck_point(X, I->d, I->c, labels, I->list[w - prefix[lo]], &I->st,
+                                           I->acc, cache[threadIdx.x >> 5], 256);
+        // decided by the FP32 pass alone: not a point re-evaluated in FP64
+        if (settled && I->settles && (threadIdx.x & 31) == 0)
+            atomicAdd(reinterpret_cast<unsigned long long*>(&I->st.rechecked_total), ~0ull);
     }
 }
 
+// gridDim.y CTAs per job share its centers (one warp each) and divisions; the job's
+// last CTA reduces and moves the job on.  FP64 bound like finalize_kernel: with one
+// CTA per job a k = 256, d = 64 job held an SM for 200 us an iteration, 41 of the 151
+// ms of a batch of 64.
 __global__ void __launch_bounds__(kThreads) batch_finalize_kernel(BatchInst* insts, int* active)
 {
     __shared__ FinalizeSmem sm;
-    __shared__ int switched;
+    __shared__ int switched, last;
     BatchInst* I = insts + blockIdx.x;
     const int stage = I->stage;
     if (stage >= 2) return;
-    if (I->st.error) {
+    const bool error = I->st.error != 0;
+    if (!error) {
+        const double inv = I->st.inv_scaleF;
+        const int it = I->st.iter, k = I->k;
+        const TrajDev none{nullptr, nullptr, nullptr, nullptr};
+        for (int j = (int)(blockIdx.y + gridDim.y * (threadIdx.x >> 5)); j < k;
+             j += (int)(gridDim.y * (blockDim.x >> 5)))
+            finalize_center_warp(I->acc, I->c, inv, j, I->clus, none, it);
+        __syncthreads();
+        for (int j = (int)(blockIdx.y + gridDim.y * threadIdx.x); j < k; j += (int)(gridDim.y * blockDim.x))
+            finalize_divide(k, I->acc.cnt, inv, I->clus, j);
+    }
+    if (gridDim.y > 1) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&I->st.ticket, 1u) == gridDim.y - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) I->st.ticket = 0;
+    } else {
+        __syncthreads();
+    }
+    if (error) {
         if (threadIdx.x == 0) { I->stage = 2; I->error = I->st.error; }
         return;
     }
-    finalize_block(I->acc, I->c, &I->st, TrajDev{nullptr, nullptr, nullptr, nullptr}, I->clus, sm);
+    finalize_reduce_block(I->k, I->acc.cnt, &I->st, TrajDev{nullptr, nullptr, nullptr, nullptr}, I->clus, sm);
     if (threadIdx.x == 0) {
         switched = 0;
         if (I->st.done) {
@@ -698,11 +975,30 @@ int launch_batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int
     return KMEANS2_OK;
 }
 
-// Tile shape of the distance kernel: point slots per lane and lanes per point.
+// Tile shape of the distance kernel: point slots per lane and lanes per point;
+// p = kMmaShape: the tensor-core screen.
 struct TileShape {
     int p = 0;
     int g = 0;
 };
+constexpr int kMmaShape = -1;
+
+// Dimensions the screen takes (its keys are less precise than the FP32 chain's below 8).
+bool mma_dims(int d) { return d >= 8; }
+
+template <int DP>
+int launch_batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item,
+                     cudaStream_t s, int sm_count)
+{
+    const size_t sm = batch_mma_smem<DP>();
+    const void* kfn = (const void*)batch_mma<DP>;
+    KM2_TRY(set_max_dynamic_smem(kfn, (int)sm));
+    const int grid = std::max(1, std::min(sm_count * BMma<DP>::MINB, nitems));
+    ++g_launches;
+    batch_mma<DP><<<grid, BMma<DP>::THREADS, sm, s>>>(insts, items, nitems, next_item);
+    KM2_CUDA(cudaGetLastError());
+    return KMEANS2_OK;
+}
 
 // Tile shapes the autotuner may pick for a dimension class: as many point
 // slots as the registers hold (a lane keeps p DC / g floats); shared points
@@ -717,11 +1013,13 @@ std::vector<TileShape> tile_shapes(int dc)
 
 // Debug builds (KM2_DEBUG_CHECKS): KMEANS2_DEBUG_BATCH_POINTS = "p" or "pxg"
 // forces one tile shape on every dimension class that offers it, without
-// tuning, so that a test can run each kernel variant; p = 0 otherwise.
+// tuning, so that a test can run each kernel variant, and "mma" the screen on
+// every job it may take; p = 0 otherwise.
 TileShape forced_tile_shape(int dc)
 {
 #ifdef KM2_DEBUG_CHECKS
     const char* v = std::getenv("KMEANS2_DEBUG_BATCH_POINTS");
+    if (v && std::strcmp(v, "mma") == 0) return TileShape{kMmaShape, 0};
     if (v && *v) {
         char* end = nullptr;
         TileShape f;
@@ -739,6 +1037,12 @@ TileShape forced_tile_shape(int dc)
 int launch_class(int dc, TileShape sh, BatchInst* insts, const WorkItem* items, int nitems,
                  int* next_item, cudaStream_t s, int sm_count)
 {
+    if (sh.p == kMmaShape) {
+        if (dc == 8) return launch_batch_mma<8>(insts, items, nitems, next_item, s, sm_count);
+        if (dc == 16) return launch_batch_mma<16>(insts, items, nitems, next_item, s, sm_count);
+        if (dc == 32) return launch_batch_mma<32>(insts, items, nitems, next_item, s, sm_count);
+        return launch_batch_mma<64>(insts, items, nitems, next_item, s, sm_count);
+    }
 #define KM2_BA(DD, PP, GG)                                                                  \
     if (dc == DD && sh.p == PP && sh.g == GG)                                               \
         return launch_batch_assign<DD, PP, GG>(insts, items, nitems, next_item, s, sm_count);
@@ -753,6 +1057,12 @@ int launch_class(int dc, TileShape sh, BatchInst* insts, const WorkItem* items, 
 std::mutex g_tune_mu;
 // dimension class -> (tile shape, tiles per work item)
 std::map<int, std::pair<TileShape, int>> g_tuned;
+// dimension class -> tiles per work item of the screen where it is faster than the
+// class's CUDA-core shape (0: it is not)
+std::map<int, int> g_tuned_mma;
+
+// Six dimension classes, each split in jobs the screen takes and others.
+constexpr int kMaxClasses = 12;
 
 struct ClassItems {
     int dc = 0;
@@ -808,7 +1118,7 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
     kmeans2_default_options(&o);
     if (opt) o = *opt;
     if (o.precision != KMEANS2_PRECISION_FP32 && o.precision != KMEANS2_PRECISION_AUTO) {
-        set_last_error_text("the batched form runs the FP32 CUDA-core kernels only");
+        set_last_error_text("the batched form runs the FP32 form only");
         return KMEANS2_ERR_UNSUPPORTED;
     }
     for (int j = 0; j < count; ++j) {
@@ -863,8 +1173,8 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
         int* counters = nullptr;
         KM2_TRY(ws.alloc((void**)&arena, total, s));
         KM2_TRY(ws.alloc((void**)&dinst, sizeof(BatchInst) * (size_t)count, s));
-        // active, iteration, 6 item counters, active count handed to the host
-        KM2_TRY(ws.alloc((void**)&counters, 9 * sizeof(int), s));
+        // active, iteration, an item counter per class, active count handed to the host
+        KM2_TRY(ws.alloc((void**)&counters, (kMaxClasses + 3) * sizeof(int), s));
         long long* rprefix = nullptr;      // flat recheck list: per-job offsets, total
         KM2_TRY(ws.alloc((void**)&rprefix, sizeof(long long) * ((size_t)count + 1), s));
         for (int j = 0; j < count; ++j) {
@@ -908,79 +1218,111 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
         }
         KM2_CUDA(cudaMemcpyAsync(dinst, hi.data(), sizeof(BatchInst) * (size_t)count,
                                  cudaMemcpyHostToDevice, s));
-        KM2_CUDA(cudaMemsetAsync(counters, 0, 9 * sizeof(int), s));
+        KM2_CUDA(cudaMemsetAsync(counters, 0, (kMaxClasses + 3) * sizeof(int), s));
         g_launches += 3;
-        batch_sample_kernel<<<count, kThreads, 0, s>>>(dinst);
-        batch_gather_kernel<<<count, kThreads, 0, s>>>(dinst);
+        batch_sample_kernel<<<count, kSampleThreads, 0, s>>>(dinst);
+        // finalize: centers over up to 32 CTAs per job while the jobs leave SMs idle
+        const int fslices = std::max(1, std::min(32, ws.sm_count * 8 / count));
+        // about eight CTAs per SM over all jobs, at least one and at most 64 per job
+        const int slices = std::max(1, std::min(64, ws.sm_count * 8 / count));
+        batch_gather_kernel<<<dim3((unsigned)count, (unsigned)slices), kThreads, 0, s>>>(dinst);
         batch_prep_kernel<<<count, kThreads, 0, s>>>(dinst);
         KM2_CUDA(cudaGetLastError());
 
         // ---- work items per dimension class, item size from the autotuner
+        // key: 2 class + (the screen may take the job: precision AUTO)
+        const bool screen = o.precision == KMEANS2_PRECISION_AUTO;
         std::map<int, std::vector<int>> members;
-        for (int j = 0; j < count; ++j) members[dclass(jobs[j].d)].push_back(j);
+        for (int j = 0; j < count; ++j)
+            members[2 * dclass(jobs[j].d) + ((screen && mma_dims(jobs[j].d)) ? 1 : 0)].push_back(j);
         std::vector<ClassItems> classes;
+        bool settle32 = false, settle64 = false;
         for (auto& kv : members) {
             ClassItems ci;
-            ci.dc = kv.first;
+            ci.dc = kv.first / 2;
+            const bool mma_ok = (kv.first & 1) != 0;
             int tpi = 0;
             TileShape shape = forced_tile_shape(ci.dc);
-            if (shape.p > 0) {
+            const bool forced_mma = shape.p == kMmaShape;
+            const bool forced = shape.p > 0 || forced_mma;
+            int mma_tpi = forced || !mma_ok ? 0 : -1;     // -1: not tuned yet
+            if (forced) {
                 tpi = 2;
+                if (forced_mma) {
+                    shape = tile_shapes(ci.dc)[0];
+                    mma_tpi = mma_ok ? 2 : 0;
+                }
             } else {
                 std::lock_guard<std::mutex> lock(g_tune_mu);
                 auto f = g_tuned.find(ci.dc);
                 if (f != g_tuned.end()) { shape = f->second.first; tpi = f->second.second; }
+                auto m = g_tuned_mma.find(ci.dc);
+                if (mma_tpi < 0 && m != g_tuned_mma.end()) mma_tpi = m->second;
             }
-            if (tpi == 0) {
+            if (tpi == 0 || mma_tpi < 0) {
                 // time the real first pass and a delta pass after it for each
                 // tile shape and item size (tiles per work item), resetting the
                 // sums between trials: small items keep every SM busy once only a
                 // few jobs still run, more point slots per lane reuse each center
-                // load more often
+                // load more often.  The delta pass counts ten times where the
+                // screen is compared: its full pass, with the sums, is no measure
+                // of the iterations that follow.
                 const int cand[4] = {1, 2, 4, 8};
                 static_assert(8 <= kMaxTilesPerItem, "item partial sums must stay below 2^62");
-                float best_ms = 0.f;
-                bool first = true;
                 cudaEvent_t e0, e1, e2, e3;
                 KM2_CUDA(cudaEventCreate(&e0));
                 KM2_CUDA(cudaEventCreate(&e1));
                 KM2_CUDA(cudaEventCreate(&e2));
                 KM2_CUDA(cudaEventCreate(&e3));
-                for (const TileShape& sh : tile_shapes(ci.dc)) {
-                    for (int c = 0; c < 4; ++c) {
-                        ClassItems trial;
-                        build_items(trial, kv.second, nvec, cand[c]);
-                        KM2_TRY(ws.alloc((void**)&trial.dev, sizeof(WorkItem) * (size_t)trial.count, s));
-                        KM2_CUDA(cudaMemcpyAsync(trial.dev, trial.host.data(),
-                                                 sizeof(WorkItem) * (size_t)trial.count,
-                                                 cudaMemcpyHostToDevice, s));
-                        // the full first pass, then a delta pass over the labels it
-                        // wrote (same centers: no label moves), which is what the
-                        // later iterations of a fit cost
-                        KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
-                        KM2_CUDA(cudaEventRecord(e0, s));
-                        KM2_TRY(launch_class(ci.dc, sh, dinst, trial.dev, trial.count, counters + 2,
-                                             s, ws.sm_count));
-                        KM2_CUDA(cudaEventRecord(e1, s));
-                        g_launches += 2;
-                        batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
-                        batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-                            dinst, count, kModeDelta);
-                        KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
-                        KM2_CUDA(cudaEventRecord(e2, s));
-                        KM2_TRY(launch_class(ci.dc, sh, dinst, trial.dev, trial.count, counters + 2,
-                                             s, ws.sm_count));
-                        KM2_CUDA(cudaEventRecord(e3, s));
-                        g_launches += 2;
-                        batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
-                        batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-                            dinst, count, kModeFull);
-                        KM2_CUDA(cudaEventSynchronize(e3));
-                        float ms = 0.f, ms2 = 0.f;
-                        KM2_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-                        KM2_CUDA(cudaEventElapsedTime(&ms2, e2, e3));
-                        ms += ms2;
-                        if (first || ms < best_ms) { best_ms = ms; tpi = cand[c]; shape = sh; first = false; }
+                auto trial = [&](const TileShape& sh, int tiles, float& full, float& later) -> int {
+                    ClassItems tr;
+                    build_items(tr, kv.second, nvec, tiles);
+                    KM2_TRY(ws.alloc((void**)&tr.dev, sizeof(WorkItem) * (size_t)tr.count, s));
+                    KM2_CUDA(cudaMemcpyAsync(tr.dev, tr.host.data(), sizeof(WorkItem) * (size_t)tr.count,
+                                             cudaMemcpyHostToDevice, s));
+                    // the full first pass, then a delta pass over the labels it
+                    // wrote (same centers: no label moves), which is what the
+                    // later iterations of a fit cost
+                    KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
+                    KM2_CUDA(cudaEventRecord(e0, s));
+                    KM2_TRY(launch_class(ci.dc, sh, dinst, tr.dev, tr.count, counters + 2, s, ws.sm_count));
+                    KM2_CUDA(cudaEventRecord(e1, s));
+                    g_launches += 2;
+                    batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
+                    batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+                        dinst, count, kModeDelta);
+                    KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
+                    KM2_CUDA(cudaEventRecord(e2, s));
+                    KM2_TRY(launch_class(ci.dc, sh, dinst, tr.dev, tr.count, counters + 2, s, ws.sm_count));
+                    KM2_CUDA(cudaEventRecord(e3, s));
+                    g_launches += 2;
+                    batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
+                    batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+                        dinst, count, kModeFull);
+                    KM2_CUDA(cudaEventSynchronize(e3));
+                    KM2_CUDA(cudaEventElapsedTime(&full, e0, e1));
+                    KM2_CUDA(cudaEventElapsedTime(&later, e2, e3));
+                    return KMEANS2_OK;
+                };
+                float core_full = 0.f, core_later = 0.f, full = 0.f, later = 0.f;
+                if (tpi == 0) {
+                    bool first = true;
+                    for (const TileShape& sh : tile_shapes(ci.dc))
+                        for (int c : cand) {
+                            KM2_TRY(trial(sh, c, full, later));
+                            if (first || full + later < core_full + core_later) {
+                                core_full = full; core_later = later; tpi = c; shape = sh; first = false;
+                            }
+                        }
+                } else if (mma_tpi < 0) {
+                    KM2_TRY(trial(shape, tpi, core_full, core_later));
+                }
+                if (mma_tpi < 0) {
+                    float best = core_full + 10.f * core_later;
+                    mma_tpi = 0;
+                    for (int c : cand) {
+                        KM2_TRY(trial(TileShape{kMmaShape, 0}, c, full, later));
+                        if (full + 10.f * later < best) { best = full + 10.f * later; mma_tpi = c; }
                     }
                 }
                 cudaEventDestroy(e0);
@@ -989,6 +1331,13 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                 cudaEventDestroy(e3);
                 std::lock_guard<std::mutex> lock(g_tune_mu);
                 g_tuned[ci.dc] = std::make_pair(shape, tpi);
+                if (mma_ok) g_tuned_mma[ci.dc] = mma_tpi;
+            }
+            if (mma_tpi > 0) {
+                shape = TileShape{kMmaShape, 0};
+                tpi = mma_tpi;
+                settle32 = settle32 || ci.dc == 32;
+                settle64 = settle64 || ci.dc == 64;
             }
             ci.shape = shape;
             build_items(ci, kv.second, nvec, tpi);
@@ -998,7 +1347,12 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
             classes.push_back(std::move(ci));
         }
 
-        KM2_CUDA(cudaMemsetAsync(counters + 2, 0, 6 * sizeof(int), s));
+        if (settle32 || settle64) {
+            ++g_launches;
+            batch_settles_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+                dinst, count, settle32 ? 17 : 33, settle64 ? 64 : 32);
+        }
+        KM2_CUDA(cudaMemsetAsync(counters + 2, 0, kMaxClasses * sizeof(int), s));
         // one side stream per dimension class: the classes' distance kernels run
         // side by side (parallel branches of the graph body)
         std::vector<cudaStream_t> side(classes.size(), nullptr);
@@ -1045,12 +1399,12 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                 batch_recheck_scan_kernel<<<1, 1024, 0, s>>>(dinst, count, rprefix);
                 batch_recheck_flat_kernel<<<ws.sm_count * 4, kThreads, 0, s>>>(dinst, count, rprefix);
                 ++g_launches;
-                batch_finalize_kernel<<<count, kThreads, 0, s>>>(dinst, counters);
+                batch_finalize_kernel<<<dim3((unsigned)count, (unsigned)fslices), kThreads, 0, s>>>(dinst, counters);
                 ++g_launches;
                 batch_step_kernel<<<1, 1, 0, s>>>(counters, counters + 1, counters + 2,
-                                                  (int)classes.size(), counters + 8);
+                                                  (int)classes.size(), counters + 2 + kMaxClasses);
                 int active = 0;
-                cudaError_t e = cudaMemcpyAsync(&active, counters + 8, sizeof(int),
+                cudaError_t e = cudaMemcpyAsync(&active, counters + 2 + kMaxClasses, sizeof(int),
                                                 cudaMemcpyDeviceToHost, s);
                 if (e == cudaSuccess) e = cudaStreamSynchronize(s);
                 if (e != cudaSuccess) { set_last_error("batched loop", e); rc = KMEANS2_ERR_CUDA; break; }
@@ -1089,7 +1443,7 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
             if (rc == KMEANS2_OK) {
                 batch_recheck_scan_kernel<<<1, 1024, 0, s>>>(dinst, count, rprefix);
                 batch_recheck_flat_kernel<<<ws.sm_count * 4, kThreads, 0, s>>>(dinst, count, rprefix);
-                batch_finalize_kernel<<<count, kThreads, 0, s>>>(dinst, counters);
+                batch_finalize_kernel<<<dim3((unsigned)count, (unsigned)fslices), kThreads, 0, s>>>(dinst, counters);
                 batch_control_kernel<<<1, 1, 0, s>>>(counters, counters + 1, counters + 2,
                                                      (int)classes.size(), cap,
                                                      (unsigned long long)handle);

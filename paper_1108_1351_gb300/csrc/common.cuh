@@ -155,6 +155,31 @@ __device__ __forceinline__ unsigned __int128 sq_fixed(float x, float scale)
     return (unsigned __int128)a * a;
 }
 
+// Partial sum of s^2 over coordinates, s = to_fixed(x, 2^F) = a 2^24 + b with |a| <=
+// 2^22, |b| <= 2^23: three 64-bit sums (wide multiply-adds), folded into 128
+// bits every 2^16 coordinates at most (each term is below 2^47).
+struct QSum {
+    unsigned __int128 total = 0;
+    unsigned long long aa = 0, bb = 0;
+    long long ab = 0;
+    __device__ __forceinline__ void add(float x, float scale)
+    {
+        const float t = x * scale;                                   // |t| < 2^46, exact
+        const float v = fmaf(t, 5.9604644775390625e-8f, 12582912.0f);   // 1.5 2^23 + rint(t 2^-24)
+        const int a = __float_as_int(v) - 0x4b400000;
+        const int b = __float2int_rn(fmaf(v - 12582912.0f, -16777216.0f, t));
+        aa += (unsigned long long)((long long)a * a);
+        ab += (long long)a * b;
+        bb += (unsigned long long)((long long)b * b);
+    }
+    __device__ __forceinline__ void fold()
+    {
+        total += ((unsigned __int128)aa << 48) + bb + (unsigned __int128)((__int128)ab * ((__int128)1 << 25));
+        aa = bb = 0;
+        ab = 0;
+    }
+};
+
 // Adds v (< 2^128) to a wide accumulator w[0..3] whose value is
 // sum_i w[i] 2^(32 i): piece i of v (32 bits) goes to w[i].  Each word gains
 // less than 2^32 per call, so fewer than 2^31 calls cannot wrap it.

@@ -66,31 +66,6 @@ __global__ void maxabs_kernel(const float* __restrict__ X, long long count, int 
     block_max_to(m, st);
 }
 
-// Partial sum of s^2 over coordinates, s = to_fixed(x, 2^F) = a 2^24 + b with |a| <=
-// 2^22, |b| <= 2^23: three 64-bit sums (wide multiply-adds), folded into 128
-// bits every 2^16 coordinates at most (each term is below 2^47).
-struct QSum {
-    unsigned __int128 total = 0;
-    unsigned long long aa = 0, bb = 0;
-    long long ab = 0;
-    __device__ __forceinline__ void add(float x, float scale)
-    {
-        const float t = x * scale;                                   // |t| < 2^46, exact
-        const float v = fmaf(t, 5.9604644775390625e-8f, 12582912.0f);   // 1.5 2^23 + rint(t 2^-24)
-        const int a = __float_as_int(v) - 0x4b400000;
-        const int b = __float2int_rn(fmaf(v - 12582912.0f, -16777216.0f, t));
-        aa += (unsigned long long)((long long)a * a);
-        ab += (long long)a * b;
-        bb += (unsigned long long)((long long)b * b);
-    }
-    __device__ __forceinline__ void fold()
-    {
-        total += ((unsigned __int128)aa << 48) + bb + (unsigned __int128)((__int128)ab * ((__int128)1 << 25));
-        aa = bb = 0;
-        ab = 0;
-    }
-};
-
 // Exact sum of s^2 over count coordinates (the same integers the cluster sums
 // add), into st->q.  Memory-bound: ~9 instructions per coordinate (one 128-bit
 // product and sum per coordinate took 2.5x the time of reading X; n = 5e5, d =

@@ -3,7 +3,7 @@
 // that both run exactly the same arithmetic:
 //   center_prep_block  FP32 / transposed copies of the FP64 centers, ||c||^2
 //   stage_init_dev     fixed-point scales and loop state of one stage
-//   finalize_block     new centers = cluster means (Lloyd's method, Section 4.1),
+//   finalize_*         new centers = cluster means (Lloyd's method, Section 4.1),
 //                      largest movement (stop test, Sections 5-6), J (Eq. 3)
 //   recheck_warps      FP64 re-evaluation of near-tie points (ties -> lowest index)
 #pragma once
@@ -421,22 +421,6 @@ static __device__ void finalize_reduce_block(int k, const unsigned long long* cn
         }
     }
     __syncthreads();
-}
-
-// Whole block of 256 threads.  New centers, movement, J; loop control for the
-// next iteration (thread 0 updates st).  clus: kClusSlots k words of scratch.
-// Ends with the block synchronised.
-static __device__ void finalize_block(Accum acc, Centers c, StageState* st, TrajDev tr,
-                                      double* clus, FinalizeSmem& sm)
-{
-    const double inv = st->inv_scaleF;
-    const int it = st->iter;
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int j = warp; j < c.k; j += nw) finalize_center_warp(acc, c, inv, j, clus, tr, it);
-    __syncthreads();
-    for (int j = threadIdx.x; j < c.k; j += blockDim.x) finalize_divide(c.k, acc.cnt, inv, clus, j);
-    __syncthreads();
-    finalize_reduce_block(c.k, acc.cnt, st, tr, clus, sm);
 }
 
 // FP32 D_j = ||c_j||^2 - 2 x.c_j of one point against centers j0 + 32 i

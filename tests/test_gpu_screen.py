@@ -6,6 +6,10 @@ must equal the oracle's (labels exactly; centers and J within the helpers'
 derived tolerances) and the plain FP32 form's bit for bit.  Sizes lie around
 the edges of its tiles: 32 / 64 rows per warp and 256 to 512 per step, 8 centers per
 block, 16 / 32 per chunk, d at, between and outside the padded sizes 8 .. 128."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -84,3 +88,37 @@ def test_fits_and_other_entry_points(n, d, k):
     C = Xd[:k].double()
     p, q = km.step_noalloc(Xd, C), km.step(Xd, C, precision="fp32")
     assert torch.equal(p[1], q[1]) and torch.equal(p[0], q[0]) and p[2:] == q[2:]
+
+
+BATCH = r"""
+import sys, torch
+sys.path.insert(0, ROOT)
+import paper_1108_1351_gb300 as km
+from paper_1108_1351_gb300 import synth
+assert km.LIB_PATH.endswith("libkmeans2_debug.so")
+jobs = [(1, 8, 1), (33, 9, 5), (1023, 16, 16), (1024, 8, 33), (1025, 17, 32), (4099, 31, 70),
+        (6001, 32, 256), (5000, 33, 12), (3001, 50, 100), (7003, 64, 200), (2500, 7, 20), (2049, 2, 9)]
+Xs = [synth.aniso_gaussian_noise(n, d, max(2, k // 2), 7 + j, device="cuda") if n > 40 else
+      synth.iso_gaussian_mixture(n, d, 1, j, device="cuda") for j, (n, d, k) in enumerate(jobs)]
+ks = [k for _, _, k in jobs]
+rs, rc = km.fit_batched(Xs, ks, 0.3, list(range(len(jobs))), 1e-6, 25)
+assert rc == 0
+for j, (X, k, r) in enumerate(zip(Xs, ks, rs)):
+    a = km.fit(X, k, 0.3, j, 1e-6, 25, precision="fp32")
+    assert torch.equal(a.labels, r.labels) and torch.equal(a.centers, r.centers), jobs[j]
+    assert (a.J, a.iters_fast, a.iters_slow, a.empty_clusters) == (r.J, r.iters_fast, r.iters_slow, r.empty_clusters), jobs[j]
+print("ok")
+"""
+
+
+def test_batched_screen_equals_single_fits():
+    """The batched form with the screen forced on every job it may take (debug
+    build, device index checks on): items of 1,024 rows and their remainders,
+    every dimension class, k at the chunk edges."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    from paper_1108_1351_gb300 import build
+    build.build(debug=True)
+    env = dict(os.environ, KMEANS2_DEBUG="1", KMEANS2_DEBUG_BATCH_POINTS="mma")
+    r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % root + BATCH], capture_output=True,
+                       text=True, env=env, timeout=600, cwd=root)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-3000:]
