@@ -198,21 +198,35 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
     w.c.dpad = (d + 7) / 8 * 8;
     w.max_iter = max_iter;
     w.ws = &ws;
-    size_t kd = (size_t)k * d;
-    KM2_TRY(ws.alloc((void**)&w.c.c64, kd * sizeof(double), s));
-    KM2_TRY(ws.alloc((void**)&w.c.c32, kd * sizeof(float), s));
-    KM2_TRY(ws.alloc((void**)&w.c.c32t, (size_t)w.c.dpad * w.c.kpad * sizeof(float), s));
-    KM2_TRY(ws.alloc((void**)&w.c.cnorm, (size_t)center_norm_len(k, w.c.kpad) * sizeof(float), s));
-    KM2_TRY(ws.alloc((void**)&w.acc.s_lo, kd * 8, s));
-    KM2_TRY(ws.alloc((void**)&w.acc.s_hi, kd * 8, s));
-    KM2_TRY(ws.alloc((void**)&w.acc.cnt, (size_t)k * 8, s));
-    KM2_TRY(ws.alloc((void**)&w.st, sizeof(StageState), s));
-    KM2_TRY(ws.alloc((void**)&w.list, (size_t)(list_cap > 0 ? list_cap : 1) * sizeof(int), s));
-    KM2_TRY(ws.alloc((void**)&w.clus, (size_t)kClusSlots * k * sizeof(double), s));
-    KM2_TRY(ws.alloc((void**)&w.traj_J, (size_t)max_iter * sizeof(double), s));
-    KM2_TRY(ws.alloc((void**)&w.traj_shift, (size_t)max_iter * sizeof(double), s));
-    // (the split layout: a fit may switch from FP16 to split BF16 between stages)
-    if (tc16_form(w.form)) KM2_TRY(ws.alloc((void**)&w.cb, bf16_cb_bytes(d, k, 0), s));
+    // one allocation, carved in 256-byte steps: a pool allocation and its release
+    // cost the host 2 us, a dozen of them a fifth of a small step
+    const size_t kd = (size_t)k * d;
+    struct Piece { void** p; size_t bytes; };
+    const Piece pieces[] = {
+        {(void**)&w.c.c64, kd * sizeof(double)},
+        {(void**)&w.c.c32, kd * sizeof(float)},
+        {(void**)&w.c.c32t, (size_t)w.c.dpad * w.c.kpad * sizeof(float)},
+        {(void**)&w.c.cnorm, (size_t)center_norm_len(k, w.c.kpad) * sizeof(float)},
+        {(void**)&w.acc.s_lo, kd * 8},
+        {(void**)&w.acc.s_hi, kd * 8},
+        {(void**)&w.acc.cnt, (size_t)k * 8},
+        {(void**)&w.st, sizeof(StageState)},
+        {(void**)&w.list, (size_t)(list_cap > 0 ? list_cap : 1) * sizeof(int)},
+        {(void**)&w.clus, (size_t)kClusSlots * k * sizeof(double)},
+        {(void**)&w.traj_J, (size_t)max_iter * sizeof(double)},
+        {(void**)&w.traj_shift, (size_t)max_iter * sizeof(double)},
+        // (the split layout: a fit may switch from FP16 to split BF16 between stages)
+        {(void**)&w.cb, tc16_form(w.form) ? bf16_cb_bytes(d, k, 0) : 0},
+    };
+    size_t total = 0;
+    for (const Piece& q : pieces) total += (q.bytes + 255) / 256 * 256;
+    unsigned char* base = nullptr;
+    KM2_TRY(ws.alloc((void**)&base, total, s));
+    for (const Piece& q : pieces) {
+        if (q.bytes == 0) continue;
+        *q.p = base;
+        base += (q.bytes + 255) / 256 * 256;
+    }
     return KMEANS2_OK;
 }
 
@@ -322,12 +336,11 @@ int choose_form(int requested, int d, int k, const float* X, int* form)
 
 // One Lloyd iteration: assign -> recheck -> finalize.
 int launch_iteration(const float* X, long long n, int d, Workspace& w, int* labels,
-                     unsigned long long handle, int use_cond, cudaStream_t s, int sm_count)
+                     unsigned long long handle, int use_cond, int stop, cudaStream_t s, int sm_count)
 {
     KM2_TRY(launch_assign(X, n, d, w, labels, s, sm_count));
     KM2_TRY(launch_stage_recheck(X, d, w, labels, s, sm_count));
-    KM2_TRY(launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, handle, use_cond,
-                            s));
+    KM2_TRY(launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, handle, use_cond, stop, s));
     return KMEANS2_OK;
 }
 
@@ -360,7 +373,7 @@ int run_loop_graph(const float* X, long long n, int d, Workspace& w, int* labels
                                           cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) { set_last_error("cudaStreamBeginCaptureToGraph", e); rc = KMEANS2_ERR_CUDA; break; }
         const long long body0 = g_launches;
-        rc = launch_iteration(X, n, d, w, labels, (unsigned long long)handle, 1, s, sm_count);
+        rc = launch_iteration(X, n, d, w, labels, (unsigned long long)handle, 1, 0, s, sm_count);
         const long long body_launches = g_launches - body0;
         cudaGraph_t captured = nullptr;
         e = cudaStreamEndCapture(s, &captured);
@@ -404,9 +417,9 @@ int run_loop_host(const float* X, long long n, int d, Workspace& w, int* labels,
             if (rc == KMEANS2_OK)
                 rc = launch_stage_recheck(X, d, w, labels, s, sm_count);
             if (rc == KMEANS2_OK)
-                rc = launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, 0ull, 0, s);
+                rc = launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, 0ull, 0, 0, s);
         } else {
-            rc = launch_iteration(X, n, d, w, labels, 0ull, 0, s, sm_count);
+            rc = launch_iteration(X, n, d, w, labels, 0ull, 0, 0, s, sm_count);
         }
         if (rc != KMEANS2_OK) break;
         int done = 0;
@@ -427,6 +440,35 @@ int run_loop_host(const float* X, long long n, int d, Workspace& w, int* labels,
     if (ev1) cudaEventDestroy(ev1);
     return rc;
 }
+
+// Iterations queued ahead of the read-back that says whether the stage is done:
+// what is queued behind the last one returns at once (kErrStopped).  For short
+// iterations, where a while-graph costs more to build than the stage to run and a
+// read-back per iteration as much as the iteration.  out: the final state;
+// publish: device buffer that receives the centers before the read-back, or null.
+int run_loop_queued(const float* X, long long n, int d, Workspace& w, int* labels, int max_iter,
+                    cudaStream_t s, int sm_count, StageState& out, double* publish)
+{
+    int queued = 0, chunk = 4;
+    for (;;) {
+        const int b = std::min(chunk, max_iter - queued);
+        for (int i = 0; i < b; ++i)
+            KM2_TRY(launch_iteration(X, n, d, w, labels, 0ull, 0, 1, s, sm_count));
+        queued += b;
+        if (publish) KM2_TRY(launch_publish_centers(w.st, w.c.c64, (long long)w.c.k * d, publish, s));
+        KM2_CUDA(cudaMemcpyAsync(&out, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
+        KM2_CUDA(cudaStreamSynchronize(s));
+        if (out.error || out.done || queued >= max_iter) break;
+        chunk = std::min(2 * chunk, 32);
+    }
+    if (out.error == kErrStopped) out.error = 0;
+    return KMEANS2_OK;
+}
+
+// n k d of an iteration up to which the queued loop runs it (at most ~60 us on the
+// CUDA cores, ~20 through the screen; building and starting a while-graph takes
+// ~150 us per stage).
+constexpr double kQueuedWork = 2.0e9;
 
 int map_stage_error(int err)
 {
@@ -456,15 +498,26 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
               int max_iter, bool use_graph, cudaStream_t s, int sm_count, StageState& out,
               double* traj_J_host, double* traj_shift_host, kmeans2_profile* prof,
               const char* name = "kmeans2 stage", double* traj_c_host = nullptr,
-              int64_t* traj_n_host = nullptr, bool probe16 = false)
+              int64_t* traj_n_host = nullptr, bool probe16 = false, double* publish = nullptr,
+              bool* published = nullptr)
 {
     NvtxRange stage_range(name);
     KM2_TRY(launch_stage_begin(w.c, w.acc, w.st, tol, max_iter, s));
     KM2_TRY(launch_qsum(X, n, d, w.st, s, sm_count));
     KM2_TRY(prepare_stage_points(X, n, d, w, *w.ws, s));
-    bool finished = false;
+    bool finished = false, have_out = false;
     int remaining = max_iter;
-    if (probe16 && w.form == KMEANS2_PRECISION_FP16) {
+    if (w.form == KMEANS2_PRECISION_FP32 && !prof &&
+        (max_iter == 1 || (double)n * w.c.k * d <= kQueuedWork)) {
+        KM2_TRY(run_loop_queued(X, n, d, w, labels, max_iter, s, sm_count, out, publish));
+        finished = have_out = true;
+        if (published) *published = publish != nullptr;
+    } else if (max_iter == 1 && !prof && !use_graph) {
+        // one iteration: its end is read with the final state
+        KM2_TRY(launch_iteration(X, n, d, w, labels, 0ull, 0, 0, s, sm_count));
+        finished = true;
+    }
+    if (!finished && probe16 && w.form == KMEANS2_PRECISION_FP16) {
         // one FP16 iteration from the host; if its single pass left too many
         // rows undecided, the rest of the stage runs the split form (every
         // form decides each row exactly, so the switch changes no result)
@@ -485,8 +538,10 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
         else
             KM2_TRY(run_loop_host(X, n, d, w, labels, remaining, s, sm_count, prof));
     }
-    KM2_CUDA(cudaMemcpyAsync(&out, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
-    KM2_CUDA(cudaStreamSynchronize(s));
+    if (!have_out) {
+        KM2_CUDA(cudaMemcpyAsync(&out, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
+        KM2_CUDA(cudaStreamSynchronize(s));
+    }
     if (out.error) return map_stage_error(out.error);
     if (traj_J_host && out.iter > 0)
         KM2_CUDA(cudaMemcpyAsync(traj_J_host, w.traj_J, sizeof(double) * out.iter,
@@ -501,7 +556,7 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
     if (traj_n_host && w.traj_n && out.iter > 0)
         KM2_CUDA(cudaMemcpyAsync(traj_n_host, w.traj_n, sizeof(int64_t) * (size_t)out.iter * w.c.k,
                                  cudaMemcpyDeviceToHost, s));
-    KM2_CUDA(cudaStreamSynchronize(s));
+    if (traj_J_host || traj_shift_host || traj_c_host || traj_n_host) KM2_CUDA(cudaStreamSynchronize(s));
     return KMEANS2_OK;
 }
 
@@ -768,16 +823,19 @@ int kmeans_step(const float* X, int64_t n, int32_t d, int32_t k, const double* c
     KM2_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StageState), s));
     KM2_TRY(launch_maxabs(Xd, n, d, w.st, s, ws.sm_count));
     StageState out;
+    const bool cen_dev = is_device_ptr(centers_out);
+    bool published = false;
     KM2_TRY(run_stage(Xd, n, d, w, labels, 0.0, 1, false, s, ws.sm_count, out, nullptr, nullptr,
-                      r.opt.profile));
-    KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
-                             is_device_ptr(centers_out) ? cudaMemcpyDeviceToDevice
-                                                        : cudaMemcpyDeviceToHost, s));
+                      r.opt.profile, "kmeans2 step", nullptr, nullptr, false,
+                      cen_dev ? centers_out : nullptr, &published));
+    if (!published)
+        KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
+                                 cen_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     if (!lab_dev)
         KM2_CUDA(cudaMemcpyAsync(labels_out, labels, sizeof(int) * (size_t)n,
                                  is_device_ptr(labels_out) ? cudaMemcpyDeviceToDevice
                                                            : cudaMemcpyDeviceToHost, s));
-    KM2_CUDA(cudaStreamSynchronize(s));
+    if (!published || !lab_dev) KM2_CUDA(cudaStreamSynchronize(s));
     if (J_out) *J_out = out.J;
     if (shift_out) *shift_out = out.shift;
     if (empty_out) *empty_out = out.empty;
@@ -826,10 +884,7 @@ int kmeans_step_noalloc(const float* X, int64_t n, int32_t d, int32_t k,
     KM2_TRY(launch_maxabs(X, n, d, w.st, s, ws.sm_count));
     StageState out;
     KM2_TRY(run_stage(X, n, d, w, labels_out, 0.0, 1, false, s, ws.sm_count, out, nullptr,
-                      nullptr, nullptr));
-    KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
-                             cudaMemcpyDeviceToDevice, s));
-    KM2_CUDA(cudaStreamSynchronize(s));
+                      nullptr, nullptr, "kmeans2 step", nullptr, nullptr, false, centers_out));
     if (J_out) *J_out = out.J;
     if (shift_out) *shift_out = out.shift;
     if (empty_out) *empty_out = out.empty;
@@ -896,10 +951,17 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
         long long* pos = nullptr;
         float* Xs = nullptr;
         int* labels_s = nullptr;
-        KM2_TRY(ws.alloc((void**)&subset, sizeof(long long) * (size_t)m, s));
-        KM2_TRY(ws.alloc((void**)&pos, sizeof(long long) * (size_t)k, s));
-        KM2_TRY(ws.alloc((void**)&Xs, sizeof(float) * (size_t)m * d, s));
-        KM2_TRY(ws.alloc((void**)&labels_s, sizeof(int) * (size_t)m, s));
+        auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+        unsigned char* base = nullptr;
+        KM2_TRY(ws.alloc((void**)&base, up(sizeof(float) * (size_t)m * d) + up(sizeof(long long) * (size_t)m) +
+                                            up(sizeof(long long) * (size_t)k) + sizeof(int) * (size_t)m, s));
+        Xs = (float*)base;
+        base += up(sizeof(float) * (size_t)m * d);
+        subset = (long long*)base;
+        base += up(sizeof(long long) * (size_t)m);
+        pos = (long long*)base;
+        base += up(sizeof(long long) * (size_t)k);
+        labels_s = (int*)base;
         KM2_TRY(sample_device(n, k, m, seed, subset, pos, s, ws));
         KM2_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StageState), s));
         KM2_TRY(launch_gather(Xd, d, subset, m, Xs, w.st, s, ws.sm_count));
@@ -923,9 +985,12 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
     KM2_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StageState), s));
     KM2_TRY(launch_maxabs(Xd, n, d, w.st, s, ws.sm_count));
     StageState ss;
+    const bool cen_dev = is_device_ptr(centers_out);
+    bool published = false;
     KM2_TRY(run_stage(Xd, n, d, w, labels, tol, max_iter, use_graph, s, ws.sm_count, ss,
                       o.traj_J_slow, o.traj_shift_slow, o.profile, "kmeans2 slow stage",
-                      o.traj_centers_slow, o.traj_counts_slow));
+                      o.traj_centers_slow, o.traj_counts_slow, false,
+                      cen_dev ? centers_out : nullptr, &published));
     rr.precision_used = w.form;
     rr.iters_slow = ss.iter;
     rr.converged_slow = ss.converged;
@@ -936,14 +1001,14 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
     rr.undecided_slow = ss.undecided16_total;
     rr.distance_evals = (int64_t)rr.iters_fast * m * k + (int64_t)rr.iters_slow * n * k;
 
-    KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
-                             is_device_ptr(centers_out) ? cudaMemcpyDeviceToDevice
-                                                        : cudaMemcpyDeviceToHost, s));
+    if (!published)
+        KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
+                                 cen_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     if (!lab_dev)
         KM2_CUDA(cudaMemcpyAsync(labels_out, labels, sizeof(int) * (size_t)n,
                                  is_device_ptr(labels_out) ? cudaMemcpyDeviceToDevice
                                                            : cudaMemcpyDeviceToHost, s));
-    KM2_CUDA(cudaStreamSynchronize(s));
+    if (!published || !lab_dev) KM2_CUDA(cudaStreamSynchronize(s));
     rr.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (res) *res = rr;
     if (o.profile) o.profile->kernel_launches += g_launches - launches0;
@@ -1167,7 +1232,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
             KM2_TRY(launch_stage_recheck(Xc, d, w, lab, s, ws.sm_count));
             return launch_recheck_reset(w.st, s);
         }));
-        KM2_TRY(launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, 0ull, 0, s));
+        KM2_TRY(launch_finalize(w.acc, w.c, w.st, w.traj(), w.clus, 0ull, 0, 0, s));
         KM2_CUDA(cudaMemcpyAsync(&ss, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
         KM2_CUDA(cudaStreamSynchronize(s));
         if (ss.error) return map_stage_error(ss.error);

@@ -104,9 +104,14 @@ inline long long center_norm_len(int k, int kpad)
 // Loop state, scales, zero sums, the centers' copies (st zeroed, max |x| recorded).
 int launch_stage_begin(const Centers& c, const Accum& acc, StageState* st, double tol,
                        int max_iter, cudaStream_t s);
-// clus: kClusSlots*k 8-byte words of scratch; tr: the stage's optional per-iteration records.
+// clus: kClusSlots*k 8-byte words of scratch; tr: the stage's optional per-iteration
+// records; stop: once the stage is done, set kErrStopped for the passes queued behind.
 int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const TrajDev& tr,
-                    double* clus, unsigned long long cond_handle, int use_cond, cudaStream_t s);
+                    double* clus, unsigned long long cond_handle, int use_cond, int stop,
+                    cudaStream_t s);
+// The stage's centers (count doubles) to a device buffer, unless the stage failed.
+int launch_publish_centers(const StageState* st, const double* c64, long long count, double* out,
+                           cudaStream_t s);
 int launch_recheck(const float* X, int d, const Centers& c, int* labels, const int* list,
                    StageState* st, const Accum& acc, int settles, cudaStream_t s, int sm_count);
 // Folds this pass's recheck count into the stage total and empties the list

@@ -37,6 +37,7 @@
 
 #include "api_internal.h"
 #include "mma_dev.cuh"
+#include "select_dev.cuh"
 #include "stage_dev.cuh"
 
 namespace km2 {
@@ -87,95 +88,10 @@ __device__ __forceinline__ unsigned int abs_bits(float v)
 
 // ---------------------------------------------------------------- sampling
 
-constexpr int kSampleThreads = 1024;
-
-// Block-level exact radix select: ascending positions (relative to `off`) of
-// the `want` smallest keys splitmix64_at(seed, off + i), i in [0, count).
-__device__ void select_block(unsigned long long seed, unsigned long long off, long long count,
-                             long long want, long long* out)
-{
-    __shared__ unsigned int hist[256];
-    __shared__ unsigned long long prefix;
-    __shared__ long long need;
-    __shared__ long long scan[kSampleThreads];
-    if (threadIdx.x == 0) { prefix = 0; need = want; }
-    __syncthreads();
-    for (int pass = 0; pass < 8; ++pass) {
-        const int shift = 56 - 8 * pass;
-        for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
-        __syncthreads();
-        const unsigned long long pf = prefix;
-        for (long long i = threadIdx.x; i < count; i += blockDim.x) {
-            const unsigned long long key = splitmix64_at(seed, off + (unsigned long long)i);
-            const bool match = pass == 0 || (key >> (shift + 8)) == (pf >> (shift + 8));
-            if (match) atomicAdd(&hist[(key >> shift) & 255ull], 1u);
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            // eight bins per lane: the lane whose range holds the need-th key
-            const long long nd = need;
-            const int lane = threadIdx.x;
-            long long sum = 0;
-            for (int b = 0; b < 8; ++b) sum += hist[8 * lane + b];
-            long long incl = sum;
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            long long acc = incl - sum;
-            if (nd > acc && nd <= incl) {
-                int b = 8 * lane;
-                while (nd > acc + (long long)hist[b]) acc += hist[b++];
-                prefix = pf | ((unsigned long long)b << shift);
-                need = nd - acc;
-            }
-        }
-        __syncthreads();
-    }
-    const unsigned long long T = prefix;     // the want-th smallest key (keys are distinct)
-    const long long per = (count + blockDim.x - 1) / blockDim.x;
-    const long long i0 = min(count, (long long)threadIdx.x * per), i1 = min(count, i0 + per);
-    long long c = 0;
-    for (long long i = i0; i < i1; ++i) c += splitmix64_at(seed, off + (unsigned long long)i) <= T;
-    scan[threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        // exclusive scan, 32 threads' counts per lane
-        long long sum = 0;
-        for (int t = 0; t < kSampleThreads / 32; ++t) sum += scan[threadIdx.x * (kSampleThreads / 32) + t];
-        long long a = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long v = __shfl_up_sync(0xffffffffu, a, o);
-            if ((int)threadIdx.x >= o) a += v;
-        }
-        a -= sum;
-        for (int t = 0; t < kSampleThreads / 32; ++t) {
-            const int e = threadIdx.x * (kSampleThreads / 32) + t;
-            const long long v = scan[e];
-            scan[e] = a;
-            a += v;
-        }
-    }
-    __syncthreads();
-    long long o = scan[threadIdx.x];
-    for (long long i = i0; i < i1; ++i)
-        if (splitmix64_at(seed, off + (unsigned long long)i) <= T) out[o++] = i;
-    __syncthreads();
-}
-
 __global__ void __launch_bounds__(kSampleThreads) batch_sample_kernel(BatchInst* insts)
 {
     BatchInst* I = insts + blockIdx.x;
-    select_block(I->seed, 0ull, I->n, I->m, I->subset);
-    select_block(I->seed, (unsigned long long)I->n, I->m, I->k, I->seltmp);
-    // initial centers: the k selected positions in increasing key order
-    for (int a = threadIdx.x; a < I->k; a += blockDim.x) {
-        const unsigned long long ka = splitmix64_at(I->seed, (unsigned long long)(I->n + I->seltmp[a]));
-        int rank = 0;
-        for (int b = 0; b < I->k; ++b)
-            rank += splitmix64_at(I->seed, (unsigned long long)(I->n + I->seltmp[b])) < ka;
-        I->pos[rank] = I->seltmp[a];
-    }
+    sample_block(I->seed, I->n, I->m, I->k, I->subset, I->pos, I->seltmp);
 }
 
 // Gather X_s, its max |x|, the initial centers, and max |x| over X: gridDim.y CTAs

@@ -66,6 +66,9 @@ constexpr int kErrNonFinite = 1;
 constexpr int kErrRange = 2;       // max|x| >= 2^50
 constexpr int kErrTimeout = 3;     // a bounded device-side wait gave up
 constexpr int kErrBounds = 4;      // a debug-build index check failed (KM2_DEBUG_CHECKS)
+// not an error: the stage is done and the passes already queued behind it return
+// at once, as after an error (the host clears it)
+constexpr int kErrStopped = 5;
 
 // Debug builds (-DKM2_DEBUG_CHECKS) check every decided label, and every old
 // label read back in delta mode (-1 = none), against [0, k) before it

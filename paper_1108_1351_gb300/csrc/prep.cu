@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(256) stage_begin_kernel(Centers c, Accum acc, 
 // 27 us.
 __global__ void __launch_bounds__(256) finalize_kernel(Accum acc, Centers c, StageState* st,
                                                        TrajDev tr, double* clus,
-                                                       unsigned long long handle, int use_cond)
+                                                       unsigned long long handle, int use_cond,
+                                                       int stop)
 {
     __shared__ FinalizeSmem sm;
     __shared__ int last;
@@ -229,7 +230,20 @@ __global__ void __launch_bounds__(256) finalize_kernel(Accum acc, Centers c, Sta
         __syncthreads();
     }
     finalize_reduce_block(c.k, acc.cnt, st, tr, clus, sm);
-    if (threadIdx.x == 0 && use_cond) cudaGraphSetConditional(handle, st->done ? 0u : 1u);
+    if (threadIdx.x == 0) {
+        if (use_cond) cudaGraphSetConditional(handle, st->done ? 0u : 1u);
+        if (stop && st->done) st->error = kErrStopped;
+    }
+}
+
+// The stage's centers to a caller's device buffer, unless it failed.
+__global__ void publish_centers_kernel(const StageState* st, const double* __restrict__ c64,
+                                       long long count, double* __restrict__ out)
+{
+    if (st->error != 0 && st->error != kErrStopped) return;
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < count;
+         e += (long long)gridDim.x * blockDim.x)
+        out[e] = c64[e];
 }
 
 constexpr int kRecheckThreads = 256;
@@ -342,13 +356,23 @@ int launch_stage_begin(const Centers& c, const Accum& acc, StageState* st, doubl
 }
 
 int launch_finalize(const Accum& acc, const Centers& c, StageState* st, const TrajDev& tr,
-                    double* clus, unsigned long long cond_handle, int use_cond, cudaStream_t s)
+                    double* clus, unsigned long long cond_handle, int use_cond, int stop,
+                    cudaStream_t s)
 {
     ++g_launches;
     // one CTA for a handful of centers (no hand-over to a last CTA), else one
     // center per CTA up to about one CTA per SM
     finalize_kernel<<<c.k <= 8 ? 1 : std::min(c.k, 152), 256, 0, s>>>(acc, c, st, tr, clus,
-                                                                     cond_handle, use_cond);
+                                                                     cond_handle, use_cond, stop);
+    KM2_CUDA(cudaGetLastError());
+    return KMEANS2_OK;
+}
+
+int launch_publish_centers(const StageState* st, const double* c64, long long count, double* out,
+                           cudaStream_t s)
+{
+    ++g_launches;
+    publish_centers_kernel<<<(int)std::min(152ll, (count + 255) / 256), 256, 0, s>>>(st, c64, count, out);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }

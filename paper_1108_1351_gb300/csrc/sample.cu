@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "api_internal.h"
+#include "select_dev.cuh"
 
 namespace km2 {
 
@@ -55,27 +56,44 @@ __global__ void hist_top(unsigned long long seed, unsigned long long offset, lon
         if (h[b]) atomicAdd(&ghist[b], h[b]);
 }
 
+// Exclusive prefix sum over the block's threads (a multiple of 32, at most 1024);
+// *total: the sum of all.  ws: 32 words of shared memory.
+__device__ __forceinline__ long long block_exclusive(long long v, long long* ws, long long* total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    long long incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) ws[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const long long own = lane < nw ? ws[lane] : 0;
+        long long w = own;
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        ws[lane] = w - own;
+        if (lane == 31) *total = w;
+    }
+    __syncthreads();
+    return ws[warp] + incl - v;
+}
+
 // Single CTA: find the bucket of the need-th key in st->hist, fix its digit.
 // `shift` is the bit position of the digit's least significant bit.
 __global__ void find_bucket(SelectState* st, int shift, int width)
 {
-    __shared__ unsigned int part[kThreads];
-    __shared__ long long base[kThreads + 1];
+    __shared__ long long ws[32], total;
     int nb = 1 << width;
     int per = (nb + kThreads - 1) / kThreads;
     unsigned int s = 0;
     for (int b = threadIdx.x * per; b < min(nb, (int)(threadIdx.x + 1) * per); ++b) s += st->hist[b];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long acc = 0;
-        for (int t = 0; t < kThreads; ++t) { base[t] = acc; acc += part[t]; }
-        base[kThreads] = acc;
-    }
-    __syncthreads();
-    long long need = st->need;
-    long long lo = base[threadIdx.x];
-    long long hi = base[threadIdx.x + 1];
+    const long long need = st->need;
+    const long long lo = block_exclusive((long long)s, ws, &total);
+    const long long hi = lo + s;
     if (need > lo && need <= hi) {
         long long acc = lo;
         for (int b = threadIdx.x * per; b < min(nb, (int)(threadIdx.x + 1) * per); ++b) {
@@ -152,22 +170,15 @@ __global__ void count_sel(unsigned long long seed, unsigned long long offset, lo
     }
 }
 
-// Exclusive scan of chunk counts (single CTA, sequential over thread slices).
+// Exclusive scan of chunk counts (single CTA, thread slices in order).
 __global__ void scan_counts(const unsigned int* counts, long long nchunks, long long* offsets)
 {
-    __shared__ long long part[1024];
+    __shared__ long long ws[32], total;
     long long per = (nchunks + blockDim.x - 1) / blockDim.x;
     long long b0 = threadIdx.x * per, b1 = min(nchunks, b0 + per);
     long long s = 0;
     for (long long c = b0; c < b1; ++c) s += counts[c];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long acc = 0;
-        for (int t = 0; t < (int)blockDim.x; ++t) { long long v = part[t]; part[t] = acc; acc += v; }
-    }
-    __syncthreads();
-    long long acc = part[threadIdx.x];
+    long long acc = block_exclusive(s, ws, &total);
     for (long long c = b0; c < b1; ++c) { offsets[c] = acc; acc += counts[c]; }
 }
 
@@ -216,6 +227,20 @@ __global__ void order_by_key(unsigned long long seed, unsigned long long offset,
         out[rank] = sel[a];
     }
 }
+
+// Both draws of a small problem in one launch.
+__global__ void __launch_bounds__(kSampleThreads) sample_small_kernel(unsigned long long seed,
+                                                                      long long n, long long m, int k,
+                                                                      long long* subset,
+                                                                      long long* pos, long long* tmp)
+{
+    sample_block(seed, n, m, k, subset, pos, tmp);
+}
+
+// Rows up to which one CTA draws: its nine passes over the keys take 25 us at n =
+// 20,000 and grow with n; the 35 launches and the read-back of the other way take
+// about 250 us however small n is.
+constexpr long long kSampleSmall = 1 << 17;
 
 }  // namespace
 
@@ -290,9 +315,15 @@ static int select_smallest(unsigned long long seed, unsigned long long offset, l
 int sample_device(long long n, int k, long long m, unsigned long long seed, long long* subset,
                   long long* init_pos, cudaStream_t s, DeviceScratch& ws)
 {
-    KM2_TRY(select_smallest(seed, 0ull, n, m, subset, s, ws));
     long long* sel = nullptr;
     KM2_TRY(ws.alloc((void**)&sel, sizeof(long long) * (size_t)k, s));
+    if (n <= kSampleSmall) {
+        ++g_launches;
+        sample_small_kernel<<<1, kSampleThreads, 0, s>>>(seed, n, m, k, subset, init_pos, sel);
+        KM2_CUDA(cudaGetLastError());
+        return KMEANS2_OK;
+    }
+    KM2_TRY(select_smallest(seed, 0ull, n, m, subset, s, ws));
     KM2_TRY(select_smallest(seed, (unsigned long long)n, m, k, sel, s, ws));
     int grid = (k + kThreads - 1) / kThreads;
     ++g_launches;

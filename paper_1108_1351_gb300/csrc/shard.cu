@@ -291,7 +291,7 @@ int resume_iter(kmeans2_shard* sh, kmeans2_exchange* next)
                                                                  sh->w.st);
     KM2_CUDA(cudaGetLastError());
     KM2_TRY(launch_finalize(sh->tot, sh->w.c, sh->w.st, sh->w.traj(),
-                            sh->w.clus, 0ull, 0, s));
+                            sh->w.clus, 0ull, 0, 0, s));
     StageState st;
     KM2_CUDA(cudaMemcpyAsync(&st, sh->w.st, sizeof(st), cudaMemcpyDeviceToHost, s));
     KM2_CUDA(cudaStreamSynchronize(s));
