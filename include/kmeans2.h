@@ -217,7 +217,8 @@ KMEANS2_API int kmeans2_fit(const float* X, int64_t n, int32_t d, int32_t k, dou
  * and copied to the device once (the fast stage runs resident); every
  * iteration of the slow stage streams X through the device in chunks of
  * chunk_points rows (two device buffers, copies on a second stream
- * overlapping the distance kernel of the previous chunk), with the near-tie
+ * overlapping the distance kernel of the previous chunk; the two chunks that
+ * the last pass left in the buffers are not copied again), with the near-tie
  * recheck of each chunk done while it is resident and the exact integer
  * cluster sums accumulated across chunks.  The device holds the labels (n
  * int32, unless labels_out is device memory), two chunks, S_s and the

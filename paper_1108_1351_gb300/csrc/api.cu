@@ -1045,7 +1045,12 @@ namespace {
 constexpr long long kDefaultChunkPoints = 1ll << 26;
 
 // Host-resident X streamed through two device chunk buffers: copies run on a
-// stream of their own and overlap the kernels of the previous chunk.
+// stream of their own and overlap the kernels of the previous chunk.  Passes go
+// over the chunks forward and backward in turn, so a pass starts with the two
+// chunks that the last one left in the buffers and copies only the others: X of
+// one or two chunks crosses the link once per fit (n = 1e7, d = 8, 50 iterations:
+// 51 copies of 0.32 GB, 77 ms at the link's 211 GB/s, became one).  The integer
+// sums do not depend on the order of the chunks.
 struct ChunkStreamer {
     const float* X = nullptr;
     long long n = 0, chunk = 0, nchunks = 0;
@@ -1053,6 +1058,8 @@ struct ChunkStreamer {
     float* buf[2] = {nullptr, nullptr};
     cudaStream_t copy = nullptr;
     cudaEvent_t copied[2] = {nullptr, nullptr}, used[2] = {nullptr, nullptr};
+    long long held[2] = {-1, -1};       // the chunk in each buffer
+    bool backward = false;              // direction of the next pass
 
     long long rows(long long c) const { return c + 1 < nchunks ? chunk : n - c * chunk; }
 
@@ -1074,10 +1081,13 @@ struct ChunkStreamer {
         }
         return KMEANS2_OK;
     }
-    // Copy chunk c into buffer c % 2 once the kernels that read it last are done.
+    // Copy chunk c into buffer c % 2, unless it is there, once the kernels that read
+    // it last are done.
     int fetch(long long c)
     {
         const int b = (int)(c & 1);
+        if (held[b] == c) return KMEANS2_OK;
+        held[b] = c;
         KM2_CUDA(cudaStreamWaitEvent(copy, used[b], 0));
         KM2_CUDA(cudaMemcpyAsync(buf[b], X + (size_t)(c * chunk) * d, (size_t)rows(c) * d * sizeof(float),
                                  cudaMemcpyHostToDevice, copy));
@@ -1100,9 +1110,11 @@ struct ChunkStreamer {
 template <class Fn>
 int stream_pass(ChunkStreamer& cs, cudaStream_t s, Fn&& on_chunk)
 {
-    KM2_TRY(cs.fetch(0));
-    for (long long c = 0; c < cs.nchunks; ++c) {
-        if (c + 1 < cs.nchunks) KM2_TRY(cs.fetch(c + 1));
+    const long long first = cs.backward ? cs.nchunks - 1 : 0, step = cs.backward ? -1 : 1;
+    cs.backward = !cs.backward;
+    KM2_TRY(cs.fetch(first));
+    for (long long i = 0, c = first; i < cs.nchunks; ++i, c += step) {
+        if (i + 1 < cs.nchunks) KM2_TRY(cs.fetch(c + step));
         const int b = (int)(c & 1);
         KM2_CUDA(cudaStreamWaitEvent(s, cs.copied[b], 0));
         KM2_TRY(on_chunk(c, cs.buf[b], cs.rows(c)));

@@ -72,3 +72,17 @@ def test_recheck_forms(d, k):
     X = np.concatenate([C[rng.integers(0, k, 600)], 0.5 * (C[0] + C[rng.integers(0, k, 600)])])
     X = (X + 1e-3 * rng.normal(size=X.shape) * (rng.random((X.shape[0], 1)) < 0.5)).astype(np.float32)
     _check(X, np.ascontiguousarray(C))
+
+
+@pytest.mark.parametrize("chunk", [0, 4_000, 2_001, 1_999, 700, 1_000_000])
+def test_streamed_chunk_orders(chunk):
+    """One, two, odd and even chunk counts, ragged last chunks: passes alternate
+    their direction and reuse the chunks still in the buffers."""
+    from paper_1108_1351_gb300 import synth
+    X = synth.aniso_gaussian_noise(4_001, 8, 12, 4).numpy()
+    o = oracle.fit(X, 12, 0.1, 3, 1e-6, 40)
+    s = km.fit_streamed(X, 12, 0.1, 3, 1e-6, 40, chunk)
+    r = km.fit(torch.as_tensor(X, device="cuda"), 12, 0.1, 3, 1e-6, 40)
+    assert np.array_equal(to_np(s.labels), o["labels"])
+    assert np.array_equal(to_np(s.centers), to_np(r.centers)) and s.J == r.J
+    assert (s.iters_fast, s.iters_slow) == (o["iters_fast"], o["iters_slow"])
