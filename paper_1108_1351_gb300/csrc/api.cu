@@ -201,6 +201,7 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
     // one allocation, carved in 256-byte steps: a pool allocation and its release
     // cost the host 2 us, a dozen of them a fifth of a small step
     const size_t kd = (size_t)k * d;
+    w.mv.cap = tc16_form(w.form) && k <= kMovedMaxK ? (unsigned)std::min(list_cap, kMovedCap) : 0u;
     struct Piece { void** p; size_t bytes; };
     const Piece pieces[] = {
         {(void**)&w.c.c64, kd * sizeof(double)},
@@ -217,6 +218,10 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
         {(void**)&w.traj_shift, (size_t)max_iter * sizeof(double)},
         // (the split layout: a fit may switch from FP16 to split BF16 between stages)
         {(void**)&w.cb, tc16_form(w.form) ? bf16_cb_bytes(d, k, 0) : 0},
+        {(void**)&w.mv.moved, (size_t)w.mv.cap * sizeof(int2)},
+        {(void**)&w.mv.sorted, (size_t)w.mv.cap * 2 * sizeof(int2)},
+        {(void**)&w.mv.hist, w.mv.cap ? (size_t)k * 4 * sizeof(unsigned) : 0},
+        {(void**)&w.mv.state, w.mv.cap ? 2 * sizeof(unsigned) : 0},
     };
     size_t total = 0;
     for (const Piece& q : pieces) total += (q.bytes + 255) / 256 * 256;
@@ -226,6 +231,11 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
         if (q.bytes == 0) continue;
         *q.p = base;
         base += (q.bytes + 255) / 256 * 256;
+    }
+    if (w.mv.cap) {
+        w.mv.cur = w.mv.hist + 2 * (size_t)k;
+        KM2_CUDA(cudaMemsetAsync(w.mv.hist, 0, (size_t)k * 4 * sizeof(unsigned), s));
+        KM2_CUDA(cudaMemsetAsync(w.mv.state, 0, 2 * sizeof(unsigned), s));
     }
     return KMEANS2_OK;
 }
@@ -277,12 +287,16 @@ int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels,
         return launch_assign_tc32(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
     if (w.form == KMEANS2_PRECISION_FP16) {
         KM2_TRY(launch_assign_bf16(X, w.xt, w.xn2, w.cb, n, d, w.c, labels, w.st, w.acc, w.list,
-                                   1, s, sm_count));
+                                   1, w.mv, s, sm_count));
+        // before the second pass, which changes labels of listed rows of its own
+        KM2_TRY(launch_moved_sums(X, n, d, w.mv, w.c.k, labels, w.st, w.acc, s, sm_count));
         return launch_stage_b(X, d, w.c, labels, w.st, w.acc, w.list, w.sb, s, sm_count);
     }
-    if (tc16_form(w.form))
-        return launch_assign_bf16(X, w.xt, w.xn2, w.cb, n, d, w.c, labels, w.st, w.acc, w.list,
-                                  0, s, sm_count);
+    if (tc16_form(w.form)) {
+        KM2_TRY(launch_assign_bf16(X, w.xt, w.xn2, w.cb, n, d, w.c, labels, w.st, w.acc, w.list,
+                                   0, w.mv, s, sm_count));
+        return launch_moved_sums(X, n, d, w.mv, w.c.k, labels, w.st, w.acc, s, sm_count);
+    }
     if (screened(X, d, w))
         return launch_assign_mma(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
     return launch_assign_fp32(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
@@ -706,7 +720,13 @@ uint64_t kmeans2_fit_footprint(int64_t n, int32_t d, int32_t k, double subset_fr
     add(N * 4);
     add((unsigned long long)kClusSlots * K * 8);
     add(2 * (unsigned long long)max_iter * 8);
-    if (tc16_form(form)) add(bf16_cb_bytes(d, k, 0));
+    if (tc16_form(form)) {
+        add(bf16_cb_bytes(d, k, 0));
+        if (k <= kMovedMaxK) {       // moved rows, sorted
+            add(std::min<unsigned long long>(N, kMovedCap) * 24);
+            add(K * 16 + 512);
+        }
+    }
     if (labels_on_host) add(N * 4);
     // fast stage: S_s indices, init positions, X_s, its labels
     add(m * 8);

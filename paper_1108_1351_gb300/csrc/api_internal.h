@@ -124,6 +124,23 @@ int launch_assign_tc32(const float* X, long long n, int d, const Centers& c, int
                        StageState* st, const Accum& acc, int* list, cudaStream_t s,
                        int sm_count);
 
+// moved.cu: rows whose label a pass changed, listed by the 16-bit distance kernels
+// and added to the sums by cluster afterwards.  The list holds at most kMovedCap
+// rows (100 MB of scratch); the distance kernel itself adds those past it, and all
+// of them where k is above kMovedMaxK (moved null).
+constexpr long long kMovedCap = 1ll << 22;
+constexpr int kMovedMaxK = 4096;
+struct MovedRows {
+    unsigned cap = 0;
+    int2* moved = nullptr;       // cap: row, label before (-1: none)
+    int2* sorted = nullptr;      // 2 cap: row, bin (cluster joined, or k + cluster left)
+    unsigned* hist = nullptr;    // 2 k: entries per bin; zero between passes
+    unsigned* cur = nullptr;     // 2 k: entries placed; zero between passes
+    unsigned* state = nullptr;   // list length (zero between passes), sorted entries
+};
+int launch_moved_sums(const float* X, long long n, int d, const MovedRows& mv, int k, const int* labels,
+                      const StageState* st, const Accum& acc, cudaStream_t s, int sm_count);
+
 // assign_bf16.cu: tensor-core split-BF16 form, d a multiple of 16 in [16, 128]
 int assign_bf16_supported(int d, int k, const float* X);
 // single = 1: the single-pass FP16 variant (one operand part, scaled by powers
@@ -134,8 +151,9 @@ int launch_convert_x_bf16(const float* X, long long n, int d, unsigned char* Xt,
                           const StageState* st, int single, cudaStream_t s, int sm_count);
 int launch_assign_bf16(const float* X, const unsigned char* Xt, const float* xn2,
                        unsigned char* Cb, long long n, int d, const Centers& c, int* labels,
-                       StageState* st, const Accum& acc, int* list, int single, cudaStream_t s,
-                       int sm_count, const long long* n_dev = nullptr);
+                       StageState* st, const Accum& acc, int* list, int single,
+                       const MovedRows& mv, cudaStream_t s, int sm_count,
+                       const long long* n_dev = nullptr);
 // Second pass of the single-pass FP16 form: buffers for up to `cap` rows that
 // its bound could not decide, re-run through the split-BF16 kernel.
 struct StageB {
@@ -192,6 +210,7 @@ struct Workspace {
     float* xn2 = nullptr;
     unsigned char* cb = nullptr;
     StageB sb{};                   // FP16 form: its second pass
+    MovedRows mv{};                // rows moved by the pass
 };
 
 int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, int d,

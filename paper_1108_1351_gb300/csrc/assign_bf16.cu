@@ -105,6 +105,7 @@ struct Bf16Args {
     float kappa, kpack;
     float kabs;              // single-pass form: coefficient of the bound's absolute term
     int ctries;              // wait limit of the consumer roles (MMA issuer, epilogue)
+    MovedRows mv;            // where its list is set, moved rows go there (moved.cu)
 };
 
 // Scales of the single-pass FP16 operands: x as x 2^-a with a = E - 14, where
@@ -521,8 +522,23 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
                 old = (lab_bulk && in_ring) ? side.lab[r][row] : labels[p];
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.side_empty[r]);
-            const bool moved = valid && !flag && label_ok(BI, a.k, st) && old_label_ok(old, a.k, st) &&
+            bool moved = valid && !flag && label_ok(BI, a.k, st) && old_label_ok(old, a.k, st) &&
                                BI != old;
+            if (a.mv.moved) {
+                const unsigned m = __ballot_sync(0xffffffffu, moved);
+                if (m) {
+                    unsigned at = 0;
+                    if (lane == 0) at = atomicAdd(a.mv.state, (unsigned)__popc(m));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & lanemask_lt());
+                    if (moved && at < a.mv.cap) {
+                        a.mv.moved[at] = make_int2((int)p, old);
+                        atomicAdd(a.mv.hist + BI, 1u);
+                        if (old >= 0) atomicAdd(a.mv.hist + a.k + old, 1u);
+                        labels[p] = BI;
+                        moved = false;
+                    }
+                }
+            }
             if (moved) {
                 atomicAdd(acc.cnt + BI, 1ull);
                 if (old >= 0) atomicAdd(acc.cnt + old, ~0ull);
@@ -939,8 +955,8 @@ int launch_convert_x_bf16(const float* X, long long n, int d, unsigned char* Xt,
 
 int launch_assign_bf16(const float* X, const unsigned char* Xt, const float* xn2,
                        unsigned char* Cb, long long n, int d, const Centers& c, int* labels,
-                       StageState* st, const Accum& acc, int* list, int single, cudaStream_t s,
-                       int sm_count, const long long* n_dev)
+                       StageState* st, const Accum& acc, int* list, int single,
+                       const MovedRows& mv, cudaStream_t s, int sm_count, const long long* n_dev)
 {
     const int NC = bf16_chunk(d, c.k, single);
     const int nch = (c.k + NC - 1) / NC;
@@ -1013,6 +1029,7 @@ int launch_assign_bf16(const float* X, const unsigned char* Xt, const float* xn2
     a.kabs = single ? f16_kabs(d) : 0.0f;
     a.kpack = kPackSlack;
     a.ctries = consumer_wait_tries(kWaitTries);
+    a.mv = mv;
     ++g_launches;
     if (single) {
         if (NC == 64)
@@ -1054,8 +1071,9 @@ int launch_stage_b(const float* X, int d, const Centers& c, int* labels, StageSt
     stageb_compact_kernel<<<(int)blocks, 256, 0, s>>>(X, d, list, b.nb, labels, st, b.Xc, b.Xt,
                                                       b.xn2, b.lab);
     KM2_CUDA(cudaGetLastError());
+    // few rows, with labels of their own: their sums are added by the kernel
     KM2_TRY(launch_assign_bf16(b.Xc, b.Xt, b.xn2, b.cb, b.cap, d, c, b.lab, b.st, acc, b.list, 0,
-                               s, sm_count, b.nb));
+                               MovedRows{}, s, sm_count, b.nb));
     long long sb = (b.cap + 255) / 256;
     if (sb > (long long)sm_count * 8) sb = (long long)sm_count * 8;
     stageb_scatter_kernel<<<(int)sb, 256, 0, s>>>(list, b.nb, b.lab, labels, b.list, b.st);

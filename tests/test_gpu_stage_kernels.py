@@ -86,3 +86,36 @@ def test_streamed_chunk_orders(chunk):
     assert np.array_equal(to_np(s.labels), o["labels"])
     assert np.array_equal(to_np(s.centers), to_np(r.centers)) and s.J == r.J
     assert (s.iters_fast, s.iters_slow) == (o["iters_fast"], o["iters_slow"])
+
+
+def _same(a, b):
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and a[2:] == b[2:]
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp16"])
+@pytest.mark.parametrize("n,d,k", [(1, 16, 1), (33, 16, 3), (5003, 48, 4), (20_001, 128, 130),
+                                   (9_000, 32, 4096), (9_000, 32, 4097)])
+def test_moved_row_sums(precision, n, d, k):
+    """First and later passes of the 16-bit forms, whose moved rows are listed and
+    added by cluster: up to the largest k of the list and past it, runs of one
+    cluster and of many, and passes that move few rows or none."""
+    rng = np.random.default_rng(n + k)
+    X = (rng.normal(size=(n, d)) + 4.0 * rng.integers(0, 3, size=(n, 1))).astype(np.float32)
+    C = X[rng.integers(0, n, size=k)].astype(np.float64)
+    C[: k // 2] += 50.0                               # clusters that no row joins
+    Xd = torch.as_tensor(X, device="cuda")
+    Cd = torch.as_tensor(C, device="cuda")
+    _same(km.step(Xd, Cd, precision=precision), km.step(Xd, Cd, precision="fp32"))
+    if k <= n // 8:
+        f = km.fit(Xd, k, 0.3, 1, 1e-7, 60, precision=precision)
+        g = km.fit(Xd, k, 0.3, 1, 1e-7, 60, precision="fp32")
+        assert torch.equal(f.labels, g.labels) and torch.equal(f.centers, g.centers)
+        assert f.J == g.J and f.iters_slow == g.iters_slow
+
+
+def test_moved_rows_past_the_list():
+    """More moved rows than the list holds (2^22): the distance kernel adds the rest."""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.randn(4_500_000, 16, device="cuda", generator=g)
+    C = X[:40].double().contiguous()
+    _same(km.step(X, C, precision="bf16"), km.step(X, C, precision="fp32"))
