@@ -30,7 +30,7 @@
 //           accumulators to the epilogues;
 //   warps 3-6, 7-10  two epilogue groups taking alternate tiles, each with its
 //           own two TMEM accumulators (4 x NC columns in all): a thread owns
-//           one row (TMEM lane) of the tile, keeps a packed-key top-2 across
+//           one row (TMEM lane) of the tile, keeps the best and second-best across
 //           the chunks (the next 32 columns load while the current ones are
 //           compared) and decides the row (near-tie flag, label, exact
 //           fixed-point cluster sums).
@@ -59,11 +59,6 @@ constexpr int kSA = 2;                 // A ring depth (tiles)
 constexpr int kMaxSB = 8;              // B ring depth (slices)
 constexpr int kSmemBudget = 226 * 1024;    // dynamic + static shared memory of the CTA
 constexpr int kWaitTries = 1 << 22;
-
-__device__ __forceinline__ float pack_key(float v, unsigned j)
-{
-    return __uint_as_float((__float_as_uint(v) & ~31u) | j);
-}
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes)
 {
@@ -102,7 +97,7 @@ struct Bf16Args {
     int kps;                 // K-steps per B ring slot
     int lab_bulk;            // old labels can be bulk-copied (16-byte aligned)
     uint32_t tmem_cols;
-    float kappa, kpack;
+    float kappa;
     float kabs;              // single-pass form: coefficient of the bound's absolute term
     int ctries;              // wait limit of the consumer roles (MMA issuer, epilogue)
     MovedRows mv;            // where its list is set, moved rows go there (moved.cu)
@@ -179,44 +174,52 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
     return false;
 }
 
-// Packed-key top-2 of 32 accumulator columns (center indices j0 .. j0 + 31)
-// folded into the running (B1, B2, BI) of a row.  Eight independent chains
-// of two column pairs each keep the dependent path short.
-__device__ __forceinline__ void top2_cols(const uint32_t* r, int j0, float& B1, float& B2, int& BI)
+// What a row keeps of the columns seen so far.
+struct RowBest {
+    float B1;           // smallest key
+    float B2;           // smallest of the other blocks' minima
+    uint32_t near;      // columns of B1's block of 32 within the bound of B1: column c at bit 31 - c
+    int BB;             // B1's block: its first column
+};
+
+// The largest key that may still beat m by the bound thr > 0, rounded up (and
+// above m).
+__device__ __forceinline__ float near_limit(float m, float thr)
 {
-    float q1[8], q2[8];
+    return fmaf(fabsf(m), 0x1p-21f, m + thr);
+}
+
+// 32 accumulator columns (center indices j0 .. j0 + 31) folded into the row.
+// The scan runs on the ALU pipe (2 cycles per instruction), so its instructions
+// count.  The block's minimum takes half a min per column (three operands); then
+// one subtraction (FMA pipe) and one funnel shift collect the signs of
+// key - limit: 1.8 ALU instructions per column.  Keys that carry their index in
+// the low bits and a running top-2 took 4.7 (FP16, n = 1e6, d = 128, k = 1024:
+// a pass 0.47 -> 0.36 ms, the fit 38.0 -> 31.2 ms).
+__device__ __forceinline__ void scan_cols(const uint32_t* r, int j0, float thr, RowBest& w)
+{
+    float m4[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { q1[q] = INFINITY; q2[q] = INFINITY; }
-#pragma unroll
-    for (int j = 0; j < 32; j += 16) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int jj = j + 2 * q;
-            const float k0 = pack_key(__uint_as_float(r[jj]), (unsigned)jj);
-            const float k1 = pack_key(__uint_as_float(r[jj + 1]), (unsigned)jj + 1u);
-            const float lo = fminf(k0, k1), hi = fmaxf(k0, k1);
-            q2[q] = fmin3(q2[q], hi, fmaxf(q1[q], lo));
-            q1[q] = fminf(q1[q], lo);
-        }
+    for (int q = 0; q < 4; ++q) {
+        float a = fmin3(__uint_as_float(r[8 * q]), __uint_as_float(r[8 * q + 1]), __uint_as_float(r[8 * q + 2]));
+        float b = fmin3(__uint_as_float(r[8 * q + 3]), __uint_as_float(r[8 * q + 4]),
+                        __uint_as_float(r[8 * q + 5]));
+        m4[q] = fminf(fmin3(a, __uint_as_float(r[8 * q + 6]), __uint_as_float(r[8 * q + 7])), b);
     }
-    // pairwise merge of the chains: (a1, a2) + (b1, b2) -> (min, second)
+    const float m = fminf(fmin3(m4[0], m4[1], m4[2]), m4[3]);
+    const float lim = near_limit(m, thr);
+    uint32_t s[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int w = 4; w >= 1; w >>= 1) {
+    for (int c = 0; c < 8; ++c)
 #pragma unroll
-        for (int q = 0; q < w; ++q) {
-            const float m = fmin3(q2[q], q2[q + w], fmaxf(q1[q], q1[q + w]));
-            q1[q] = fminf(q1[q], q1[q + w]);
-            q2[q] = m;
-        }
+        for (int q = 0; q < 4; ++q)
+            s[q] = __funnelshift_l(__float_as_uint(__uint_as_float(r[8 * q + c]) - lim), s[q], 1);
+    if (m < w.B1) {
+        w.BB = j0;
+        w.near = __byte_perm(__byte_perm(s[3], s[2], 0x0040), __byte_perm(s[1], s[0], 0x0040), 0x5410);
     }
-    const float b1 = q1[0], b2 = q2[0];
-    if (b1 < B1) {
-        B2 = fminf(B1, b2);
-        B1 = b1;
-        BI = j0 + (int)(__float_as_uint(b1) & 31u);
-    } else {
-        B2 = fminf(B2, b1);
-    }
+    w.B2 = fminf(w.B2, fmaxf(w.B1, m));
+    w.B1 = fminf(w.B1, m);
 }
 
 // SINGLE = 0: split BF16 (two parts per operand, three MMAs per K-step);
@@ -459,8 +462,19 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
         uint32_t phase = 0u;                 // bit s: parity of accumulator 2 g + s's next use
         bool ok = true;
         for (long long i = g; i < cnt && ok; i += kEpiGroups) {
-            float B1 = INFINITY, B2 = INFINITY;
-            int BI = 0;
+            const long long tile = blockIdx.x + i * gridDim.x;
+            const long long p = tile * kRows + row;
+            const bool valid = p < n;
+            const int r = (int)(i % kSR);
+            {
+                const bool w = wait_bar(&bars.side_full[r], (uint32_t)((i / kSR) & 1), abort_v, st, ctries);
+                if (!__all_sync(0xffffffffu, w)) break;
+            }
+            const bool in_ring = (long long)row < ((n - tile * kRows) & ~3ll);
+            const float xx = valid ? (in_ring ? side.xn2[r][row] : __ldg(a.xn2 + p)) : 0.0f;
+            const float thr = (ldexpf(a.kappa * (thr_base + xx) + tabs, kexp) + kabs) * (1.0f + 0x1p-20f) +
+                              0x1p-120f;
+            RowBest rb = {INFINITY, INFINITY, 0u, 0};
             for (int ch = 0; ch < nch; ++ch) {
                 const int b = g * kAccBufs<NC> + ch % kAccBufs<NC>;
                 bool w = wait_bar(&bars.acc_full[b], (phase >> (ch % kAccBufs<NC>)) & 1u, abort_v,
@@ -486,7 +500,7 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
 #pragma unroll
                 for (int i = 0; i < NB; ++i) {
                     if (i + 2 < NB) tc::tmem_ld32_async(cb + (uint32_t)(32 * (i + 2)), rr[(i + 2) % 3]);
-                    top2_cols(rr[i % 3], ch * NC + 32 * i, B1, B2, BI);
+                    scan_cols(rr[i % 3], ch * NC + 32 * i, thr, rb);
                     if (i + 2 < NB) {
                         tc::tmem_wait_ld();
                         if (i + 3 == NB) release();
@@ -495,20 +509,9 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
                 phase ^= 1u << (ch % kAccBufs<NC>);
             }
             if (!ok) break;
-            // ---- decide row `row` of tile i
-            const long long tile = blockIdx.x + i * gridDim.x;
-            const long long p = tile * kRows + row;
-            const bool valid = p < n;
-            const int r = (int)(i % kSR);
-            {
-                const bool w = wait_bar(&bars.side_full[r], (uint32_t)((i / kSR) & 1), abort_v, st, ctries);
-                if (!__all_sync(0xffffffffu, w)) break;
-            }
-            const bool in_ring = (long long)row < ((n - tile * kRows) & ~3ll);
-            const float xx = valid ? (in_ring ? side.xn2[r][row] : __ldg(a.xn2 + p)) : 0.0f;
-            const float thr = ldexpf(a.kappa * (thr_base + xx) + tabs, kexp) + kabs +
-                              a.kpack * (fabsf(B1) + fabsf(B2));
-            const bool flag = valid && (B2 - B1 <= thr);
+            // ---- decide row `row` of tile i: open unless one column is within the bound
+            const int BI = rb.BB + __clz(rb.near);
+            const bool flag = valid && (__popc(rb.near) != 1 || rb.B2 <= near_limit(rb.B1, thr));
             {
                 const unsigned m = __ballot_sync(0xffffffffu, flag);
                 if (m) {
@@ -1027,7 +1030,6 @@ int launch_assign_bf16(const float* X, const unsigned char* Xt, const float* xn2
     a.tmem_cols = cols;
     a.kappa = single ? f16_kappa(d) : bf16_kappa(d);
     a.kabs = single ? f16_kabs(d) : 0.0f;
-    a.kpack = kPackSlack;
     a.ctries = consumer_wait_tries(kWaitTries);
     a.mv = mv;
     ++g_launches;
