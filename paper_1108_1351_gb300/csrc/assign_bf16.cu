@@ -21,11 +21,12 @@
 // Warp-specialised pipeline, one CTA per SM, 11 warps:
 //   warp 0  A producer: one bulk TMA copy per tile into a 2-stage ring;
 //   warp 1  B producer: one bulk TMA copy per ring slot (SB <= 8 slots) of
-//           one (chunk, K-step) slice, five of a chunk in the single pass;
+//           one (chunk, K-step) slice, a whole chunk in the single pass;
 //   warp 2  MMA issuer: tiles go in pairs (one per epilogue group and A
 //           stage); per (pair, chunk) unit and K-step it issues 3 MMAs
 //           (M 128, N NC, K 16) for each tile of the pair into its TMEM
-//           accumulator, so each B slice is read from L2 once for 256 points;
+//           accumulator, so each B slice is read from L2 once for 256 points
+//           (single pass: a chunk for one tile, then for the other);
 //           tcgen05.commit frees each slot and both tiles and hands the
 //           accumulators to the epilogues;
 //   warps 3-6, 7-10  two epilogue groups taking alternate tiles, each with its
@@ -94,7 +95,6 @@ struct Bf16Args {
     const unsigned char* Cb; // BF16 -2c slices
     long long n;
     int d, k, nc, nch, sb;   // chunk width NC, chunk count, B ring depth (slots)
-    int kps;                 // K-steps per B ring slot
     int lab_bulk;            // old labels can be bulk-copied (16-byte aligned)
     uint32_t tmem_cols;
     float kappa;
@@ -148,7 +148,8 @@ static_assert(sizeof(float) * kRows % 16 == 0, "side ring rows must keep 16-byte
 
 // Static shared memory of the kernel (barriers, side ring, recheck queues),
 // rounded up; the dynamic part must fit beside it.
-constexpr int kStaticSmem = 16 * 1024;
+// (14 KB: two whole chunks of 256 centers, d = 128, fit exactly in the single pass)
+constexpr int kStaticSmem = 14 * 1024;
 static_assert(sizeof(Bars) + sizeof(SideRing) + kEpiWarps * kRecheckQ * 4 + 64 <= kStaticSmem,
               "static shared memory estimate too small");
 
@@ -249,14 +250,13 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
     constexpr uint32_t kParts = SINGLE ? 1u : 2u;                // operand parts
     const uint32_t Ahalf = (uint32_t)ksteps * 4096u;             // one part of a tile
     const uint32_t Abytes = kParts * Ahalf;
-    // A slot of the B ring holds kps consecutive (chunk, K-step) slices of one
-    // chunk (contiguous in Cb): one bulk copy and one commit per slot, so the
-    // commits per chunk drop from d/16 + 1 to (d/16 + 1) / kps.  The split
-    // form keeps one slice per slot (a compile-time 1, no extra issuer work).
-    const int kPerSlot = SINGLE ? a.kps : 1;
+    // A slot of the B ring holds one (chunk, K-step) slice in the split form, a
+    // whole chunk (contiguous in Cb) in the single pass: one bulk copy and one
+    // commit per chunk.
+    const int kPerSlot = SINGLE ? kslices : 1;
     const uint32_t Kbytes = (uint32_t)NC * 32u * kParts;         // one (chunk, K-step) slice
     const uint32_t Sbytes = Kbytes * (uint32_t)kPerSlot;         // one slot of the B ring
-    const int kunits = (kslices + kPerSlot - 1) / kPerSlot;      // slots per chunk
+    const int kunits = SINGLE ? 1 : kslices;                     // slots per chunk
     unsigned char* sA = smem;                                    // kSA x Abytes
     unsigned char* sB = smem + kSA * Abytes;                     // SB x Sbytes
     unsigned char* sOnes = sB + (size_t)SB * Sbytes;             // 128 x 16 BF16: [1, 1, 1, 0, ...]
@@ -341,11 +341,10 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
                 if (!wait_bar(&bars.b_empty[slot], (uint32_t)(((q / SB) & 1) ^ 1), abort_v, st))
                     break;
                 const long long unit = q / kunits;
-                const int ch = (int)(unit % nch), ks0 = (int)(q % kunits) * kPerSlot;
-                const uint32_t bytes = Kbytes * (uint32_t)min(kPerSlot, kslices - ks0);
-                mbar_expect_tx(&bars.b_full[slot], bytes);
+                const int ch = (int)(unit % nch), ks0 = (int)(q % kunits);
+                mbar_expect_tx(&bars.b_full[slot], Sbytes);
                 bulk_load(sB + (size_t)slot * Sbytes, a.Cb + ((size_t)ch * kslices + ks0) * Kbytes,
-                          bytes, &bars.b_full[slot]);
+                          Sbytes, &bars.b_full[slot]);
             }
             for (long long r = q > SB ? q - SB : 0; r < q; ++r)
                 tc::mbar_wait(&bars.b_full[r % SB], (uint32_t)((r / SB) & 1), kWaitTries);
@@ -364,6 +363,40 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
             for (long long pr = 0; pr < npairs && ok; ++pr) {
                 const bool two = 2 * pr + 1 < cnt;
                 const uint32_t par = (uint32_t)(pr & 1);
+                if constexpr (SINGLE) {
+                    // tile by tile: the first group compares its accumulator while
+                    // the second tile's MMAs run, and the second group during the
+                    // first tile's next chunk.  (Both tiles per K-step, with
+                    // five K-steps per slot, so that the groups compared at the same
+                    // time and the MMAs waited: n = 1e6, d = 128, k = 1024, a pass
+                    // 0.37 ms, now 0.24.)
+                    for (int ch = 0; ch < nch && ok; ++ch, ++q) {
+                        const int slot = (int)(q % SB);
+                        if (!(ok = wait_bar(&bars.b_full[slot], (uint32_t)((q / SB) & 1), abort_v, st, ctries)))
+                            break;
+                        const uint32_t bh = sBaddr + (uint32_t)slot * Sbytes;
+                        for (int t = 0; t < (two ? 2 : 1); ++t) {
+                            const int b = t * kAccBufs<NC> + ch % kAccBufs<NC>;
+                            if (ch == 0 && !(ok = wait_bar(&bars.a_full[t], par, abort_v, st, ctries))) break;
+                            if (!(ok = wait_bar(&bars.acc_empty[b], ((phase >> b) & 1u) ^ 1u, abort_v, st, ctries)))
+                                break;
+                            tc::fence_after_sync();
+                            const uint32_t dt = tmem + (uint32_t)(b * NC);
+                            const uint32_t ah = sAaddr + (uint32_t)t * Abytes;
+                            for (int ks = 0; ks < ksteps; ++ks)
+                                tc::mma_bf16(dt, tc::smem_desc(ah + (uint32_t)ks * 4096u),
+                                             tc::smem_desc(bh + (uint32_t)ks * Kbytes), idesc16, ks > 0 ? 1u : 0u);
+                            // + ||c||^2: ones x (nh, nm, nl)
+                            tc::mma_bf16(dt, tc::smem_desc(sOnesAddr), tc::smem_desc(bh + (uint32_t)ksteps * Kbytes),
+                                         idesc, 1u);
+                            tc::mma_commit(&bars.acc_full[b]);
+                            phase ^= 1u << b;
+                            if (ch == nch - 1) tc::mma_commit(&bars.a_empty[t]);
+                        }
+                        if (ok) tc::mma_commit(&bars.b_empty[slot]);
+                    }
+                    continue;
+                }
                 if (!(ok = wait_bar(&bars.a_full[0], par, abort_v, st, ctries))) break;
                 if (two && !(ok = wait_bar(&bars.a_full[1], par, abort_v, st, ctries))) break;
                 tc::fence_after_sync();
@@ -379,18 +412,10 @@ assign_bf16(Bf16Args a, Centers c, int* __restrict__ labels, StageState* st, Acc
                         if (!(ok = wait_bar(&bars.b_full[slot], (uint32_t)((q / SB) & 1), abort_v, st, ctries)))
                             break;
                         tc::fence_after_sync();
-                        const int ks0 = u * kPerSlot, ks1 = min(ks0 + kPerSlot, kslices);
-                        for (int ks = ks0; ks < ks1; ++ks) {
-                            const uint32_t bh = sBaddr + (uint32_t)slot * Sbytes + (uint32_t)(ks - ks0) * Kbytes;
-                            if (ks < ksteps && SINGLE) {
-#pragma unroll
-                                for (int t = 0; t < 2; ++t) {
-                                    if (t == 1 && !two) break;
-                                    const uint32_t dt = t ? d1 : d0;
-                                    const uint32_t ah = sAaddr + (uint32_t)t * Abytes + (uint32_t)ks * 4096u;
-                                    tc::mma_bf16(dt, tc::smem_desc(ah), tc::smem_desc(bh), idesc16, ks > 0 ? 1u : 0u);
-                                }
-                            } else if (ks < ksteps) {
+                        const int ks = u;
+                        {
+                            const uint32_t bh = sBaddr + (uint32_t)slot * Sbytes;
+                            if (ks < ksteps) {
                                 const uint32_t bl = bh + (uint32_t)NC * 32u;
 #pragma unroll
                                 for (int t = 0; t < 2; ++t) {
@@ -987,19 +1012,15 @@ int launch_assign_bf16(const float* X, const unsigned char* Xt, const float* xn2
     while (cols < (uint32_t)(kEpiGroups * (NC >= 256 ? 1 : 2) * NC)) cols <<= 1;
     const size_t parts = single ? 1 : 2;
     const size_t abytes = parts * 2 * kRows * d, kbytes = (size_t)NC * 32 * parts;
-    // a B ring slot holds kps K-steps of a chunk: five in the single-pass form
-    // (fewer when the ring would drop below two slots), one in the split form
-    int kps = single ? 5 : 1, sb = 0;
-    for (; kps >= 1; --kps) {
-        sb = (int)((kSmemBudget - kStaticSmem - kSA * abytes - 4096) / (kbytes * kps));
-        if (sb >= 2) break;
-    }
-    if (kps < 1 || sb < 2) {
+    // a B ring slot holds a whole chunk in the single pass (two of the largest fit,
+    // NC = 256 and d = 128), one K-step in the split form
+    const size_t sbytes = kbytes * (single ? d / 16 + 1 : 1);
+    int sb = (int)((kSmemBudget - kStaticSmem - kSA * abytes - 4096) / sbytes);
+    if (sb < 2) {
         set_last_error_text("assign_bf16: shared-memory budget too small for this d");
         return KMEANS2_ERR_UNSUPPORTED;
     }
     if (sb > kMaxSB) sb = kMaxSB;
-    const size_t sbytes = kbytes * kps;
     const size_t smem = kSA * abytes + (size_t)sb * sbytes + 4096;
     // one fixed limit for both instantiations (the static part holds the
     // barriers, the side ring and the recheck queues)
@@ -1025,7 +1046,6 @@ int launch_assign_bf16(const float* X, const unsigned char* Xt, const float* xn2
     a.nc = NC;
     a.nch = nch;
     a.sb = sb;
-    a.kps = kps;
     a.lab_bulk = (reinterpret_cast<uintptr_t>(labels) & 15) == 0 ? 1 : 0;
     a.tmem_cols = cols;
     a.kappa = single ? f16_kappa(d) : bf16_kappa(d);

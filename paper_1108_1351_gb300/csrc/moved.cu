@@ -3,7 +3,7 @@
 // words (4 d 64-bit reductions per moved row) bound the distance kernel by the
 // L2's reduction rate: n = 1e6, d = 128, k = 1024, FP16, first pass 2.47 ms.  The
 // distance kernel therefore lists its moved rows and counts them by cluster
-// (0.47 ms); one kernel here sorts the list (0.08 ms: a counting sort over 2 k
+// (0.24 ms); one kernel here sorts the list (0.08 ms: a counting sort over 2 k
 // bins: joined and left), the next adds each run of sorted rows in registers, with
 // one set of reductions per run and cluster (0.24 ms).  The integer sums do not
 // depend on the order.  Two launches, so that a pass that moves nothing pays
