@@ -266,12 +266,15 @@ def select_loop_ceiling(dev, stream, peak):
     return res
 
 
-def roofline_of(form: str, d: int, k: int, prof, clk, p32=None):
+def roofline_of(form: str, d: int, k: int, prof, clk, p32=None, requested: str = "fp32"):
     """Roofline entry of the distance kernel the fit ran (the dominant kernel):
     algorithmic FLOP = 2 N k d per launch (the cross term only), achieved =
     their sum over the profiled launches / their summed CUDA-event time.  The
     CUDA-core forms are measured against the FP32 FMA peak of this GPU
-    (fp32_peak, when given) with the unit-count figure beside it."""
+    (fp32_peak, when given) with the unit-count figure beside it.  Under AUTO the
+    FP32 form of 8 <= d <= 128 runs the tensor-core screen (assign_mma_ring),
+    which reads X once per pass: below k / 2 flop per byte = the tensor / HBM
+    balance its floor is the copy bandwidth."""
     peaks, src = _peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     achieved = prof.assign_flops / (prof.assign_ms * 1e-3) / 1e12 if prof.assign_ms > 0 else None
@@ -303,6 +306,20 @@ def roofline_of(form: str, d: int, k: int, prof, clk, p32=None):
             peak = derived
             peak_source = (f"derived: {SM_COUNT_GB300} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x "
                            f"{sm_max:.0f} MHz ({src} max clock)")
+    hbm = peaks.get("hbm_gbs")
+    tensor = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
+    if form == "fp32" and requested == "auto" and 8 <= d <= 128:
+        kernel = "assign_mma_ring"
+        if hbm and tensor and 0.5 * k * float(hbm) * 1e-3 < float(tensor):
+            gbs = prof.assign_bytes / (prof.assign_ms * 1e-3) / 1e9 if prof.assign_ms > 0 else None
+            return {"bound": "hbm", "kernel": kernel, "achieved": gbs, "peak": float(hbm),
+                    "unit": "GB/s", "frac": gbs / float(hbm) if gbs else None, "traffic": None,
+                    "peak_source": f"{src} hbm_gbs (copy)", "achieved_tflops": achieved,
+                    "fp32_peak_tflops": peak,
+                    "kernel_ms_avg": prof.assign_ms / max(1, prof.assign_launches),
+                    "kernel_launches": prof.assign_launches}
+        bound, peak = "tensor", float(tensor)
+        peak_source = f"{src} bf16_tflops_sustained (kernel timed inside a long fit)"
     roof = {"bound": bound, "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": (achieved / peak) if achieved else None,
             "traffic": traffic_of(kernel, prof, d), "peak_source": peak_source,
@@ -570,7 +587,7 @@ def run_ours(args, cfg):
             dist.destroy_process_group()
         return 0
     r0 = results[-1]
-    roofline = roofline_of(r0.precision_used, d, k, prof, clk, p32)
+    roofline = roofline_of(r0.precision_used, d, k, prof, clk, p32, args.precision)
     roofline["measured"] = (f"{args.profile_fits} profiled fits after the timed region, CUDA "
                             f"events around each launch of the distance kernel")
     if roofline.get("kernel") == "assign_small<8>":
@@ -1038,7 +1055,7 @@ def run_batched(args):
     probe = fp32_peak(dev, stream)
     p32 = probe["tflops"] if probe else derived
     ach = prof.assign_flops / (prof.assign_ms * 1e-3) / 1e12 if prof.assign_ms > 0 else None
-    roofline = {"bound": "alu", "kernel": "batch_assign<DC> (all dimension classes)",
+    roofline = {"bound": "alu", "kernel": "batch_assign<2> and batch_mma<DP> (all dimension classes)",
                 "achieved": ach, "peak": p32, "unit": "TFLOP/s",
                 "frac": ach / p32 if ach else None, "traffic": None,
                 "peak_source": ("measured: FP32 FMA probe on this GPU (%.1f TFLOP/s); derived "
