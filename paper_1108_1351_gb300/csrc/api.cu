@@ -334,12 +334,15 @@ int choose_form(int requested, int d, int k, const float* X, int* form)
             *form = KMEANS2_PRECISION_TF32X3;
             return KMEANS2_OK;
         case KMEANS2_PRECISION_AUTO:
-            // For d <= 32 the CUDA-core form is as fast per launch as the tensor-core
-            // forms and flags far fewer near ties (measured).  From d = 64 on the
-            // BF16 tensor-core form wins once k is large (k >= 512: 1.1-2.5x
-            // faster fits); with fewer centers the CUDA-core kernel is fast
-            // enough that the BF16 form's 5-10x more near-tie rechecks lose
-            // (measured on Gaussian mixtures of 4 to 1024 components).
+            // FP32 runs the tensor-core screen for 8 <= d <= 128 where its centers fit
+            // shared memory.  From d = 64, k = 512 on the 16-bit forms win (fits of
+            // 1e6 rows, ms, FP32 on CUDA cores -> AUTO: d 64 k 1024 160 -> 32 and
+            // 142 -> 16, d 128 k 512 156 -> 39 and 158 -> 17.5; Gaussian and vMF
+            // mixtures).  Below, the screen against FP16: d 64 k 32 7.4 vs 14.2, k 128
+            // 11.4 vs 11.6, k 448 26 vs 23 (vMF 6.6 vs 9.5, 11.2 vs 10.1, 23 vs 16).
+            // At d = 128, 200 < k < 512 the centers do not fit and the CUDA cores
+            // lose (k 448 155 vs 38), but need no second copy of X: a fit or a served
+            // job that fits memory there must keep fitting.
             *form = (bf && d >= 64 && k >= 512) ? KMEANS2_PRECISION_BF16 : KMEANS2_PRECISION_FP32;
             return KMEANS2_OK;
         default:

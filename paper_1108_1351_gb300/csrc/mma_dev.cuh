@@ -412,7 +412,7 @@ __device__ __forceinline__ int mma_decide(const uint32_t (&A)[2][MmaCfg<DP>::ARE
 }
 
 // One warp: row x (global) decided with the FP32 FMA chain over all centers
-// (recheck_d4's values), as the CUDA-core kernels do.  Returns the center, or
+// (recheck_d's values), as the CUDA-core kernels do.  Returns the center, or
 // open = true when the best two are within the FP32 bound.
 __device__ __forceinline__ int decide_fp32_row(const float* __restrict__ x, int d, const Centers& c,
                                                float thr_base, bool& open)
