@@ -237,9 +237,9 @@ __global__ void __launch_bounds__(kSampleThreads) sample_small_kernel(unsigned l
     sample_block(seed, n, m, k, subset, pos, tmp);
 }
 
-// Rows up to which one CTA draws: its nine passes over the keys take 25 us at n =
-// 20,000 and grow with n; the 35 launches and the read-back of the other way take
-// about 250 us however small n is.
+// Keys (n rows and m of the subset) up to which one CTA draws: its nine passes over them
+// take 25 us at n = 20,000, m = 2,000 and grow with their number; the 35 launches
+// and the read-back of the other way take about 250 us however few there are.
 constexpr long long kSampleSmall = 1 << 17;
 
 }  // namespace
@@ -317,14 +317,15 @@ int sample_device(long long n, int k, long long m, unsigned long long seed, long
 {
     long long* sel = nullptr;
     KM2_TRY(ws.alloc((void**)&sel, sizeof(long long) * (size_t)k, s));
-    if (n <= kSampleSmall) {
+    if (n + m <= kSampleSmall) {
         ++g_launches;
         sample_small_kernel<<<1, kSampleThreads, 0, s>>>(seed, n, m, k, subset, init_pos, sel);
         KM2_CUDA(cudaGetLastError());
-        return KMEANS2_OK;
+        if (k <= kRankOneCta) return KMEANS2_OK;
+    } else {
+        KM2_TRY(select_smallest(seed, 0ull, n, m, subset, s, ws));
+        KM2_TRY(select_smallest(seed, (unsigned long long)n, m, k, sel, s, ws));
     }
-    KM2_TRY(select_smallest(seed, 0ull, n, m, subset, s, ws));
-    KM2_TRY(select_smallest(seed, (unsigned long long)n, m, k, sel, s, ws));
     int grid = (k + kThreads - 1) / kThreads;
     ++g_launches;
     order_by_key<<<grid, kThreads, 0, s>>>(seed, (unsigned long long)n, sel, k, init_pos);

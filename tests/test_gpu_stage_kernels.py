@@ -119,3 +119,12 @@ def test_moved_rows_past_the_list():
     X = torch.randn(4_500_000, 16, device="cuda", generator=g)
     C = X[:40].double().contiguous()
     _same(km.step(X, C, precision="bf16"), km.step(X, C, precision="fp32"))
+
+
+@pytest.mark.parametrize("n,k,f", [(9_000, 256, 0.5), (9_000, 257, 0.5), (9_000, 5_000, 1.0),
+                                   (65_536, 300, 1.0), (65_537, 300, 1.0), (131_071, 7, 1e-5),
+                                   (131_072, 7, 1e-5), (400, 400, 1.0), (1, 1, 1.0)])
+def test_draws_around_the_one_cta_limits(n, k, f):
+    sub, pos = km.sample(n, k, f, 11, device="cuda")
+    osub, opos = oracle.sample(n, k, f, 11)
+    assert np.array_equal(to_np(sub), osub) and np.array_equal(to_np(pos), opos)
