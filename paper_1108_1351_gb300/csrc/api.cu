@@ -188,6 +188,21 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// The caller's FP64 buffer if a kernel of this call may store to it: aligned, and
+// managed or on the current device.  Null otherwise: a copy takes any device
+// address, a kernel's 8-byte store to an odd or a foreign one is a fault.
+static double* kernel_store_f64(double* p)
+{
+    cudaPointerAttributes a;
+    int dev = -1;
+    if ((reinterpret_cast<uintptr_t>(p) & 7) != 0 || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const bool ok = a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+    return ok ? p : nullptr;
+}
 
 int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, int d,
                     int max_iter, cudaStream_t s)
@@ -850,7 +865,7 @@ int kmeans_step(const float* X, int64_t n, int32_t d, int32_t k, const double* c
     bool published = false;
     KM2_TRY(run_stage(Xd, n, d, w, labels, 0.0, 1, false, s, ws.sm_count, out, nullptr, nullptr,
                       r.opt.profile, "kmeans2 step", nullptr, nullptr, false,
-                      cen_dev ? centers_out : nullptr, &published));
+                      kernel_store_f64(centers_out), &published));
     if (!published)
         KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
                                  cen_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
@@ -906,8 +921,15 @@ int kmeans_step_noalloc(const float* X, int64_t n, int32_t d, int32_t k,
     KM2_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StageState), s));
     KM2_TRY(launch_maxabs(X, n, d, w.st, s, ws.sm_count));
     StageState out;
+    bool published = false;
     KM2_TRY(run_stage(X, n, d, w, labels_out, 0.0, 1, false, s, ws.sm_count, out, nullptr,
-                      nullptr, nullptr, "kmeans2 step", nullptr, nullptr, false, centers_out));
+                      nullptr, nullptr, "kmeans2 step", nullptr, nullptr, false,
+                      kernel_store_f64(centers_out), &published));
+    if (!published) {
+        KM2_CUDA(cudaMemcpyAsync(centers_out, w.c.c64, sizeof(double) * (size_t)k * d,
+                                 cudaMemcpyDeviceToDevice, s));
+        KM2_CUDA(cudaStreamSynchronize(s));
+    }
     if (J_out) *J_out = out.J;
     if (shift_out) *shift_out = out.shift;
     if (empty_out) *empty_out = out.empty;
@@ -1013,7 +1035,7 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
     KM2_TRY(run_stage(Xd, n, d, w, labels, tol, max_iter, use_graph, s, ws.sm_count, ss,
                       o.traj_J_slow, o.traj_shift_slow, o.profile, "kmeans2 slow stage",
                       o.traj_centers_slow, o.traj_counts_slow, false,
-                      cen_dev ? centers_out : nullptr, &published));
+                      kernel_store_f64(centers_out), &published));
     rr.precision_used = w.form;
     rr.iters_slow = ss.iter;
     rr.converged_slow = ss.converged;
