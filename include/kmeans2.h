@@ -101,7 +101,9 @@ extern "C" {
                                          tensor-core screen for 8 <= d <= 128: split-FP16
                                          products decide the rows outside their error
                                          bound, the FP32 chain the others (same labels,
-                                         centers and J; reported as FP32) */
+                                         centers and J; reported as FP32).  A stage
+                                         whose first passes leave too many rows open
+                                         goes on without it */
 #define KMEANS2_PRECISION_TF32X3 3    /* cross term on the tensor cores as three TF32
                                          products of the exact hi/lo split of the FP32
                                          operands; d in {4, 8, 16, 32}, k <= 256 */
@@ -619,6 +621,12 @@ KMEANS2_API const char* kmeans2_strerror(int status);
    its error string), or "" if none.  Thread-local storage, valid until the
    thread's next failing call. */
 KMEANS2_API const char* kmeans2_last_error(void);
+
+/* Passes of the calling thread's fits and steps so far that went through the
+   tensor-core screen (precision AUTO; the batched form and a server's worker
+   threads are not counted).  A difference over a call says whether, and for how
+   many of its iterations, the call's shape and data took it. */
+KMEANS2_API int64_t kmeans2_screen_passes(void);
 
 /* Library version, (major << 16) | minor. */
 KMEANS2_API int32_t kmeans2_version(void);

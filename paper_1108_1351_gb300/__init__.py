@@ -7,10 +7,10 @@ binds it (``binding``) and provides seeded synthetic inputs (``synth``).
 """
 from .binding import (FitResult, KMeans2Error, LIB_PATH, Profile, Served, Server, Shard,
                       batched_tile_shape, declared_symbols, fit, fit_batched, fit_data_parallel, fit_sharded,
-                      fit_streamed, footprint, load, release_memory, sample, step, step_noalloc,
+                      fit_streamed, footprint, load, release_memory, sample, screen_passes, step, step_noalloc,
                       strerror, subset_size, version)
 
 __all__ = ["FitResult", "KMeans2Error", "LIB_PATH", "Profile", "Served", "Server", "Shard",
            "batched_tile_shape", "declared_symbols", "fit", "fit_batched", "fit_data_parallel", "fit_sharded",
-           "fit_streamed", "footprint", "load", "release_memory", "sample", "step",
+           "fit_streamed", "footprint", "load", "release_memory", "sample", "screen_passes", "step",
            "step_noalloc", "strerror", "subset_size", "version"]

@@ -225,6 +225,8 @@ def load():
         lib.kmeans2_strerror.argtypes = [ctypes.c_int]
         lib.kmeans2_last_error.restype = ctypes.c_char_p
         lib.kmeans2_last_error.argtypes = []
+        lib.kmeans2_screen_passes.restype = i64
+        lib.kmeans2_screen_passes.argtypes = []
         lib.kmeans2_release_memory.restype = ctypes.c_int
         lib.kmeans2_release_memory.argtypes = []
         lib.kmeans2_version.restype = i32
@@ -600,6 +602,12 @@ def fit_data_parallel(X_local, row0: int, n_total: int, k: int, subset_fraction:
         return sh.result()
     finally:
         sh.close()
+
+
+def screen_passes() -> int:
+    """Passes of this thread's fits and steps so far that went through the
+    tensor-core screen (kmeans2_screen_passes)."""
+    return int(load().kmeans2_screen_passes())
 
 
 def release_memory() -> None:

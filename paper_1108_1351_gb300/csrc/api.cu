@@ -34,6 +34,7 @@ struct NvtxRange {
 };
 
 thread_local long long g_launches = 0;
+thread_local long long g_screen_passes = 0;
 
 namespace {
 thread_local char g_last_error[512] = "";
@@ -294,6 +295,24 @@ int launch_stage_recheck(const float* X, int d, Workspace& w, int* labels, cudaS
     return launch_recheck(X, d, w.c, labels, w.list, w.st, w.acc, settles, s, sm_count);
 }
 
+// Share of open rows up to which the screen is kept; above, its passes with the FP32
+// pass over the open rows cost more than the CUDA-core kernel's.  Fits of 20 + 20
+// iterations, us with the screen and without, open share in the slow stage: n = 4e6,
+// d = 8, k = 32 3994 / 4095 at 0.018, 5493 / 5213 at 0.044; n = 1e6, d = 16, k = 1000 19.9
+// / 22.5 ms at 0.035, 33.0 / 26.8 at 0.081; d = 32, k = 200 16.7 / 21.8 ms at 0.30-0.46,
+// 35.1 / 26.2 at 0.86; d = 64, k = 200 21.3 / 36.5 at 0.17-0.36, 41.1 / 39.5 at 0.49-0.60.
+// Above d = 16 the recheck decides open rows over the whole GPU, hence the two lines.
+constexpr double kMaxOpenNarrow = 0.04, kMaxOpenWide = 0.5;
+
+void review_screen(Workspace& w, int d, const StageState& st, long long rows, int passes)
+{
+    if (!w.first_pass) return;
+    w.first_pass = false;
+    const double open = d <= 16 ? (double)st.open_rows : (double)st.listed_total;
+    const double most = (d <= 16 ? kMaxOpenNarrow : kMaxOpenWide) * (double)rows * passes;
+    if (w.screen && open > most) w.screen = false;
+}
+
 // The fused distance kernel of the chosen form.
 int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels, cudaStream_t s,
                   int sm_count)
@@ -312,8 +331,10 @@ int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels,
                                    0, w.mv, s, sm_count));
         return launch_moved_sums(X, n, d, w.mv, w.c.k, labels, w.st, w.acc, s, sm_count);
     }
-    if (screened(X, d, w))
-        return launch_assign_mma(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
+    if (screened(X, d, w)) {
+        ++g_screen_passes;
+        return launch_assign_mma(X, n, d, w.c, labels, w.st, w.acc, w.list, w.first_pass, s, sm_count);
+    }
     return launch_assign_fp32(X, n, d, w.c, labels, w.st, w.acc, w.list, s, sm_count);
 }
 
@@ -377,8 +398,9 @@ int launch_iteration(const float* X, long long n, int d, Workspace& w, int* labe
 }
 
 // The stage loop as one graph: a WHILE conditional node whose body is one iteration.
-int run_loop_graph(const float* X, long long n, int d, Workspace& w, int* labels, cudaStream_t s,
-                   int sm_count)
+// before: iterations the stage has run already.
+int run_loop_graph(const float* X, long long n, int d, Workspace& w, int* labels, int before,
+                   cudaStream_t s, int sm_count)
 {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -404,9 +426,9 @@ int run_loop_graph(const float* X, long long n, int d, Workspace& w, int* labels
         e = cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0,
                                           cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) { set_last_error("cudaStreamBeginCaptureToGraph", e); rc = KMEANS2_ERR_CUDA; break; }
-        const long long body0 = g_launches;
+        const long long body0 = g_launches, screen0 = g_screen_passes;
         rc = launch_iteration(X, n, d, w, labels, (unsigned long long)handle, 1, 0, s, sm_count);
-        const long long body_launches = g_launches - body0;
+        const long long body_launches = g_launches - body0, body_screen = g_screen_passes - screen0;
         cudaGraph_t captured = nullptr;
         e = cudaStreamEndCapture(s, &captured);
         if (rc != KMEANS2_OK) break;
@@ -423,7 +445,9 @@ int run_loop_graph(const float* X, long long n, int d, Workspace& w, int* labels
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) { set_last_error("cudaMemcpyAsync", e); rc = KMEANS2_ERR_CUDA; break; }
         // the capture counted the body's kernels once; each further iteration reruns them
+        iters -= before;
         g_launches += body_launches * (iters > 1 ? iters - 1 : 0);
+        g_screen_passes += body_screen * (iters > 1 ? iters - 1 : 0);
     } while (0);
     if (exec) cudaGraphExecDestroy(exec);
     cudaGraphDestroy(graph);
@@ -454,10 +478,14 @@ int run_loop_host(const float* X, long long n, int d, Workspace& w, int* labels,
             rc = launch_iteration(X, n, d, w, labels, 0ull, 0, 0, s, sm_count);
         }
         if (rc != KMEANS2_OK) break;
-        int done = 0;
-        cudaError_t e = cudaMemcpyAsync(&done, &w.st->done, sizeof(int), cudaMemcpyDeviceToHost, s);
+        // (the whole state costs 2 us more than the flag)
+        StageState st;
+        cudaError_t e = w.first_pass && w.screen
+                            ? cudaMemcpyAsync(&st, w.st, sizeof(st), cudaMemcpyDeviceToHost, s)
+                            : cudaMemcpyAsync(&st.done, &w.st->done, sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) { set_last_error("stage loop", e); rc = KMEANS2_ERR_CUDA; break; }
+        if (w.screen) review_screen(w, d, st, n, 1);
         if (prof) {
             float ms = 0.f;
             cudaEventElapsedTime(&ms, ev0, ev1);
@@ -466,7 +494,7 @@ int run_loop_host(const float* X, long long n, int d, Workspace& w, int* labels,
             prof->assign_flops += 2.0 * (double)n * w.c.k * d;
             prof->assign_bytes += 4.0 * (double)n * d;
         }
-        if (done) break;
+        if (st.done) break;
     }
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);
@@ -490,6 +518,7 @@ int run_loop_queued(const float* X, long long n, int d, Workspace& w, int* label
         if (publish) KM2_TRY(launch_publish_centers(w.st, w.c.c64, (long long)w.c.k * d, publish, s));
         KM2_CUDA(cudaMemcpyAsync(&out, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
         KM2_CUDA(cudaStreamSynchronize(s));
+        review_screen(w, d, out, n, out.iter);
         if (out.error || out.done || queued >= max_iter) break;
         chunk = std::min(2 * chunk, 32);
     }
@@ -535,6 +564,7 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
 {
     NvtxRange stage_range(name);
     KM2_TRY(launch_stage_begin(w.c, w.acc, w.st, tol, max_iter, s));
+    w.first_pass = true;
     KM2_TRY(launch_qsum(X, n, d, w.st, s, sm_count));
     KM2_TRY(prepare_stage_points(X, n, d, w, *w.ws, s));
     bool finished = false, have_out = false;
@@ -549,24 +579,26 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
         KM2_TRY(launch_iteration(X, n, d, w, labels, 0ull, 0, 0, s, sm_count));
         finished = true;
     }
-    if (!finished && probe16 && w.form == KMEANS2_PRECISION_FP16) {
-        // one FP16 iteration from the host; if its single pass left too many
-        // rows undecided, the rest of the stage runs the split form (every
-        // form decides each row exactly, so the switch changes no result)
+    probe16 = probe16 && w.form == KMEANS2_PRECISION_FP16;
+    if (!finished && (probe16 || (use_graph && !prof && screened(X, d, w)))) {
+        // one iteration from the host, whose state says how the rest of the stage
+        // runs (every form decides each row exactly, so a switch changes no
+        // result): without the screen if that left too many rows open, in the
+        // split form if the FP16 pass left too many undecided
         KM2_TRY(run_loop_host(X, n, d, w, labels, 1, s, sm_count, prof));
         StageState p;
         KM2_CUDA(cudaMemcpyAsync(&p, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
         KM2_CUDA(cudaStreamSynchronize(s));
         finished = p.done != 0 || p.error != 0;
         remaining = max_iter - 1;
-        if (!finished && (double)p.undecided16_total > kFp16ProbeMaxUndecided * (double)n) {
+        if (probe16 && !finished && (double)p.undecided16_total > kFp16ProbeMaxUndecided * (double)n) {
             w.form = KMEANS2_PRECISION_BF16;
             KM2_TRY(prepare_stage_points(X, n, d, w, *w.ws, s));
         }
     }
     if (!finished) {
         if (use_graph && !prof)
-            KM2_TRY(run_loop_graph(X, n, d, w, labels, s, sm_count));
+            KM2_TRY(run_loop_graph(X, n, d, w, labels, max_iter - remaining, s, sm_count));
         else
             KM2_TRY(run_loop_host(X, n, d, w, labels, remaining, s, sm_count, prof));
     }
@@ -706,6 +738,8 @@ const char* kmeans2_strerror(int status)
 }
 
 const char* kmeans2_last_error(void) { return km2::last_error(); }
+
+int64_t kmeans2_screen_passes(void) { return g_screen_passes; }
 
 uint64_t kmeans2_fit_footprint(int64_t n, int32_t d, int32_t k, double subset_fraction,
                                int32_t max_iter, int32_t precision, int32_t x_on_host,
@@ -1278,6 +1312,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
         return launch_maxabs(Xc, rows, d, w.st, s, ws.sm_count);
     }));
     KM2_TRY(launch_stage_begin(w.c, w.acc, w.st, tol, max_iter, s));
+    w.first_pass = true;
     StageState ss;
     std::memset(&ss, 0, sizeof(ss));
     for (int it = 0; it < max_iter; ++it) {
@@ -1294,6 +1329,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
         KM2_CUDA(cudaStreamSynchronize(s));
         if (ss.error) return map_stage_error(ss.error);
         if (ss.done) break;
+        review_screen(w, d, ss, n, 1);
     }
     if (o.traj_J_slow && ss.iter > 0)
         KM2_CUDA(cudaMemcpyAsync(o.traj_J_slow, w.traj_J, sizeof(double) * ss.iter,

@@ -14,6 +14,8 @@ namespace km2 {
 
 // Kernels launched by the calling thread (every launch site increments it).
 extern thread_local long long g_launches;
+// Of them, the distance kernel's launches with the tensor-core screen (kmeans2_screen_passes).
+extern thread_local long long g_screen_passes;
 
 // Thread-local text of the last CUDA failure, returned by kmeans2_last_error().
 void set_last_error(const char* where, cudaError_t e);
@@ -185,14 +187,18 @@ int launch_assign_fp32(const float* X, long long n, int d, const Centers& c, int
 // assign_mma.cu: the FP32 form with a tensor-core screen (split-FP16 products
 // decide the rows outside their bound, the FP32 chain the others)
 int assign_mma_supported(int d, int k, const float* X);
+// first: the form of a stage's first passes (units with many open rows taken together,
+// open rows counted)
 int launch_assign_mma(const float* X, long long n, int d, const Centers& c, int* labels,
-                      StageState* st, const Accum& acc, int* list, cudaStream_t s, int sm_count);
+                      StageState* st, const Accum& acc, int* list, int first, cudaStream_t s,
+                      int sm_count);
 
 // ---------------------------------------------------------------- stage plumbing (api.cu)
 // Per-stage device state of one fit: centers, exact sums, loop state, near-tie list.
 struct Workspace {
     int form = KMEANS2_PRECISION_FP32;   // distance-kernel form used by this call
     bool screen = false;                 // FP32 form: rows go through the tensor-core screen first
+    bool first_pass = false;             // the stage's first passes, until review_screen
     Centers c{};
     Accum acc{};
     StageState* st = nullptr;
@@ -224,6 +230,9 @@ int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels,
 // The FP64 recheck of the rows that launch_assign listed.
 int launch_stage_recheck(const float* X, int d, Workspace& w, int* labels, cudaStream_t s,
                          int sm_count);
+// After a stage's first `passes` passes over `rows` rows (st: the state then): whether
+// the later ones keep the screen.
+void review_screen(Workspace& w, int d, const StageState& st, long long rows, int passes);
 // Resolves a requested precision to the form this shape runs in.
 int choose_form(int requested, int d, int k, const float* X, int* form);
 int map_stage_error(int err);

@@ -74,7 +74,11 @@ __device__ __forceinline__ void cp_async_wait_group()
 }
 
 // UNIT: rows a warp takes at a time (32 where n is too small to give every warp 64).
-template <int DP, int NT, bool SINGLE, bool FULL, int UNIT>
+// DENSE (d <= 16): units with many open rows are decided a lane per row, and the open
+// rows are counted.  A kernel of its own for a stage's first passes, whose count
+// says whether the later ones keep the screen (review_screen): the code it adds
+// costs the others 3 to 7 % (n = 1e8, d = 8, k = 32, a fit 65.6 -> 67.6 ms).
+template <int DP, int NT, bool SINGLE, bool FULL, int UNIT, bool DENSE>
 __global__ void __launch_bounds__((RingCfg<DP, SINGLE>::THREADS), (RingCfg<DP, SINGLE>::MINB))
 assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __restrict__ labels,
                 StageState* st, Accum acc, int* __restrict__ list, int ntiles, int use_sacc)
@@ -84,8 +88,10 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
     constexpr bool WIDE = R::WIDE;
     constexpr int H = UNIT / 32;
     static_assert(!WIDE || UNIT == 32, "wide rows: one 32-row block per warp and step");
+    static_assert(!(WIDE && DENSE), "wide rows: the recheck decides the open ones");
     constexpr int kFlushSteps = kFlushPoints / (kWarps * UNIT);   // steps per int64 partial
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_open;                               // DENSE: rows the screen left open
     if (st->error) return;
     const int k = c.k, d = FULL ? DP : c.d;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -144,6 +150,7 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
 #pragma unroll
     for (int s = 0; s < (WIDE ? 1 : S - 1); ++s) issue(s * stage_bytes);
 
+    if (DENSE && tid == 0) s_open = 0;
     mma_load_centers<DP>(c, ntiles, ms, sb, sn);
     if (use_sacc) {
         for (int e = tid; e < k * d; e += kThreads) sacc[e] = 0;
@@ -191,6 +198,15 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
             for (int h = 0; h < H; ++h) {
                 unsigned todo = __ballot_sync(0xffffffffu, open[h]);
                 bool listed = false;
+                if constexpr (DENSE) {
+                    if (lane == 0) atomicAdd(&s_open, __popc(todo));
+                    if (__popc(todo) >= lanes_from(d, k)) {
+                        const int l = decide_fp32_lanes<DP, FULL>(xr + (32 * h + 8 * t + g) * d, d, c.cnorm, c.c32t,
+                                                                  c.kpad, k, thr_base);
+                        if (open[h]) { lab[h] = l; listed = l < 0; }
+                        todo = 0;
+                    }
+                }
 #pragma unroll 1
                 while (todo) {
                     const int o = __ffs(todo) - 1;
@@ -289,12 +305,16 @@ assign_mma_ring(const float* __restrict__ X, long long n, Centers c, int* __rest
         }
     }
     cp_async_wait_group<0>();
+    if constexpr (DENSE) {
+        __syncthreads();
+        if (tid == 0 && s_open) atomicAdd(&st->open_rows, (unsigned long long)s_open);
+    }
 }
 
 template <int DP, bool SINGLE, int UNIT>
 size_t ring_bytes(int d) { return (size_t)RingCfg<DP, SINGLE>::W * RingCfg<DP, SINGLE>::S * 4 * UNIT * (d + 1); }
 
-template <int DP, int NT, bool SINGLE, bool FULL, int UNIT>
+template <int DP, int NT, bool SINGLE, bool FULL, int UNIT, bool DENSE>
 int launch_ring_u(const float* X, long long n, const Centers& c, int* labels, StageState* st,
                   const Accum& acc, int* list, int ntiles, cudaStream_t s, int sm_count)
 {
@@ -303,7 +323,7 @@ int launch_ring_u(const float* X, long long n, const Centers& c, int* labels, St
     const size_t sums = (size_t)c.k * c.d * 8 + (size_t)c.k * 4;
     const int use_sacc = base + sums <= (size_t)kSmemCap;
     const size_t sm = base + (use_sacc ? sums : 0);
-    const void* kfn = (const void*)assign_mma_ring<DP, NT, SINGLE, FULL, UNIT>;
+    const void* kfn = (const void*)assign_mma_ring<DP, NT, SINGLE, FULL, UNIT, DENSE>;
     KM2_TRY(set_max_dynamic_smem(kfn, kSmemCap));
     int per_sm = 0;
     KM2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, R::THREADS, sm));
@@ -311,7 +331,7 @@ int launch_ring_u(const float* X, long long n, const Centers& c, int* labels, St
     const long long steps = (n + R::W * UNIT - 1) / (R::W * UNIT);
     const int grid = (int)std::max(1ll, std::min((long long)sm_count * per_sm, steps));
     ++g_launches;
-    assign_mma_ring<DP, NT, SINGLE, FULL, UNIT><<<grid, R::THREADS, sm, s>>>(X, n, c, labels, st, acc,
+    assign_mma_ring<DP, NT, SINGLE, FULL, UNIT, DENSE><<<grid, R::THREADS, sm, s>>>(X, n, c, labels, st, acc,
                                                                            list, ntiles, use_sacc);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
@@ -319,39 +339,39 @@ int launch_ring_u(const float* X, long long n, const Centers& c, int* labels, St
 
 template <int DP, int NT, bool SINGLE>
 int launch_ring(const float* X, long long n, const Centers& c, int* labels, StageState* st,
-                const Accum& acc, int* list, int ntiles, cudaStream_t s, int sm_count)
+                const Accum& acc, int* list, int ntiles, int first, cudaStream_t s, int sm_count)
 {
     // 64 rows per warp and step once every warp of two or three CTAs per SM gets
     // some; below, 32 (too few warps otherwise)
     const bool small = n < (long long)sm_count * RingCfg<DP, SINGLE>::MINB * RingCfg<DP, SINGLE>::W * 64;
-#define KM2_RING(FULL_, UNIT_) \
-    return launch_ring_u<DP, NT, SINGLE, FULL_, UNIT_>(X, n, c, labels, st, acc, list, ntiles, s, sm_count)
-    if constexpr (DP > 16) KM2_RING(false, 32);
-    if constexpr (DP <= 16) if (c.d == DP) {
-        if (small) KM2_RING(true, 32);
-        KM2_RING(true, 64);
-    }
-    if constexpr (DP == 16) {
-        if (small) KM2_RING(false, 32);
-        KM2_RING(false, 64);
-    }
+#define KM2_RING(FULL_, UNIT_, DENSE_) \
+    return launch_ring_u<DP, NT, SINGLE, FULL_, UNIT_, DENSE_>(X, n, c, labels, st, acc, list, ntiles, s, sm_count)
+#define KM2_RING_NARROW(FULL_)                 \
+    if (small && first) KM2_RING(FULL_, 32, true); \
+    if (small) KM2_RING(FULL_, 32, false);     \
+    if (first) KM2_RING(FULL_, 64, true);      \
+    KM2_RING(FULL_, 64, false)
+    if constexpr (DP > 16) KM2_RING(false, 32, false);
+    if constexpr (DP <= 16) if (c.d == DP) { KM2_RING_NARROW(true); }
+    if constexpr (DP == 16) { KM2_RING_NARROW(false); }
+#undef KM2_RING_NARROW
 #undef KM2_RING
     return KMEANS2_ERR_UNSUPPORTED;
 }
 
 template <int DP>
 int launch_ring_k(const float* X, long long n, const Centers& c, int* labels, StageState* st,
-                  const Accum& acc, int* list, cudaStream_t s, int sm_count)
+                  const Accum& acc, int* list, int first, cudaStream_t s, int sm_count)
 {
     if constexpr (DP > 64) {
         // two accumulators per block (mma_chunk): chunks of 16 centers
-        if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, s, sm_count);
-        return launch_ring<DP, 2, false>(X, n, c, labels, st, acc, list, (c.k + 15) / 16 * 2, s, sm_count);
+        if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, first, s, sm_count);
+        return launch_ring<DP, 2, false>(X, n, c, labels, st, acc, list, (c.k + 15) / 16 * 2, first, s, sm_count);
     } else {
         if constexpr (DP <= 16)
-            if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, s, sm_count);
-        if (c.k <= 32) return launch_ring<DP, 4, true>(X, n, c, labels, st, acc, list, 4, s, sm_count);
-        return launch_ring<DP, 4, false>(X, n, c, labels, st, acc, list, (c.k + 31) / 32 * 4, s, sm_count);
+            if (c.k <= 16) return launch_ring<DP, 2, true>(X, n, c, labels, st, acc, list, 2, first, s, sm_count);
+        if (c.k <= 32) return launch_ring<DP, 4, true>(X, n, c, labels, st, acc, list, 4, first, s, sm_count);
+        return launch_ring<DP, 4, false>(X, n, c, labels, st, acc, list, (c.k + 31) / 32 * 4, first, s, sm_count);
     }
 }
 
@@ -373,10 +393,11 @@ int assign_mma_supported(int d, int k, const float* X)
 }
 
 int launch_assign_mma(const float* X, long long n, int d, const Centers& c, int* labels,
-                      StageState* st, const Accum& acc, int* list, cudaStream_t s, int sm_count)
+                      StageState* st, const Accum& acc, int* list, int first, cudaStream_t s,
+                      int sm_count)
 {
     switch (mma_dp(d)) {
-#define KM2_CASE(DD) case DD: return launch_ring_k<DD>(X, n, c, labels, st, acc, list, s, sm_count);
+#define KM2_CASE(DD) case DD: return launch_ring_k<DD>(X, n, c, labels, st, acc, list, first, s, sm_count);
         KM2_RING_DPS(KM2_CASE)
 #undef KM2_CASE
         default: return KMEANS2_ERR_UNSUPPORTED;

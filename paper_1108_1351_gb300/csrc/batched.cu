@@ -574,6 +574,7 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
         const float thr_base = 2.0f * st->cmax2;
         const MmaScale ms = mma_scale(st, d, MmaCfg<DP>::KS);
         const int ntiles = (k + 31) / 32 * 4;
+        const int lanes = lanes_from(d, k);
         mma_load_centers<DP>(c, ntiles, ms, sb, sn);
         if (B::SACC) {
             for (int e = tid; e < k * DP; e += kT) sacc[e] = 0;
@@ -623,8 +624,14 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
             unsigned todo = __ballot_sync(0xffffffffu, open);
             if (todo) {
                 bool listed = open;
-                if (DP <= 16) {
+                if constexpr (DP <= 16) {
                     listed = false;
+                    if (__popc(todo) >= lanes) {
+                        const int l = decide_fp32_lanes<DP, DP == 8>(X + (row0 + min(r, rows - 1)) * d, d,
+                                                                     c.cnorm, c.c32t, c.kpad, k, thr_base);
+                        if (open) { lab = l; listed = l < 0; }
+                        todo = 0;
+                    }
 #pragma unroll 1
                     while (todo) {
                         const int o = __ffs(todo) - 1;

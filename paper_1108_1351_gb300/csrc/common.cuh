@@ -57,6 +57,10 @@ struct StageState {
     long long undecided16_total;
     // finalize: CTAs done with their centers (the last one reduces and resets it)
     unsigned int ticket;
+    // rows the tensor-core screen left open in the stage's first passes (d <= 16), and
+    // rows listed for the recheck over all passes (d > 16: the open ones)
+    unsigned long long open_rows;
+    long long listed_total;
 };
 
 // Per-center scratch of finalize, in 8-byte words per center (finalize_center_warp).

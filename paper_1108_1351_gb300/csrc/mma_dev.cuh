@@ -452,4 +452,69 @@ __device__ __forceinline__ int decide_fp32_row(const float* __restrict__ x, int 
     return bi;
 }
 
+// The same for 32 rows at once, a lane per row (x: this lane's row, shared or
+// global): what a unit with many open rows takes.  Data far from the origin has
+// units in which nearly all rows are open, and row after row they cost up to six
+// times what the CUDA-core kernels take for them (a step with an offset of 1000 in
+// the data, us, row by row / a lane per row / on CUDA cores: n = 1e6, d = 16, k = 1000
+// 7908 / 4116 / 3373, n = 4e6, d = 8, k = 32 2249 / 1623 / 1712).  Bound by FMAs and the
+// broadcast loads of the centers.  Returns the center, or -1 for open.
+template <int DP, bool FULL>
+__device__ __forceinline__ int decide_fp32_lanes(const float* x, int d, const float* __restrict__ cnorm,
+                                              const float* __restrict__ c32t, int kpad, int k, float thr_base)
+{
+    static_assert(DP <= 16, "the row is held in registers");
+    float xm2[DP];
+    float x2 = 0.0f;
+#pragma unroll
+    for (int t = 0; t < DP; t += 4) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (FULL) {
+            v = *reinterpret_cast<const float4*>(x + t);
+        } else {
+            if (t < d) v.x = x[t];
+            if (t + 1 < d) v.y = x[t + 1];
+            if (t + 2 < d) v.z = x[t + 2];
+            if (t + 3 < d) v.w = x[t + 3];
+        }
+        x2 = fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, x2))));
+        xm2[t] = -2.0f * v.x;
+        xm2[t + 1] = -2.0f * v.y;
+        xm2[t + 2] = -2.0f * v.z;
+        xm2[t + 3] = -2.0f * v.w;
+    }
+    float b1 = INFINITY, b2 = INFINITY;
+    int bi = 0;
+#pragma unroll 1
+    for (int j0 = 0; j0 < k; j0 += 4) {            // kpad is a multiple of 128
+        const float4 n4 = __ldg(reinterpret_cast<const float4*>(cnorm + j0));
+        float a[4] = {n4.x, n4.y, n4.z, n4.w};
+        const float* ct = c32t + j0;
+#pragma unroll
+        for (int t = 0; t < DP; ++t) {
+            if (FULL || t < d) {
+                const float4 w = __ldg(reinterpret_cast<const float4*>(ct + (long long)t * kpad));
+                a[0] = fmaf(xm2[t], w.x, a[0]);
+                a[1] = fmaf(xm2[t], w.y, a[1]);
+                a[2] = fmaf(xm2[t], w.z, a[2]);
+                a[3] = fmaf(xm2[t], w.w, a[3]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float v = j0 + q < k ? a[q] : INFINITY;      // padding may hold anything
+            b2 = fminf(b2, fmaxf(b1, v));
+            if (v < b1) { b1 = v; bi = j0 + q; }
+        }
+    }
+    return b2 - b1 > tie_kappa(d) * (thr_base + x2) + tie_abs(d + 1) ? bi : -1;
+}
+
+// Open rows of a 32-row unit from which decide_fp32_lanes is cheaper than as many
+// decide_fp32_row: instructions of the one over those of the other.
+__device__ __forceinline__ int lanes_from(int d, int k)
+{
+    return (k + 3) / 4 * (5 * d + 16) / ((k + 63) / 64 * 5 * d + 60) + 1;
+}
+
 }  // namespace km2

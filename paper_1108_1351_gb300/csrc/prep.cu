@@ -311,6 +311,7 @@ int launch_qsum(const float* X, long long n, int d, StageState* st, cudaStream_t
 __global__ void recheck_reset_kernel(StageState* st)
 {
     st->rechecked_total += st->recheck_count;
+    st->listed_total += st->recheck_count;
     st->recheck_count = 0;
 }
 

@@ -270,6 +270,7 @@ int resume_maxabs(kmeans2_shard* sh, kmeans2_exchange* next)
     KM2_CUDA(cudaGetLastError());
     KM2_TRY(launch_stage_begin(sh->w.c, sh->w.acc, sh->w.st, sh->stage == 0 ? sh->tol_fast : sh->tol,
                                sh->max_iter, s));
+    sh->w.first_pass = true;
     StageState st;
     KM2_CUDA(cudaMemcpyAsync(&st, sh->w.st, sizeof(st), cudaMemcpyDeviceToHost, s));
     KM2_CUDA(cudaStreamSynchronize(s));
@@ -296,6 +297,7 @@ int resume_iter(kmeans2_shard* sh, kmeans2_exchange* next)
     KM2_CUDA(cudaMemcpyAsync(&st, sh->w.st, sizeof(st), cudaMemcpyDeviceToHost, s));
     KM2_CUDA(cudaStreamSynchronize(s));
     if (st.error) return map_stage_error(st.error);
+    review_screen(sh->w, sh->d, st, sh->stage_rows(), 1);
     if (!st.done) return run_local_pass(sh, next);
     // stage finished
     const kmeans2_options& o = sh->opt;
