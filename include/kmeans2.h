@@ -377,8 +377,8 @@ typedef struct kmeans2_job {
  *  jobs      count descriptors (host array).
  *  results   count results (host array), may be NULL.
  *  opt       may be NULL; precision must be FP32 or AUTO (the FP32 form; under
- *            AUTO the autotuner may run a class of d >= 8 through the
- *            tensor-core screen, with the same results).
+ *            AUTO jobs of d >= 8 run through the tensor-core screen, with the
+ *            same results).
  * Errors: KMEANS2_ERR_INVALID (a job out of range; nothing is run),
  * KMEANS2_ERR_NONFINITE (some job holds NaN / inf: the other jobs complete),
  * KMEANS2_ERR_NOMEM, KMEANS2_ERR_CUDA.
@@ -388,8 +388,8 @@ KMEANS2_API int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs,
 
 /*
  * kmeans2_batched_tile_shape -- the choice the batched form's autotuner made in
- * this process among the CUDA-core kernels for the dimension class of d (whether
- * or not the screen then runs the class): point slots per lane
+ * this process among the CUDA-core kernels for the dimension class of d (also
+ * where the screen runs the class): point slots per lane
  * (*points), lanes that share each point (*lanes; 1 = whole points per
  * thread) and 1024-point tiles per work item (*tiles).  Output pointers are
  * host memory and must not be NULL.  Returns KMEANS2_OK, or

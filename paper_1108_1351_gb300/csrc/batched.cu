@@ -19,12 +19,13 @@
 // order, which the bound covers, so every decision, and with it each job's
 // result, equals kmeans2_fit on that job alone.
 //
-// The tile shape (point slots per lane, lanes per point) and the tiles per
-// work item are chosen per dimension class by an autotuner: on the first call
-// for a class it times the real first pass of the batch and a delta pass
+// Under precision AUTO jobs of d >= 8 run the tensor-core screen (batch_mma); the
+// tile shape (point slots per lane, lanes per point) and the tiles per work item of
+// the CUDA-core kernels are chosen per dimension class by an autotuner: on the
+// first call for a class it times the real first pass of the batch and a delta pass
 // after it for each shape and a few item sizes (resetting the sums between
-// trials) and keeps the fastest for the rest of the process.  CTAs claim items from an atomic
-// counter, largest jobs first, so the iterations in which only a few large
+// trials) and keeps the fastest for the rest of the process.  CTAs claim items
+// from an atomic counter, largest jobs first, so the iterations in which only a few large
 // jobs still run keep every SM busy.
 #include <algorithm>
 #include <chrono>
@@ -512,10 +513,13 @@ batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item
 // through a stage of cp.async copies that is refilled while their MMAs run (after
 // the sums in a full pass, which reads every row's coordinates again).  Rows it
 // leaves open go to the FP32 chain in the same warp up to d = 16, else to the
-// recheck's FP32 pass.  The autotuner takes it where its passes are faster; in a
-// batch of 64 instances (n 1e3 .. 1e6, d 2 .. 64, k 2 .. 256) the d = 64 class went
-// from 45 % of the call to 0.2 ms an iteration, the call from 262 to 151 ms (with
-// the gather over many CTAs), and to 119 ms with the update over many CTAs.
+// recheck's FP32 pass.  It was the faster kernel in every batch tried (ms, CUDA cores
+// and screen: 64 instances 94.5 / 55.1; 256 318 / 177; one job of 1e6, k = 100, d 8 9.7 /
+// 8.1, d 16 12.7 / 9.4, d 32 18.6 / 11.7, d 64 33.0 / 18.2; four of 3,000, k = 20, d 8 1.13 /
+// 1.08, d 64 2.04 / 1.41; 256 of 1,000, k = 8, d 8 5.74 / 5.52).  In a batch of 64
+// instances (n 1e3 .. 1e6, d 2 .. 64, k 2 .. 256) the d = 64 class went from 45 % of the
+// call to 0.2 ms an iteration, the call from 262 to 151 ms (with the gather over
+// many CTAs), and to 119 ms with the update over many CTAs.
 template <int DP>
 struct BMma {
     static constexpr int W = DP <= 16 ? 8 : DP <= 32 ? 16 : 12;      // warps
@@ -980,9 +984,25 @@ int launch_class(int dc, TileShape sh, BatchInst* insts, const WorkItem* items, 
 std::mutex g_tune_mu;
 // dimension class -> (tile shape, tiles per work item)
 std::map<int, std::pair<TileShape, int>> g_tuned;
-// dimension class -> tiles per work item of the screen where it is faster than the
-// class's CUDA-core shape (0: it is not)
-std::map<int, int> g_tuned_mma;
+
+// Resident CTAs per SM of the screen's kernel for a dimension class.
+int mma_ctas(int dc) { return dc <= 16 ? BMma<16>::MINB : 1; }
+
+// Tiles per work item of the screen's kernel: as many as leave each CTA four items or
+// more, at most eight.  The centers of a job are loaded per item, so long lists
+// take large items, and short ones would leave CTAs idle with them.  ms a call with
+// items of 1, 2, 4, 8 tiles: 64 instances (n 1e3 .. 1e6, d 2 .. 64) 59.0, 55.9, 54.2, 56.5
+// (by this rule 55.1); 40 jobs of 1e3 .. 1.5e6 x 64 261, 246, 236, 235; 1e6 x 8 8.07, 8.68,
+// 9.53, 10.8; 1e6 x 16 9.24, 9.87, 11.1, 12.6.  A rule on the call's own sizes: timed once per
+// process and class, the last ran with 4 tiles after a batch of many jobs.
+int mma_tiles_per_item(const std::vector<int>& members, const std::vector<long long>& n, long long ctas)
+{
+    long long tiles = 0;
+    for (int j : members) tiles += (n[j] + kTile - 1) / kTile;
+    int p = 8;
+    while (p > 1 && tiles < 4 * p * ctas) p /= 2;
+    return p;
+}
 
 // Six dimension classes, each split in jobs the screen takes and others.
 constexpr int kMaxClasses = 12;
@@ -1168,28 +1188,20 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
             TileShape shape = forced_tile_shape(ci.dc);
             const bool forced_mma = shape.p == kMmaShape;
             const bool forced = shape.p > 0 || forced_mma;
-            int mma_tpi = forced || !mma_ok ? 0 : -1;     // -1: not tuned yet
             if (forced) {
                 tpi = 2;
-                if (forced_mma) {
-                    shape = tile_shapes(ci.dc)[0];
-                    mma_tpi = mma_ok ? 2 : 0;
-                }
+                if (forced_mma) shape = tile_shapes(ci.dc)[0];
             } else {
                 std::lock_guard<std::mutex> lock(g_tune_mu);
                 auto f = g_tuned.find(ci.dc);
                 if (f != g_tuned.end()) { shape = f->second.first; tpi = f->second.second; }
-                auto m = g_tuned_mma.find(ci.dc);
-                if (mma_tpi < 0 && m != g_tuned_mma.end()) mma_tpi = m->second;
             }
-            if (tpi == 0 || mma_tpi < 0) {
+            if (tpi == 0) {
                 // time the real first pass and a delta pass after it for each
                 // tile shape and item size (tiles per work item), resetting the
                 // sums between trials: small items keep every SM busy once only a
                 // few jobs still run, more point slots per lane reuse each center
-                // load more often.  The delta pass counts ten times where the
-                // screen is compared: its full pass, with the sums, is no measure
-                // of the iterations that follow.
+                // load more often
                 const int cand[4] = {1, 2, 4, 8};
                 static_assert(8 <= kMaxTilesPerItem, "item partial sums must stay below 2^62");
                 cudaEvent_t e0, e1, e2, e3;
@@ -1197,55 +1209,43 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                 KM2_CUDA(cudaEventCreate(&e1));
                 KM2_CUDA(cudaEventCreate(&e2));
                 KM2_CUDA(cudaEventCreate(&e3));
-                auto trial = [&](const TileShape& sh, int tiles, float& full, float& later) -> int {
-                    ClassItems tr;
-                    build_items(tr, kv.second, nvec, tiles);
-                    KM2_TRY(ws.alloc((void**)&tr.dev, sizeof(WorkItem) * (size_t)tr.count, s));
-                    KM2_CUDA(cudaMemcpyAsync(tr.dev, tr.host.data(), sizeof(WorkItem) * (size_t)tr.count,
-                                             cudaMemcpyHostToDevice, s));
-                    // the full first pass, then a delta pass over the labels it
-                    // wrote (same centers: no label moves), which is what the
-                    // later iterations of a fit cost
-                    KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
-                    KM2_CUDA(cudaEventRecord(e0, s));
-                    KM2_TRY(launch_class(ci.dc, sh, dinst, tr.dev, tr.count, counters + 2, s, ws.sm_count));
-                    KM2_CUDA(cudaEventRecord(e1, s));
-                    g_launches += 2;
-                    batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
-                    batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-                        dinst, count, kModeDelta);
-                    KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
-                    KM2_CUDA(cudaEventRecord(e2, s));
-                    KM2_TRY(launch_class(ci.dc, sh, dinst, tr.dev, tr.count, counters + 2, s, ws.sm_count));
-                    KM2_CUDA(cudaEventRecord(e3, s));
-                    g_launches += 2;
-                    batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
-                    batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-                        dinst, count, kModeFull);
-                    KM2_CUDA(cudaEventSynchronize(e3));
-                    KM2_CUDA(cudaEventElapsedTime(&full, e0, e1));
-                    KM2_CUDA(cudaEventElapsedTime(&later, e2, e3));
-                    return KMEANS2_OK;
-                };
-                float core_full = 0.f, core_later = 0.f, full = 0.f, later = 0.f;
-                if (tpi == 0) {
-                    bool first = true;
-                    for (const TileShape& sh : tile_shapes(ci.dc))
-                        for (int c : cand) {
-                            KM2_TRY(trial(sh, c, full, later));
-                            if (first || full + later < core_full + core_later) {
-                                core_full = full; core_later = later; tpi = c; shape = sh; first = false;
-                            }
-                        }
-                } else if (mma_tpi < 0) {
-                    KM2_TRY(trial(shape, tpi, core_full, core_later));
-                }
-                if (mma_tpi < 0) {
-                    float best = core_full + 10.f * core_later;
-                    mma_tpi = 0;
-                    for (int c : cand) {
-                        KM2_TRY(trial(TileShape{kMmaShape, 0}, c, full, later));
-                        if (full + 10.f * later < best) { best = full + 10.f * later; mma_tpi = c; }
+                float best_ms = 0.f;
+                bool first = true;
+                for (const TileShape& sh : tile_shapes(ci.dc)) {
+                    for (int c = 0; c < 4; ++c) {
+                        ClassItems trial;
+                        build_items(trial, kv.second, nvec, cand[c]);
+                        KM2_TRY(ws.alloc((void**)&trial.dev, sizeof(WorkItem) * (size_t)trial.count, s));
+                        KM2_CUDA(cudaMemcpyAsync(trial.dev, trial.host.data(),
+                                                 sizeof(WorkItem) * (size_t)trial.count,
+                                                 cudaMemcpyHostToDevice, s));
+                        // the full first pass, then a delta pass over the labels it
+                        // wrote (same centers: no label moves), which is what the
+                        // later iterations of a fit cost
+                        KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
+                        KM2_CUDA(cudaEventRecord(e0, s));
+                        KM2_TRY(launch_class(ci.dc, sh, dinst, trial.dev, trial.count, counters + 2,
+                                             s, ws.sm_count));
+                        KM2_CUDA(cudaEventRecord(e1, s));
+                        g_launches += 2;
+                        batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
+                        batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+                            dinst, count, kModeDelta);
+                        KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
+                        KM2_CUDA(cudaEventRecord(e2, s));
+                        KM2_TRY(launch_class(ci.dc, sh, dinst, trial.dev, trial.count, counters + 2,
+                                             s, ws.sm_count));
+                        KM2_CUDA(cudaEventRecord(e3, s));
+                        g_launches += 2;
+                        batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
+                        batch_mode_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+                            dinst, count, kModeFull);
+                        KM2_CUDA(cudaEventSynchronize(e3));
+                        float ms = 0.f, ms2 = 0.f;
+                        KM2_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+                        KM2_CUDA(cudaEventElapsedTime(&ms2, e2, e3));
+                        ms += ms2;
+                        if (first || ms < best_ms) { best_ms = ms; tpi = cand[c]; shape = sh; first = false; }
                     }
                 }
                 cudaEventDestroy(e0);
@@ -1254,11 +1254,10 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                 cudaEventDestroy(e3);
                 std::lock_guard<std::mutex> lock(g_tune_mu);
                 g_tuned[ci.dc] = std::make_pair(shape, tpi);
-                if (mma_ok) g_tuned_mma[ci.dc] = mma_tpi;
             }
-            if (mma_tpi > 0) {
+            if (mma_ok && (!forced || forced_mma)) {
                 shape = TileShape{kMmaShape, 0};
-                tpi = mma_tpi;
+                tpi = mma_tiles_per_item(kv.second, nvec, (long long)ws.sm_count * mma_ctas(ci.dc));
                 settle32 = settle32 || ci.dc == 32;
                 settle64 = settle64 || ci.dc == 64;
             }
