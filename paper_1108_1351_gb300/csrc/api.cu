@@ -302,7 +302,7 @@ int launch_stage_recheck(const float* X, int d, Workspace& w, int* labels, cudaS
 // / 22.5 ms at 0.035, 33.0 / 26.8 at 0.081; d = 32, k = 200 16.7 / 21.8 ms at 0.30-0.46,
 // 35.1 / 26.2 at 0.86; d = 64, k = 200 21.3 / 36.5 at 0.17-0.36, 41.1 / 39.5 at 0.49-0.60.
 // Above d = 16 the recheck decides open rows over the whole GPU, hence the two lines.
-constexpr double kMaxOpenNarrow = 0.04, kMaxOpenWide = 0.5;
+constexpr double kMaxOpenWide = 0.5;
 
 void review_screen(Workspace& w, int d, const StageState& st, long long rows, int passes)
 {

@@ -230,6 +230,9 @@ int launch_assign(const float* X, long long n, int d, Workspace& w, int* labels,
 // The FP64 recheck of the rows that launch_assign listed.
 int launch_stage_recheck(const float* X, int d, Workspace& w, int* labels, cudaStream_t s,
                          int sm_count);
+// Share of rows left open up to which the screen is kept for d <= 16 (both sides
+// measured: api.cu).
+constexpr double kMaxOpenNarrow = 0.04;
 // After a stage's first `passes` passes over `rows` rows (st: the state then): whether
 // the later ones keep the screen.
 void review_screen(Workspace& w, int d, const StageState& st, long long rows, int passes);

@@ -70,6 +70,7 @@ struct BatchInst {
     int d, k, max_iter;
     int stage;               // 0 fast, 1 slow, 2 done
     int settles;             // its distance kernel leaves open rows to the recheck's FP32 pass
+    int core;                // the screen left too many rows open: on CUDA cores from here on
     unsigned int maxabs_x;   // max |x| over X (scale of the slow stage)
     int iters_fast, conv_fast, error;
     double shift_fast;
@@ -249,7 +250,7 @@ __device__ __forceinline__ void group_reduce(float (&a)[P])
 
 template <int DC, int PP, int GG>
 __global__ void __launch_bounds__(kThreads, 2)
-batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
+batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item, const int* ncore)
 {
     using C = BCfg<DC, PP, GG>;
     constexpr int P = C::P, G = C::G, R = C::R, DG = C::DG;
@@ -263,6 +264,7 @@ batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item
     const int tid = threadIdx.x;
     const int q = tid % G;                   // lane within its group
     const int gi = tid / G;                  // group
+    if (ncore && *ncore == 0) return;        // beside the screen: the jobs that left it
     // ||c||^2 enters each point's sum through lane 0 of its group
     const float own0 = q == 0 ? 1.0f : 0.0f;
 
@@ -277,7 +279,7 @@ batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item
         const WorkItem w = items[it];
         BatchInst* I = insts + w.inst;
         const int stage = I->stage;
-        if (stage >= 2) continue;
+        if (stage >= 2 || (ncore && !I->core)) continue;
         const long long npts = stage == 0 ? I->m : I->n;
         const long long tiles = (npts + kTile - 1) / kTile;
         if (w.tile0 >= tiles) continue;
@@ -549,7 +551,7 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
     long long* sacc = reinterpret_cast<long long*>(stages + W * B::STAGE);   // k x DP
     int* scnt = reinterpret_cast<int*>(sacc + (size_t)kMaxK * DP);
     __shared__ unsigned long long sq[4];     // this item's sum of s^2 (wide_add4 words)
-    __shared__ int s_item;
+    __shared__ int s_item, s_open;           // rows left open (DP <= 16)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     unsigned char* stage_mem = stages + warp * B::STAGE;
     const unsigned stage_u32 = smem_u32(stage_mem);
@@ -564,7 +566,7 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
         const WorkItem w = items[it];
         BatchInst* I = insts + w.inst;
         const int stage = I->stage;
-        if (stage >= 2) continue;
+        if (stage >= 2 || (DP <= 16 && I->core)) continue;
         const long long npts = stage == 0 ? I->m : I->n;
         const long long tiles = (npts + kTile - 1) / kTile;
         if (w.tile0 >= tiles) continue;
@@ -585,6 +587,7 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
             for (int e = tid; e < k; e += kT) scnt[e] = 0;
         }
         if (tid < 4) sq[tid] = 0;
+        if (tid == 4) s_open = 0;
         __syncthreads();
 
         const long long row_begin = (long long)w.tile0 * kTile;
@@ -630,6 +633,7 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
                 bool listed = open;
                 if constexpr (DP <= 16) {
                     listed = false;
+                    if (lane == 0) atomicAdd(&s_open, __popc(todo));
                     if (__popc(todo) >= lanes) {
                         const int l = decide_fp32_lanes<DP, DP == 8>(X + (row0 + min(r, rows - 1)) * d, d,
                                                                      c.cnorm, c.c32t, c.kpad, k, thr_base);
@@ -716,6 +720,7 @@ batch_mma(BatchInst* insts, const WorkItem* items, int nitems, int* next_item)
                 if (scnt[j]) atomicAdd(I->acc.cnt + j, (unsigned long long)(long long)scnt[j]);
         }
         if (tid < 4 && sq[tid]) atomicAdd(&st->q[tid], sq[tid]);
+        if (tid == 4 && s_open) atomicAdd(&st->open_rows, (unsigned long long)s_open);
         __syncthreads();   // the next item reuses shared memory
     }
 }
@@ -783,7 +788,8 @@ __global__ void __launch_bounds__(kThreads) batch_recheck_flat_kernel(BatchInst*
 // last CTA reduces and moves the job on.  FP64 bound like finalize_kernel: with one
 // CTA per job a k = 256, d = 64 job held an SM for 200 us an iteration, 41 of the 151
 // ms of a batch of 64.
-__global__ void __launch_bounds__(kThreads) batch_finalize_kernel(BatchInst* insts, int* active)
+// ncore: jobs that left the screen, or null where nothing else would run them.
+__global__ void __launch_bounds__(kThreads) batch_finalize_kernel(BatchInst* insts, int* active, int* ncore)
 {
     __shared__ FinalizeSmem sm;
     __shared__ int switched, last;
@@ -820,6 +826,17 @@ __global__ void __launch_bounds__(kThreads) batch_finalize_kernel(BatchInst* ins
     finalize_reduce_block(I->k, I->acc.cnt, &I->st, TrajDev{nullptr, nullptr, nullptr, nullptr}, I->clus, sm);
     if (threadIdx.x == 0) {
         switched = 0;
+        if (I->st.open_rows) {
+            // as review_screen does (d <= 16; wider jobs count none: they were faster with
+            // the screen at any share, 1e6 x 64, k = 100, every row open, 37.1 ms against
+            // 51.3).  1e6 x 8, k = 100 at an offset of 1000, 80 iterations, ms with the
+            // screen throughout and on CUDA cores: 34.3, 29.8
+            if (ncore && !I->core && (double)I->st.open_rows > kMaxOpenNarrow * (double)(stage == 0 ? I->m : I->n)) {
+                I->core = 1;
+                atomicAdd(ncore, 1);
+            }
+            I->st.open_rows = 0;
+        }
         if (I->st.done) {
             I->rechecked += I->st.rechecked_total;
             if (stage == 0) {
@@ -885,7 +902,7 @@ int dclass(int d)
 
 template <int DC, int P, int G>
 int launch_batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int* next_item,
-                        cudaStream_t s, int sm_count)
+                        const int* ncore, cudaStream_t s, int sm_count)
 {
     const size_t sm = batch_smem<DC>();
     KM2_TRY(set_max_dynamic_smem((const void*)batch_assign<DC, P, G>, (int)sm));
@@ -897,7 +914,7 @@ int launch_batch_assign(BatchInst* insts, const WorkItem* items, int nitems, int
     if (grid > nitems) grid = nitems;
     if (grid < 1) grid = 1;
     ++g_launches;
-    batch_assign<DC, P, G><<<(int)grid, kThreads, sm, s>>>(insts, items, nitems, next_item);
+    batch_assign<DC, P, G><<<(int)grid, kThreads, sm, s>>>(insts, items, nitems, next_item, ncore);
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }
@@ -961,8 +978,9 @@ TileShape forced_tile_shape(int dc)
     return TileShape{};
 }
 
+// ncore: only the jobs that left the screen, if there are any (null: every job).
 int launch_class(int dc, TileShape sh, BatchInst* insts, const WorkItem* items, int nitems,
-                 int* next_item, cudaStream_t s, int sm_count)
+                 int* next_item, const int* ncore, cudaStream_t s, int sm_count)
 {
     if (sh.p == kMmaShape) {
         if (dc == 8) return launch_batch_mma<8>(insts, items, nitems, next_item, s, sm_count);
@@ -972,7 +990,7 @@ int launch_class(int dc, TileShape sh, BatchInst* insts, const WorkItem* items, 
     }
 #define KM2_BA(DD, PP, GG)                                                                  \
     if (dc == DD && sh.p == PP && sh.g == GG)                                               \
-        return launch_batch_assign<DD, PP, GG>(insts, items, nitems, next_item, s, sm_count);
+        return launch_batch_assign<DD, PP, GG>(insts, items, nitems, next_item, ncore, s, sm_count);
     KM2_BA(2, 2, 1) KM2_BA(2, 4, 1) KM2_BA(4, 2, 1) KM2_BA(4, 4, 1) KM2_BA(8, 2, 1)
     KM2_BA(8, 4, 1) KM2_BA(16, 2, 1) KM2_BA(16, 4, 1) KM2_BA(32, 1, 1) KM2_BA(32, 2, 1)
     KM2_BA(32, 4, 2) KM2_BA(32, 4, 4) KM2_BA(64, 1, 1) KM2_BA(64, 2, 2) KM2_BA(64, 4, 4)
@@ -1004,13 +1022,15 @@ int mma_tiles_per_item(const std::vector<int>& members, const std::vector<long l
     return p;
 }
 
-// Six dimension classes, each split in jobs the screen takes and others.
-constexpr int kMaxClasses = 12;
+// Six dimension classes, each split in jobs the screen takes and others, and for the
+// classes up to 16 the jobs that leave it.
+constexpr int kMaxClasses = 14;
 
 struct ClassItems {
     int dc = 0;
     TileShape shape;
     int tpi = 0;
+    bool left = false;               // the jobs that leave the screen of the class before
     std::vector<WorkItem> host;
     WorkItem* dev = nullptr;
     int count = 0;
@@ -1116,8 +1136,9 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
         int* counters = nullptr;
         KM2_TRY(ws.alloc((void**)&arena, total, s));
         KM2_TRY(ws.alloc((void**)&dinst, sizeof(BatchInst) * (size_t)count, s));
-        // active, iteration, an item counter per class, active count handed to the host
-        KM2_TRY(ws.alloc((void**)&counters, (kMaxClasses + 3) * sizeof(int), s));
+        // active, iteration, an item counter per class, active count handed to the
+        // host, jobs that left the screen
+        KM2_TRY(ws.alloc((void**)&counters, (kMaxClasses + 4) * sizeof(int), s));
         long long* rprefix = nullptr;      // flat recheck list: per-job offsets, total
         KM2_TRY(ws.alloc((void**)&rprefix, sizeof(long long) * ((size_t)count + 1), s));
         for (int j = 0; j < count; ++j) {
@@ -1161,7 +1182,7 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
         }
         KM2_CUDA(cudaMemcpyAsync(dinst, hi.data(), sizeof(BatchInst) * (size_t)count,
                                  cudaMemcpyHostToDevice, s));
-        KM2_CUDA(cudaMemsetAsync(counters, 0, (kMaxClasses + 3) * sizeof(int), s));
+        KM2_CUDA(cudaMemsetAsync(counters, 0, (kMaxClasses + 4) * sizeof(int), s));
         g_launches += 3;
         batch_sample_kernel<<<count, kSampleThreads, 0, s>>>(dinst);
         // finalize: centers over up to 32 CTAs per job while the jobs leave SMs idle
@@ -1225,7 +1246,7 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                         KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
                         KM2_CUDA(cudaEventRecord(e0, s));
                         KM2_TRY(launch_class(ci.dc, sh, dinst, trial.dev, trial.count, counters + 2,
-                                             s, ws.sm_count));
+                                             nullptr, s, ws.sm_count));
                         KM2_CUDA(cudaEventRecord(e1, s));
                         g_launches += 2;
                         batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
@@ -1234,7 +1255,7 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                         KM2_CUDA(cudaMemsetAsync(counters + 2, 0, sizeof(int), s));
                         KM2_CUDA(cudaEventRecord(e2, s));
                         KM2_TRY(launch_class(ci.dc, sh, dinst, trial.dev, trial.count, counters + 2,
-                                             s, ws.sm_count));
+                                             nullptr, s, ws.sm_count));
                         KM2_CUDA(cudaEventRecord(e3, s));
                         g_launches += 2;
                         batch_reset_kernel<<<count, kThreads, 0, s>>>(dinst);
@@ -1255,7 +1276,9 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
                 std::lock_guard<std::mutex> lock(g_tune_mu);
                 g_tuned[ci.dc] = std::make_pair(shape, tpi);
             }
-            if (mma_ok && (!forced || forced_mma)) {
+            const bool screened = mma_ok && (!forced || forced_mma);
+            const TileShape core_shape = shape;
+            if (screened) {
                 shape = TileShape{kMmaShape, 0};
                 tpi = mma_tiles_per_item(kv.second, nvec, (long long)ws.sm_count * mma_ctas(ci.dc));
                 settle32 = settle32 || ci.dc == 32;
@@ -1267,7 +1290,24 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
             KM2_CUDA(cudaMemcpyAsync(ci.dev, ci.host.data(), sizeof(WorkItem) * (size_t)ci.count,
                                      cudaMemcpyHostToDevice, s));
             classes.push_back(std::move(ci));
+            if (screened && !forced && kv.first / 2 <= 16) {
+                ClassItems lc;
+                lc.dc = kv.first / 2;
+                lc.shape = core_shape;
+                lc.left = true;
+                lc.dev = classes.back().dev;
+                lc.count = classes.back().count;
+                lc.tpi = tpi;
+                classes.push_back(std::move(lc));
+            }
         }
+        // jobs that have left the screen: counted in the first iteration, before which
+        // there are none; their kernels run beside the screen's only if there are some
+        // (idle ones cost an iteration 3 us), else every job stays
+        int* ncore = nullptr;
+        for (const ClassItems& ci : classes)
+            if (ci.left) ncore = counters + 3 + kMaxClasses;
+        bool run_left = false;
 
         if (settle32 || settle64) {
             ++g_launches;
@@ -1295,59 +1335,35 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
         auto launch_classes = [&]() -> int {
             if (cudaEventRecord(fork, s) != cudaSuccess) return KMEANS2_ERR_CUDA;
             for (size_t c = 0; c < classes.size(); ++c) {
+                if (classes[c].left && !run_left) continue;
                 if (cudaStreamWaitEvent(side[c], fork, 0) != cudaSuccess) return KMEANS2_ERR_CUDA;
                 const int r = launch_class(classes[c].dc, classes[c].shape, dinst, classes[c].dev,
-                                           classes[c].count,
-                                           counters + 2 + c, side[c], ws.sm_count);
+                                           classes[c].count, counters + 2 + c,
+                                           classes[c].left ? ncore : nullptr, side[c], ws.sm_count);
                 if (r != KMEANS2_OK) return r;
                 if (cudaEventRecord(joins[c], side[c]) != cudaSuccess) return KMEANS2_ERR_CUDA;
                 if (cudaStreamWaitEvent(s, joins[c], 0) != cudaSuccess) return KMEANS2_ERR_CUDA;
             }
             return KMEANS2_OK;
         };
+        auto launched_classes = [&]() {
+            long long c = 0;
+            for (const ClassItems& ci : classes) c += !ci.left || run_left;
+            return c;
+        };
+        auto launch_update = [&]() {
+            batch_recheck_scan_kernel<<<1, 1024, 0, s>>>(dinst, count, rprefix);
+            batch_recheck_flat_kernel<<<ws.sm_count * 4, kThreads, 0, s>>>(dinst, count, rprefix);
+            batch_finalize_kernel<<<dim3((unsigned)count, (unsigned)fslices), kThreads, 0, s>>>(dinst, counters, ncore);
+        };
         const int cap = 2 * max_iter_all + 2;
-        if (o.profile) {
-            // ---- profiled: host-driven loop, CUDA events around each iteration's
-            // distance kernels (every kernel is then visible to profilers)
-            cudaEvent_t e0 = nullptr, e1 = nullptr;
-            cudaEventCreate(&e0);
-            cudaEventCreate(&e1);
-            for (int it = 0; it < cap && rc == KMEANS2_OK; ++it) {
-                cudaEventRecord(e0, s);
-                rc = launch_classes();
-                if (rc != KMEANS2_OK) break;
-                cudaEventRecord(e1, s);
-                g_launches += 2;
-                batch_recheck_scan_kernel<<<1, 1024, 0, s>>>(dinst, count, rprefix);
-                batch_recheck_flat_kernel<<<ws.sm_count * 4, kThreads, 0, s>>>(dinst, count, rprefix);
-                ++g_launches;
-                batch_finalize_kernel<<<dim3((unsigned)count, (unsigned)fslices), kThreads, 0, s>>>(dinst, counters);
-                ++g_launches;
-                batch_step_kernel<<<1, 1, 0, s>>>(counters, counters + 1, counters + 2,
-                                                  (int)classes.size(), counters + 2 + kMaxClasses);
-                int active = 0;
-                cudaError_t e = cudaMemcpyAsync(&active, counters + 2 + kMaxClasses, sizeof(int),
-                                                cudaMemcpyDeviceToHost, s);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-                if (e != cudaSuccess) { set_last_error("batched loop", e); rc = KMEANS2_ERR_CUDA; break; }
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                o.profile->assign_launches += (long long)classes.size();
-                o.profile->assign_ms += ms;
-                if (active == 0) break;
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-        }
         // ---- the iteration loop as one graph with a device-side while condition
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
-        if (!o.profile) KM2_CUDA(cudaGraphCreate(&graph, 0));
-        do {
-            if (o.profile) break;
+        auto build_graph = [&]() -> int {
+            KM2_CUDA(cudaGraphCreate(&graph, 0));
             cudaGraphConditionalHandle handle;
-            cudaError_t e = cudaGraphConditionalHandleCreate(&handle, graph, 1u, cudaGraphCondAssignDefault);
-            if (e != cudaSuccess) { set_last_error("cudaGraphConditionalHandleCreate", e); rc = KMEANS2_ERR_CUDA; break; }
+            KM2_CUDA(cudaGraphConditionalHandleCreate(&handle, graph, 1u, cudaGraphCondAssignDefault));
             alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
             std::memset(raw, 0, sizeof(raw));
             cudaGraphNodeParams* gp = reinterpret_cast<cudaGraphNodeParams*>(raw);
@@ -1356,39 +1372,96 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
             gp->conditional.type = cudaGraphCondTypeWhile;
             gp->conditional.size = 1;
             cudaGraphNode_t node;
-            e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, gp);
-            if (e != cudaSuccess) { set_last_error("cudaGraphAddNode", e); rc = KMEANS2_ERR_CUDA; break; }
+            KM2_CUDA(cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, gp));
             cudaGraph_t body = gp->conditional.phGraph_out[0];
-            e = cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-            if (e != cudaSuccess) { set_last_error("cudaStreamBeginCaptureToGraph", e); rc = KMEANS2_ERR_CUDA; break; }
-            rc = launch_classes();
-            if (rc == KMEANS2_OK) {
-                batch_recheck_scan_kernel<<<1, 1024, 0, s>>>(dinst, count, rprefix);
-                batch_recheck_flat_kernel<<<ws.sm_count * 4, kThreads, 0, s>>>(dinst, count, rprefix);
-                batch_finalize_kernel<<<dim3((unsigned)count, (unsigned)fslices), kThreads, 0, s>>>(dinst, counters);
+            KM2_CUDA(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+            const long long l0 = g_launches;
+            const int r = launch_classes();
+            g_launches = l0;                             // counted by iterations below
+            if (r == KMEANS2_OK) {
+                launch_update();
                 batch_control_kernel<<<1, 1, 0, s>>>(counters, counters + 1, counters + 2,
-                                                     (int)classes.size(), cap,
-                                                     (unsigned long long)handle);
+                                                     (int)classes.size(), cap, (unsigned long long)handle);
             }
             cudaGraph_t captured = nullptr;
-            e = cudaStreamEndCapture(s, &captured);
-            if (rc != KMEANS2_OK) break;
-            if (e != cudaSuccess) { set_last_error("cudaStreamEndCapture", e); rc = KMEANS2_ERR_CUDA; break; }
-            e = cudaGraphInstantiate(&exec, graph, 0);
-            if (e != cudaSuccess) { set_last_error("cudaGraphInstantiate", e); rc = KMEANS2_ERR_CUDA; break; }
-            e = cudaGraphLaunch(exec, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e != cudaSuccess) { set_last_error("batched graph", e); rc = KMEANS2_ERR_CUDA; break; }
-        } while (0);
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
+            const cudaError_t e = cudaStreamEndCapture(s, &captured);
+            if (r != KMEANS2_OK) return r;
+            if (e != cudaSuccess) { set_last_error("cudaStreamEndCapture", e); return KMEANS2_ERR_CUDA; }
+            KM2_CUDA(cudaGraphInstantiate(&exec, graph, 0));
+            return KMEANS2_OK;
+        };
+        auto destroy_graph = [&]() {
+            if (exec) cudaGraphExecDestroy(exec);
+            if (graph) cudaGraphDestroy(graph);
+            exec = nullptr;
+            graph = nullptr;
+        };
+        // iterations from the host: the first one where jobs may leave the screen (the
+        // graph is built meanwhile, again if some did), and all of a profiled call,
+        // with CUDA events around the distance kernels (every kernel is then visible
+        // to profilers)
+        int host_iters = 0, active = 1;
+        int* const count_left = ncore;
+        if (o.profile || ncore) {
+            cudaEvent_t e0 = nullptr, e1 = nullptr;
+            if (o.profile) {
+                cudaEventCreate(&e0);
+                cudaEventCreate(&e1);
+            }
+            while (host_iters < (o.profile ? cap : 1)) {
+                if (o.profile) cudaEventRecord(e0, s);
+                rc = launch_classes();
+                if (rc != KMEANS2_OK) break;
+                if (o.profile) cudaEventRecord(e1, s);
+                g_launches += 4;
+                launch_update();
+                batch_step_kernel<<<1, 1, 0, s>>>(counters, counters + 1, counters + 2,
+                                                  (int)classes.size(), counters + 2 + kMaxClasses);
+                ++host_iters;
+                if (!o.profile) {
+                    ncore = nullptr;
+                    rc = build_graph();
+                    if (rc != KMEANS2_OK) break;
+                }
+                int out[2] = {0, 0};                     // jobs still running, jobs that left
+                cudaError_t e = cudaMemcpyAsync(out, counters + 2 + kMaxClasses, sizeof(out),
+                                                cudaMemcpyDeviceToHost, s);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+                if (e != cudaSuccess) { set_last_error("batched loop", e); rc = KMEANS2_ERR_CUDA; break; }
+                if (o.profile) {
+                    float ms = 0.f;
+                    cudaEventElapsedTime(&ms, e0, e1);
+                    o.profile->assign_launches += launched_classes();
+                    o.profile->assign_ms += ms;
+                }
+                active = out[0];
+                if (host_iters == 1 && count_left) {
+                    run_left = out[1] > 0;
+                    ncore = run_left ? count_left : nullptr;
+                    if (run_left) destroy_graph();
+                }
+                if (active == 0) break;
+            }
+            if (e0) cudaEventDestroy(e0);
+            if (e1) cudaEventDestroy(e1);
+        }
+        const bool use_graph = !o.profile && rc == KMEANS2_OK && active != 0;
+        if (use_graph) {
+            if (!exec) rc = build_graph();
+            if (rc == KMEANS2_OK) {
+                cudaError_t e = cudaGraphLaunch(exec, s);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+                if (e != cudaSuccess) { set_last_error("batched graph", e); rc = KMEANS2_ERR_CUDA; }
+            }
+        }
+        destroy_graph();
         cudaStreamSynchronize(s);
         destroy_side();
-        if (rc == KMEANS2_OK && !o.profile) {
+        if (rc == KMEANS2_OK && use_graph) {
             int iters = 0;
             KM2_CUDA(cudaMemcpyAsync(&iters, counters + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
             KM2_CUDA(cudaStreamSynchronize(s));
-            g_launches += (long long)iters * ((long long)classes.size() + 4);
+            g_launches += (long long)(iters - host_iters) * (launched_classes() + 4);
         }
         if (rc == KMEANS2_OK) {
             // ---- results

@@ -138,3 +138,26 @@ def test_batched_jobs_with_most_rows_open():
     r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % root + BATCH], capture_output=True,
                        text=True, env=env, timeout=600, cwd=root)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-3000:]
+
+
+def test_batched_jobs_leave_the_screen():
+    """A job whose first pass leaves too many rows open goes on with the CUDA-core
+    kernels, the others of the batch do not: a screen that stayed would list about a
+    third of the rows that the CUDA-core kernel's wider bound lists."""
+    jobs = [(200_000, 8, 32), (150_001, 12, 20), (100_000, 16, 100), (200_000, 8, 32), (50_000, 24, 30), (40_000, 4, 9)]
+    Xs = [synth.iso_gaussian_mixture(n, d, k, j, device="cuda") + (0.0 if j == 3 else 60.0)
+          for j, (n, d, k) in enumerate(jobs)]
+    Xs[0] += 60.0
+    ks = [k for _, _, k in jobs]
+    for _ in range(2):
+        rs, rc = km.fit_batched(Xs, ks, 0.3, list(range(len(jobs))), 1e-6, 25)
+        assert rc == 0
+        for j, (X, k, r) in enumerate(zip(Xs, ks, rs)):
+            a = km.fit(X, k, 0.3, j, 1e-6, 25, precision="fp32")
+            assert torch.equal(a.labels, r.labels) and torch.equal(a.centers, r.centers), jobs[j]
+            assert (a.J, a.iters_fast, a.iters_slow) == (r.J, r.iters_fast, r.iters_slow), jobs[j]
+            share = r.rechecked_points / max(1, a.rechecked_points)
+            if j == 0:
+                assert share > 0.8, (jobs[j], share)
+            if j == 3:
+                assert share < 0.7, (jobs[j], share)
