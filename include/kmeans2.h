@@ -435,7 +435,9 @@ typedef struct {
  * scratch, the BF16 copies when that form is chosen, the labels when the
  * caller's are not on the device, and a staged copy of X when x_on_host.
  * precision: as kmeans2_options.precision (AUTO resolves as kmeans2_fit does
- * for 16-byte aligned device X).  Returns 0 for invalid arguments.
+ * for 16-byte aligned device X).  Returns 0 for invalid arguments.  For d >= 64
+ * in the 16-bit forms it counts up to 100 MB of scratch (the list of moved rows)
+ * that a fit gives back, and a server admits a job without, where memory is short.
  */
 KMEANS2_API uint64_t kmeans2_fit_footprint(int64_t n, int32_t d, int32_t k,
                                            double subset_fraction, int32_t max_iter,

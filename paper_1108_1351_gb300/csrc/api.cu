@@ -131,6 +131,17 @@ cudaError_t pool_malloc_async(void** p, size_t bytes, cudaStream_t s)
     return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
 }
 
+// Debug builds (KM2_DEBUG_CHECKS) let a call have at most KMEANS2_DEBUG_SCRATCH_BYTES
+// bytes of scratch when that is set, so that a test can make memory run out.
+static size_t scratch_limit()
+{
+#ifdef KM2_DEBUG_CHECKS
+    const char* v = std::getenv("KMEANS2_DEBUG_SCRATCH_BYTES");
+    if (v && *v) return (size_t)std::strtoull(v, nullptr, 10);
+#endif
+    return ~(size_t)0;
+}
+
 DeviceScratch::DeviceScratch(cudaStream_t s) : stream(s)
 {
     cudaGetDevice(&device);
@@ -165,7 +176,22 @@ int DeviceScratch::alloc(void** p, size_t bytes, cudaStream_t s)
         return KMEANS2_OK;
     }
     cudaMemPool_t pool = library_pool(device);
-    cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+    auto get = [&]() -> cudaError_t {
+        if (used + bytes > scratch_limit()) return cudaErrorMemoryAllocation;
+        return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+    };
+    cudaError_t e = get();
+    if (e == cudaErrorMemoryAllocation && spare) {
+        cudaGetLastError();
+        *spare = MovedRows{};
+        spare = nullptr;
+        ptrs.erase(std::find(ptrs.begin(), ptrs.end(), spare_ptr));
+        used -= spare_bytes;
+        cudaFreeAsync(spare_ptr, s);
+        cudaStreamSynchronize(s);
+        if (pool) cudaMemPoolTrimTo(pool, 0);
+        e = get();
+    }
     if (e != cudaSuccess) {
         set_last_error("cudaMallocFromPoolAsync", e);
         cudaGetLastError();
@@ -173,7 +199,17 @@ int DeviceScratch::alloc(void** p, size_t bytes, cudaStream_t s)
         return KMEANS2_ERR_NOMEM;
     }
     ptrs.push_back(*p);
+    used += bytes;
     return KMEANS2_OK;
+}
+
+void DeviceScratch::alloc_spare(void** p, size_t bytes, MovedRows* owner, cudaStream_t s)
+{
+    *p = nullptr;
+    if (arena || bytes == 0 || alloc(p, bytes, s) != KMEANS2_OK) return;
+    spare = owner;
+    spare_ptr = *p;
+    spare_bytes = bytes;
 }
 
 // ---------------------------------------------------------------- stage plumbing
@@ -217,7 +253,6 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
     // one allocation, carved in 256-byte steps: a pool allocation and its release
     // cost the host 2 us, a dozen of them a fifth of a small step
     const size_t kd = (size_t)k * d;
-    w.mv.cap = tc16_form(w.form) && k <= kMovedMaxK ? (unsigned)std::min(list_cap, kMovedCap) : 0u;
     struct Piece { void** p; size_t bytes; };
     const Piece pieces[] = {
         {(void**)&w.c.c64, kd * sizeof(double)},
@@ -234,10 +269,6 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
         {(void**)&w.traj_shift, (size_t)max_iter * sizeof(double)},
         // (the split layout: a fit may switch from FP16 to split BF16 between stages)
         {(void**)&w.cb, tc16_form(w.form) ? bf16_cb_bytes(d, k, 0) : 0},
-        {(void**)&w.mv.moved, (size_t)w.mv.cap * sizeof(int2)},
-        {(void**)&w.mv.sorted, (size_t)w.mv.cap * 2 * sizeof(int2)},
-        {(void**)&w.mv.hist, w.mv.cap ? (size_t)k * 4 * sizeof(unsigned) : 0},
-        {(void**)&w.mv.state, w.mv.cap ? 2 * sizeof(unsigned) : 0},
     };
     size_t total = 0;
     for (const Piece& q : pieces) total += (q.bytes + 255) / 256 * 256;
@@ -248,10 +279,21 @@ int alloc_workspace(Workspace& w, DeviceScratch& ws, long long list_cap, int k, 
         *q.p = base;
         base += (q.bytes + 255) / 256 * 256;
     }
-    if (w.mv.cap) {
+    // an allocation of its own, which the call gives back where memory runs out: what
+    // fitted without the list has to fit still
+    const unsigned cap = tc16_form(w.form) && k <= kMovedMaxK && w.moved_rows && list_cap > 0
+                             ? (unsigned)std::min(list_cap, kMovedCap) : 0u;
+    const size_t hist = ((size_t)k * 4 * sizeof(unsigned) + 255) / 256 * 256;
+    const size_t rows = ((size_t)cap * sizeof(int2) + 255) / 256 * 256;
+    ws.alloc_spare((void**)&base, cap ? hist + 256 + 3 * rows : 0, &w.mv, s);
+    if (base) {
+        w.mv.hist = (unsigned*)base;
         w.mv.cur = w.mv.hist + 2 * (size_t)k;
-        KM2_CUDA(cudaMemsetAsync(w.mv.hist, 0, (size_t)k * 4 * sizeof(unsigned), s));
-        KM2_CUDA(cudaMemsetAsync(w.mv.state, 0, 2 * sizeof(unsigned), s));
+        w.mv.state = (unsigned*)(base + hist);
+        w.mv.moved = (int2*)(base + hist + 256);
+        w.mv.sorted = (int2*)(base + hist + 256 + rows);
+        w.mv.cap = cap;
+        KM2_CUDA(cudaMemsetAsync(base, 0, hist + 256, s));
     }
     return KMEANS2_OK;
 }
@@ -745,6 +787,15 @@ uint64_t kmeans2_fit_footprint(int64_t n, int32_t d, int32_t k, double subset_fr
                                int32_t max_iter, int32_t precision, int32_t x_on_host,
                                int32_t labels_on_host)
 {
+    return footprint_call(n, d, k, subset_fraction, max_iter, precision, x_on_host, labels_on_host, true);
+}
+
+}  // extern "C"
+
+uint64_t km2::footprint_call(int64_t n, int32_t d, int32_t k, double subset_fraction, int32_t max_iter,
+                             int32_t precision, int32_t x_on_host, int32_t labels_on_host,
+                             bool moved_rows)
+{
     if (!valid_shape(n, d, k) || !(subset_fraction > 0.0 && subset_fraction <= 1.0) ||
         max_iter < 1)
         return 0;
@@ -774,8 +825,8 @@ uint64_t kmeans2_fit_footprint(int64_t n, int32_t d, int32_t k, double subset_fr
     add(2 * (unsigned long long)max_iter * 8);
     if (tc16_form(form)) {
         add(bf16_cb_bytes(d, k, 0));
-        if (k <= kMovedMaxK) {       // moved rows, sorted
-            add(std::min<unsigned long long>(N, kMovedCap) * 24);
+        if (k <= kMovedMaxK && moved_rows) {       // moved rows, sorted
+            add(std::min<unsigned long long>(N, kMovedCap) * 24 + 768);
             add(K * 16 + 512);
         }
     }
@@ -829,6 +880,8 @@ uint64_t kmeans2_fit_footprint(int64_t n, int32_t d, int32_t k, double subset_fr
     }
     return b + (unsigned long long)allocs * 1024ull + (4ull << 20);
 }
+
+extern "C" {
 
 int32_t kmeans2_version(void) { return (1 << 16) | 0; }
 
@@ -996,6 +1049,7 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
     Workspace w;
     KM2_TRY(choose_form(o.precision, d, k, Xd, &w.form));
     w.screen = r.screen;
+    w.moved_rows = r.moved_rows;
     // AUTO on a 16-bit tensor-core shape: the fast stage runs the single-pass
     // FP16 form and the slow stage keeps it only if that left few rows
     // undecided there (on tie-heavy data its second pass and the FP64 recheck
@@ -1096,11 +1150,10 @@ int fit_on(const float* Xd, int64_t n, int32_t d, int32_t k, double subset_fract
 
 }  // namespace
 
-extern "C" {
-
-int kmeans2_fit(const float* X, int64_t n, int32_t d, int32_t k, double subset_fraction,
-                uint64_t seed, double tol, int32_t max_iter, double* centers_out,
-                int32_t* labels_out, kmeans2_result* res, const kmeans2_options* opt)
+int km2::fit_call(const float* X, int64_t n, int32_t d, int32_t k, double subset_fraction,
+                  uint64_t seed, double tol, int32_t max_iter, double* centers_out,
+                  int32_t* labels_out, kmeans2_result* res, const kmeans2_options* opt,
+                  bool moved_rows)
 {
     auto t0 = std::chrono::steady_clock::now();
     const long long launches0 = g_launches;
@@ -1108,6 +1161,7 @@ int kmeans2_fit(const float* X, int64_t n, int32_t d, int32_t k, double subset_f
         !(subset_fraction > 0.0 && subset_fraction <= 1.0) || !(tol >= 0.0) || max_iter < 1)
         return KMEANS2_ERR_INVALID;
     Resolved r = resolve_options(opt);
+    r.moved_rows = moved_rows;
     if (r.opt.start_stage != 0 && r.opt.start_stage != 1) return KMEANS2_ERR_INVALID;
     if (r.opt.start_stage == 1 && !r.opt.init_centers) return KMEANS2_ERR_INVALID;
     DeviceScratch ws(r.stream);
@@ -1117,7 +1171,12 @@ int kmeans2_fit(const float* X, int64_t n, int32_t d, int32_t k, double subset_f
                   r, ws, t0, launches0);
 }
 
-}  // extern "C"
+extern "C" int kmeans2_fit(const float* X, int64_t n, int32_t d, int32_t k, double subset_fraction,
+                           uint64_t seed, double tol, int32_t max_iter, double* centers_out,
+                           int32_t* labels_out, kmeans2_result* res, const kmeans2_options* opt)
+{
+    return fit_call(X, n, d, k, subset_fraction, seed, tol, max_iter, centers_out, labels_out, res, opt, true);
+}
 
 namespace {
 

@@ -47,6 +47,8 @@ cudaMemPool_t library_pool(int device);
 // cudaMallocAsync from the library pool of the current device.
 cudaError_t pool_malloc_async(void** p, size_t bytes, cudaStream_t s);
 
+struct MovedRows;
+
 // Stream-ordered scratch: every allocation is released (cudaFreeAsync on the
 // same stream) when the object goes out of scope.
 struct DeviceScratch {
@@ -61,10 +63,19 @@ struct DeviceScratch {
     size_t arena_bytes = 0;
     size_t arena_used = 0;
 
+    // An allocation that the call can do without: given back, and *spare emptied,
+    // before another one fails for lack of memory.
+    MovedRows* spare = nullptr;
+    void* spare_ptr = nullptr;
+    size_t spare_bytes = 0;
+    size_t used = 0;              // bytes allocated (debug builds limit them)
+
     explicit DeviceScratch(cudaStream_t s);
     DeviceScratch(cudaStream_t s, void* arena_base, size_t bytes);
     ~DeviceScratch();
     int alloc(void** p, size_t bytes, cudaStream_t s);
+    // alloc for MovedRows *owner, without an error if there is no room.
+    void alloc_spare(void** p, size_t bytes, MovedRows* owner, cudaStream_t s);
     DeviceScratch(const DeviceScratch&) = delete;
     DeviceScratch& operator=(const DeviceScratch&) = delete;
 };
@@ -129,7 +140,7 @@ int launch_assign_tc32(const float* X, long long n, int d, const Centers& c, int
 // moved.cu: rows whose label a pass changed, listed by the 16-bit distance kernels
 // and added to the sums by cluster afterwards.  The list holds at most kMovedCap
 // rows (100 MB of scratch); the distance kernel itself adds those past it, and all
-// of them where k is above kMovedMaxK (moved null).
+// of them where k is above kMovedMaxK or there was no room for the list (moved null).
 constexpr long long kMovedCap = 1ll << 22;
 constexpr int kMovedMaxK = 4096;
 struct MovedRows {
@@ -199,6 +210,7 @@ struct Workspace {
     int form = KMEANS2_PRECISION_FP32;   // distance-kernel form used by this call
     bool screen = false;                 // FP32 form: rows go through the tensor-core screen first
     bool first_pass = false;             // the stage's first passes, until review_screen
+    bool moved_rows = true;              // 16-bit forms: with the list of moved rows, if there is room
     Centers c{};
     Accum acc{};
     StageState* st = nullptr;
@@ -248,7 +260,15 @@ struct Resolved {
     cudaStream_t stream;
     kmeans2_options opt;
     bool screen;       // precision AUTO: the FP32 form may screen rows on the tensor cores
+    bool moved_rows = true;   // the 16-bit forms may list their moved rows (100 MB of scratch at most)
 };
 Resolved resolve_options(const kmeans2_options* opt);
+
+// kmeans2_fit and kmeans2_fit_footprint with or without that list.
+int fit_call(const float* X, int64_t n, int32_t d, int32_t k, double subset_fraction, uint64_t seed,
+             double tol, int32_t max_iter, double* centers_out, int32_t* labels_out,
+             kmeans2_result* res, const kmeans2_options* opt, bool moved_rows);
+uint64_t footprint_call(int64_t n, int32_t d, int32_t k, double subset_fraction, int32_t max_iter,
+                        int32_t precision, int32_t x_on_host, int32_t labels_on_host, bool moved_rows);
 
 }  // namespace km2

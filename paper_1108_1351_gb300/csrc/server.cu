@@ -44,7 +44,9 @@ struct Ticket {
     kmeans2_materialize_fn materialize = nullptr;   // lazy input (NULL: job.X given)
     kmeans2_consume_fn consume = nullptr;
     void* user = nullptr;
-    uint64_t footprint = 0;
+    // device bytes with and without the list of moved rows (api_internal.h), and those
+    // it runs with: a job is admitted without the list where only that fits
+    uint64_t footprint = 0, least = 0, charged = 0;
     double work = 0.0;          // n k d: the cost of one iteration
     JobState state = JobState::Queued;
     int status = KMEANS2_PENDING;
@@ -102,7 +104,7 @@ struct kmeans2_server {
         if (policy == KMEANS2_POLICY_SHORTEST) return pick_shortest();
         for (size_t i = 0; i < queue.size(); ++i) {
             km2::Ticket& t = tickets[queue[i]];
-            if (in_use + t.footprint <= budget) {
+            if (in_use + t.least <= budget) {
                 const uint64_t id = queue[i];
                 for (size_t j = 0; j < i; ++j) tickets[queue[j]].bypassed += 1;
                 queue.erase(queue.begin() + (long)i);
@@ -123,14 +125,14 @@ struct kmeans2_server {
         const uint64_t head = queue.front();
         km2::Ticket& h = tickets[head];
         if (t - h.times.t_submit >= aging_s) {
-            if (in_use + h.footprint > budget) return 0;
+            if (in_use + h.least > budget) return 0;
             queue.pop_front();
             return head;
         }
         size_t best = queue.size();
         for (size_t i = 0; i < queue.size(); ++i) {
             const km2::Ticket& c = tickets[queue[i]];
-            if (in_use + c.footprint > budget) continue;
+            if (in_use + c.least > budget) continue;
             if (best == queue.size() || c.work < tickets[queue[best]].work) best = i;
         }
         if (best == queue.size()) return 0;
@@ -148,6 +150,7 @@ struct kmeans2_server {
             kmeans2_materialize_fn materialize = nullptr;
             kmeans2_consume_fn consume = nullptr;
             void* user = nullptr;
+            bool moved_rows = true;
             {
                 std::unique_lock<std::mutex> lk(mu);
                 cv_work.wait(lk, [&] {
@@ -170,7 +173,9 @@ struct kmeans2_server {
                 km2::Ticket& t = tickets[id];
                 t.state = km2::JobState::Running;
                 t.times.t_admit = now();
-                in_use += t.footprint;
+                moved_rows = in_use + t.footprint <= budget;
+                t.charged = moved_rows ? t.footprint : t.least;
+                in_use += t.charged;
                 if (in_use > peak) peak = in_use;
                 ++running;
                 ++admitted;
@@ -186,10 +191,10 @@ struct kmeans2_server {
             const long long l0 = km2::g_launches;
             int rc = KMEANS2_OK;
             if (materialize)
-                rc = run_lazy(job, materialize, consume, user, o, &r);
+                rc = run_lazy(job, materialize, consume, user, o, moved_rows, &r);
             else
-                rc = kmeans2_fit(job.X, job.n, job.d, job.k, job.subset_fraction, job.seed,
-                                 job.tol, job.max_iter, job.centers_out, job.labels_out, &r, &o);
+                rc = km2::fit_call(job.X, job.n, job.d, job.k, job.subset_fraction, job.seed, job.tol,
+                                   job.max_iter, job.centers_out, job.labels_out, &r, &o, moved_rows);
             const long long dl = km2::g_launches - l0;
             {
                 std::lock_guard<std::mutex> lk(mu);
@@ -198,7 +203,7 @@ struct kmeans2_server {
                 t.status = rc;
                 t.res = r;
                 t.times.t_done = now();
-                in_use -= t.footprint;
+                in_use -= t.charged;
                 --running;
                 if (rc == KMEANS2_OK) ++completed; else ++failed;
                 launches += dl;
@@ -213,7 +218,7 @@ struct kmeans2_server {
     // stream, the caller's materialize, the fit, the caller's consume.
     int run_lazy(const kmeans2_job& job, kmeans2_materialize_fn materialize,
                  kmeans2_consume_fn consume, void* user, const kmeans2_options& o,
-                 kmeans2_result* r)
+                 bool moved_rows, kmeans2_result* r)
     {
         cudaStream_t s = static_cast<cudaStream_t>(o.stream);
         float* X = nullptr;
@@ -233,8 +238,8 @@ struct kmeans2_server {
             rc = KMEANS2_ERR_INVALID;
         }
         if (rc == KMEANS2_OK)
-            rc = kmeans2_fit(X, job.n, job.d, job.k, job.subset_fraction, job.seed, job.tol,
-                             job.max_iter, cen, lab, r, &o);
+            rc = km2::fit_call(X, job.n, job.d, job.k, job.subset_fraction, job.seed, job.tol,
+                               job.max_iter, cen, lab, r, &o, moved_rows);
         if (rc == KMEANS2_OK && consume) consume(user, cen, lab, o.stream);
         if (lab) cudaFreeAsync(lab, s);
         if (cen) cudaFreeAsync(cen, s);
@@ -314,17 +319,21 @@ int submit_common(kmeans2_server* srv, const kmeans2_job* job, kmeans2_materiali
     }
     const bool x_dev = lazy || km2::on_device(J.X, 16);
     const bool lab_dev = lazy || km2::on_device(J.labels_out, 4);
-    uint64_t fp = kmeans2_fit_footprint(J.n, J.d, J.k, J.subset_fraction, J.max_iter,
-                                        srv->opt.precision, x_dev ? 0 : 1, lab_dev ? 0 : 1);
-    if (fp == 0) {
+    uint64_t fp[2];                       // without the list of moved rows, with it
+    for (int l = 0; l < 2; ++l)
+        fp[l] = km2::footprint_call(J.n, J.d, J.k, J.subset_fraction, J.max_iter, srv->opt.precision,
+                                    x_dev ? 0 : 1, lab_dev ? 0 : 1, l != 0);
+    if (fp[0] == 0) {
         km2::set_last_error_text("kmeans2_server_submit: shape or precision not supported");
         return KMEANS2_ERR_INVALID;
     }
-    if (x_dev) fp += (uint64_t)J.n * (uint64_t)J.d * 4;   // resident data counts against the budget
-    if (lazy) fp += (uint64_t)J.k * (uint64_t)J.d * 8 + (uint64_t)J.n * 4;   // server-owned outputs
+    for (uint64_t& b : fp) {
+        if (x_dev) b += (uint64_t)J.n * (uint64_t)J.d * 4;   // resident data counts against the budget
+        if (lazy) b += (uint64_t)J.k * (uint64_t)J.d * 8 + (uint64_t)J.n * 4;   // server-owned outputs
+    }
     std::lock_guard<std::mutex> lk(srv->mu);
     if (srv->stop) return KMEANS2_ERR_ADMISSION;
-    if (fp > srv->budget) {
+    if (fp[0] > srv->budget) {
         ++srv->rejected;
         km2::set_last_error_text("kmeans2_server_submit: job footprint exceeds the HBM budget");
         return KMEANS2_ERR_ADMISSION;
@@ -335,7 +344,8 @@ int submit_common(kmeans2_server* srv, const kmeans2_job* job, kmeans2_materiali
     t.materialize = materialize;
     t.consume = consume;
     t.user = user;
-    t.footprint = fp;
+    t.least = fp[0];
+    t.footprint = fp[1];
     t.work = (double)J.n * (double)J.k * (double)J.d;
     t.times.t_submit = srv->now();
     srv->queue.push_back(id);
