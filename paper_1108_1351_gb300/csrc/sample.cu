@@ -237,12 +237,12 @@ __global__ void __launch_bounds__(kSampleThreads) sample_small_kernel(unsigned l
     sample_block(seed, n, m, k, subset, pos, tmp);
 }
 
-// Keys (n rows and m of the subset) up to which one CTA draws: its nine passes over them
-// take 25 us at n = 20,000, m = 2,000 and grow with their number; the 35 launches
-// and the read-back of the other way take about 250 us however few there are.  (A
-// whole kmeans2_sample call: 67 us at 3,600 keys, 110 at 3,000 with k = 512, 337 at
-// 130,000, against 312-320 the other way for 137,000 to a million keys.)
-constexpr long long kSampleSmall = 1 << 17;
+// Keys (n rows and m of the subset) up to which one CTA draws: its nine passes over
+// them grow with their number; the 35 launches and the read-back of the other way
+// take about 300 us however few there are.  A kmeans2_sample call, one CTA / the other
+// way, us: 22,000 keys 100 / 304, 66,000 172 / 300, 99,000 236 / 299, 120,000 (n = m)
+// 283 / 300, 121,000 271 / 300, 130,000 (n = m) 308 / 300, with k = 3,000 567 / 562.
+constexpr long long kSampleSmall = 120000;
 
 }  // namespace
 
