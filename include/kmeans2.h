@@ -135,9 +135,14 @@ typedef struct kmeans2_options {
                                    NULL for the random draw of the Algorithm */
     int32_t start_stage;        /* with init_centers: 0 = run both stages from them,
                                    1 = skip the fast stage (resume a slow stage) */
-    int32_t use_graph;          /* 1 (default when options are NULL): run each stage
-                                   loop as one CUDA graph with a device-side while
-                                   loop; 0: one host round trip per iteration.
+    int32_t use_graph;          /* 1 (default when options are NULL): run a stage's
+                                   iterations as one CUDA graph with a device-side
+                                   while loop, after its first one (screened and
+                                   16-bit forms) or, where n k d <= 2e9 in the FP32
+                                   form, its first twelve, which run from the host;
+                                   0: run them from the host: several queued ahead
+                                   of each read-back where n k d <= 2e9 (FP32
+                                   form), else one round trip per iteration.
                                    Fits meant to run side by side on several
                                    streams should use 0: on GB300 a second
                                    while-graph waits for a running one to end */

@@ -6,8 +6,10 @@
 // One stage = stage_init, then per iteration: assign (fused distance, argmin,
 // exact sums) -> recheck (FP64 near ties) -> finalize (means, movement, J,
 // loop control).  With use_graph the iteration body is captured once into the
-// body of a CUDA-graph WHILE node whose condition finalize sets on the device,
-// so a whole stage is one graph launch with no host round trip per iteration.
+// body of a CUDA-graph WHILE node whose condition finalize sets on the device, so
+// the iterations are one graph launch with no host round trip each; the first ones
+// of a small stage, and all of them without use_graph, are queued ahead of the
+// read-back that ends the stage.
 #include <algorithm>
 #include <cfloat>
 #include <chrono>
@@ -545,15 +547,15 @@ int run_loop_host(const float* X, long long n, int d, Workspace& w, int* labels,
 
 // Iterations queued ahead of the read-back that says whether the stage is done:
 // what is queued behind the last one returns at once (kErrStopped).  For short
-// iterations, where a while-graph costs more to build than the stage to run and a
-// read-back per iteration as much as the iteration.  out: the final state;
-// publish: device buffer that receives the centers before the read-back, or null.
-int run_loop_queued(const float* X, long long n, int d, Workspace& w, int* labels, int max_iter,
+// iterations, where a read-back per iteration costs as much as the iteration.
+// most: iterations at most; out: the state after them; publish: device buffer that
+// receives the centers before the read-back, or null.
+int run_loop_queued(const float* X, long long n, int d, Workspace& w, int* labels, int most,
                     cudaStream_t s, int sm_count, StageState& out, double* publish)
 {
     int queued = 0, chunk = 4;
     for (;;) {
-        const int b = std::min(chunk, max_iter - queued);
+        const int b = std::min(chunk, most - queued);
         for (int i = 0; i < b; ++i)
             KM2_TRY(launch_iteration(X, n, d, w, labels, 0ull, 0, 1, s, sm_count));
         queued += b;
@@ -561,17 +563,34 @@ int run_loop_queued(const float* X, long long n, int d, Workspace& w, int* label
         KM2_CUDA(cudaMemcpyAsync(&out, w.st, sizeof(StageState), cudaMemcpyDeviceToHost, s));
         KM2_CUDA(cudaStreamSynchronize(s));
         review_screen(w, d, out, n, out.iter);
-        if (out.error || out.done || queued >= max_iter) break;
+        if (out.error || out.done || queued >= most) break;
         chunk = std::min(2 * chunk, 32);
     }
     if (out.error == kErrStopped) out.error = 0;
     return KMEANS2_OK;
 }
 
-// n k d of an iteration up to which the queued loop runs it (at most ~60 us on the
-// CUDA cores, ~20 through the screen; building and starting a while-graph takes
-// ~150 us per stage).
+// n k d of an iteration up to which the queued loop starts a stage, and the iterations
+// after which a long stage goes on as a while-graph (use_graph).  A graph takes some
+// 60 us to build and start and then 3 us less per iteration; a queued chunk ends with
+// up to 31 passes that return at once, 5 us each.  Fits, us, queued to the end /
+// graph from the first iteration / graph after 12: 300,000 x 2, k = 4, 4 + 4 iterations
+// 620 / 710 / 620, 29 + 27 2430 / 1965 / 2100; 500,000 x 8, k = 32, 38 + 60 4000 / 3575 /
+// 3650; 1e7 x 12, k = 16, 60 + 60 13340 / 13220 / 13285; 5e7 x 2, k = 4, 6 + 3 5230 / 5212 /
+// 5227: at 2e9 the loops are within 1 % of one another, and host-driven is 10 % behind.
+// Debug builds take the limit from KMEANS2_DEBUG_QUEUED_WORK when that is set, so that
+// tests reach the other loops with small data.
 constexpr double kQueuedWork = 2.0e9;
+constexpr int kQueuedBeforeGraph = 12;
+
+double queued_work()
+{
+#ifdef KM2_DEBUG_CHECKS
+    const char* v = std::getenv("KMEANS2_DEBUG_QUEUED_WORK");
+    if (v && *v) return std::strtod(v, nullptr);
+#endif
+    return kQueuedWork;
+}
 
 int map_stage_error(int err)
 {
@@ -612,17 +631,20 @@ int run_stage(const float* X, long long n, int d, Workspace& w, int* labels, dou
     bool finished = false, have_out = false;
     int remaining = max_iter;
     if (w.form == KMEANS2_PRECISION_FP32 && !prof &&
-        (max_iter == 1 || (double)n * w.c.k * d <= kQueuedWork)) {
-        KM2_TRY(run_loop_queued(X, n, d, w, labels, max_iter, s, sm_count, out, publish));
-        finished = have_out = true;
-        if (published) *published = publish != nullptr;
+        (max_iter == 1 || (double)n * w.c.k * d <= queued_work())) {
+        const bool then_graph = use_graph && max_iter >= 3 * kQueuedBeforeGraph;
+        KM2_TRY(run_loop_queued(X, n, d, w, labels, then_graph ? kQueuedBeforeGraph : max_iter, s,
+                                sm_count, out, publish));
+        finished = have_out = out.error || out.done;
+        if (published) *published = finished && publish != nullptr;
+        remaining = max_iter - out.iter;
     } else if (max_iter == 1 && !prof && !use_graph) {
         // one iteration: its end is read with the final state
         KM2_TRY(launch_iteration(X, n, d, w, labels, 0ull, 0, 0, s, sm_count));
         finished = true;
     }
     probe16 = probe16 && w.form == KMEANS2_PRECISION_FP16;
-    if (!finished && (probe16 || (use_graph && !prof && screened(X, d, w)))) {
+    if (!finished && (probe16 || (w.first_pass && use_graph && !prof && screened(X, d, w)))) {
         // one iteration from the host, whose state says how the rest of the stage
         // runs (every form decides each row exactly, so a switch changes no
         // result): without the screen if that left too many rows open, in the
