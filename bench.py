@@ -266,13 +266,14 @@ def select_loop_ceiling(dev, stream, peak):
     return res
 
 
-def roofline_of(form: str, d: int, k: int, prof, clk, p32=None, requested: str = "fp32"):
+def roofline_of(form: str, d: int, k: int, prof, clk, p32=None, screened: int = 0):
     """Roofline entry of the distance kernel the fit ran (the dominant kernel):
     algorithmic FLOP = 2 N k d per launch (the cross term only), achieved =
     their sum over the profiled launches / their summed CUDA-event time.  The
     CUDA-core forms are measured against the FP32 FMA peak of this GPU
-    (fp32_peak, when given) with the unit-count figure beside it.  Under AUTO the
-    FP32 form of 8 <= d <= 128 runs the tensor-core screen (assign_mma_ring),
+    (fp32_peak, when given) with the unit-count figure beside it.  `screened`: the
+    profiled launches that went through the tensor-core screen
+    (kmeans2_screen_passes); where most did, the kernel is assign_mma_ring,
     which reads X once per pass: below k / 2 flop per byte = the tensor / HBM
     balance its floor is the copy bandwidth."""
     peaks, src = _peaks()
@@ -308,12 +309,14 @@ def roofline_of(form: str, d: int, k: int, prof, clk, p32=None, requested: str =
                            f"{sm_max:.0f} MHz ({src} max clock)")
     hbm = peaks.get("hbm_gbs")
     tensor = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
-    if form == "fp32" and requested == "auto" and 8 <= d <= 128:
-        kernel = "assign_mma_ring"
+    if form == "fp32" and 2 * screened > prof.assign_launches:
+        dp = next(p for p in (8, 16, 32, 48, 64, 96, 128) if d <= p)
+        kernel = f"assign_mma_ring<{dp}>"
         if hbm and tensor and 0.5 * k * float(hbm) * 1e-3 < float(tensor):
             gbs = prof.assign_bytes / (prof.assign_ms * 1e-3) / 1e9 if prof.assign_ms > 0 else None
             return {"bound": "hbm", "kernel": kernel, "achieved": gbs, "peak": float(hbm),
-                    "unit": "GB/s", "frac": gbs / float(hbm) if gbs else None, "traffic": None,
+                    "unit": "GB/s", "frac": gbs / float(hbm) if gbs else None,
+                    "traffic": traffic_of(kernel, prof, d), "screened_launches": screened,
                     "peak_source": f"{src} hbm_gbs (copy)", "achieved_tflops": achieved,
                     "fp32_peak_tflops": peak,
                     "kernel_ms_avg": prof.assign_ms / max(1, prof.assign_launches),
@@ -336,13 +339,14 @@ def roofline_of(form: str, d: int, k: int, prof, clk, p32=None, requested: str =
 def traffic_of(kernel: str, prof, d: int):
     """DRAM bytes per launch of `kernel` from its committed ncu summary
     (profiles/<kernel>*.md lines 'traffic-per-point: <kernel> <bytes> <sha256 of
-    the kernel source>'), scaled by the points of an average timed launch; None
+    the kernel source>', 'dram-per-point:' for the screen), scaled by the points of an average timed launch; None
     when there is no summary or the kernel source changed since the capture."""
     import glob
     import hashlib
     base = kernel.split("<")[0]
     src = {"assign_small": "assign_fp32.cu", "assign_large": "assign_fp32.cu",
-           "assign_bf16": "assign_bf16.cu", "assign_tc32": "assign_tc32.cu"}.get(base)
+           "assign_bf16": "assign_bf16.cu", "assign_tc32": "assign_tc32.cu",
+           "assign_mma_ring": "assign_mma.cu"}.get(base)
     if not src or prof.assign_launches == 0:
         return None
     path = os.path.join(ROOT, "paper_1108_1351_gb300", "csrc", src)
@@ -355,7 +359,8 @@ def traffic_of(kernel: str, prof, d: int):
         with open(f) as fh:
             for ln in fh:
                 parts = ln.strip().strip("`").split()
-                if len(parts) == 4 and parts[0] == "traffic-per-point:" and parts[1] == kernel:
+                if len(parts) == 4 and parts[0] in ("traffic-per-point:", "dram-per-point:") and \
+                        parts[1] == kernel:
                     if parts[3] != sha:
                         return None
                     # assign_bytes counts 4 d bytes per point of every timed launch
@@ -525,10 +530,12 @@ def run_ours(args, cfg):
     # distance kernel on the call's stream), after the timed region
     prof = km.Profile()
     prng = torch.cuda.nvtx.range_start("profiled")   # the launch list's ncu range
+    screened = km.screen_passes()
     for _ in range(args.profile_fits):
         one(prof)
     torch.cuda.synchronize()
     torch.cuda.nvtx.range_end(prng)
+    screened = km.screen_passes() - screened
 
     # end to end through the same C-ABI call with HOST buffers
     e2e = None
@@ -587,7 +594,7 @@ def run_ours(args, cfg):
             dist.destroy_process_group()
         return 0
     r0 = results[-1]
-    roofline = roofline_of(r0.precision_used, d, k, prof, clk, p32, args.precision)
+    roofline = roofline_of(r0.precision_used, d, k, prof, clk, p32, screened)
     roofline["measured"] = (f"{args.profile_fits} profiled fits after the timed region, CUDA "
                             f"events around each launch of the distance kernel")
     if roofline.get("kernel") == "assign_small<8>":
@@ -1055,7 +1062,11 @@ def run_batched(args):
     probe = fp32_peak(dev, stream)
     p32 = probe["tflops"] if probe else derived
     ach = prof.assign_flops / (prof.assign_ms * 1e-3) / 1e12 if prof.assign_ms > 0 else None
-    roofline = {"bound": "alu", "kernel": "batch_assign<2> and batch_mma<DP> (all dimension classes)",
+    # the batched form screens jobs of d >= 8 (precision AUTO) and runs the others on
+    # CUDA cores, by dimension class
+    cls = lambda dd: next(p for p in (2, 4, 8, 16, 32, 64) if dd <= p)
+    kernels = sorted({(f"batch_mma<{cls(dd)}>" if dd >= 8 else f"batch_assign<{cls(dd)}>") for dd in dims})
+    roofline = {"bound": "alu", "kernel": ", ".join(kernels),
                 "achieved": ach, "peak": p32, "unit": "TFLOP/s",
                 "frac": ach / p32 if ach else None, "traffic": None,
                 "peak_source": ("measured: FP32 FMA probe on this GPU (%.1f TFLOP/s); derived "
