@@ -251,6 +251,14 @@ constexpr int kRecheckCache = 1024;     // pass-1 values kept per warp (k <= 102
 
 // Warps of the grid share the listed points (see recheck_warps), or blocks do when
 // there are many centers and no more points than warps (recheck_point_block).
+// More centers than kRecheckCache have two launches, of which one has work: kBlocks for
+// the points that blocks take, kLarge for those of warps (in one kernel the block form
+// is slower, n = 1e5, d = 100, k = 5000 3.2 -> 3.5 ms).  kBlocks keeps the code of kAll and
+// leaves it by a flag: without that code it is given 40 registers, fewer loads in
+// flight and 3.3 ms.
+enum RecheckKind { kAll, kBlocks, kLarge };
+constexpr int kOnlyBlocks = 2;          // in settles
+template <RecheckKind KIND>
 __global__ void __launch_bounds__(kRecheckThreads) recheck_kernel(const float* __restrict__ X, int d, Centers c,
                                int* __restrict__ labels, const int* __restrict__ list,
                                StageState* st, Accum acc, int settles)
@@ -261,18 +269,21 @@ __global__ void __launch_bounds__(kRecheckThreads) recheck_kernel(const float* _
     if (st->error) return;
     const long long nw = (long long)gridDim.x * W;
     if (c.k >= 256 && c.kpad <= W * kRecheckCache && st->recheck_count <= nw) {
-        const int count = st->recheck_count;
-        long long settled = 0;
-        for (int p = blockIdx.x; p < count; p += gridDim.x)
-            settled += recheck_point_block(X, d, c, labels, list[p], st, acc, cache, sm) ? 1 : 0;
-        if (settles && settled && threadIdx.x == 0)
-            atomicAdd(reinterpret_cast<unsigned long long*>(&st->rechecked_total),
-                      (unsigned long long)(-settled));
+        if constexpr (KIND != kLarge) {
+            const int count = st->recheck_count;
+            long long settled = 0;
+            for (int p = blockIdx.x; p < count; p += gridDim.x)
+                settled += recheck_point_block(X, d, c, labels, list[p], st, acc, cache, sm) ? 1 : 0;
+            if ((KIND == kBlocks ? settles & 1 : settles) && settled && threadIdx.x == 0)
+                atomicAdd(reinterpret_cast<unsigned long long*>(&st->rechecked_total),
+                          (unsigned long long)(-settled));
+        }
         return;
     }
+    if (KIND == kBlocks && (settles & kOnlyBlocks)) return;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    recheck_warps(X, d, c, labels, list, st, acc, gw, nw, cache + (threadIdx.x >> 5) * kRecheckCache,
-                  kRecheckCache, settles);
+    recheck_warps<KIND == kLarge>(X, d, c, labels, list, st, acc, gw, nw,
+                                  cache + (threadIdx.x >> 5) * kRecheckCache, kRecheckCache, settles);
 }
 
 }  // namespace
@@ -381,8 +392,16 @@ int launch_publish_centers(const StageState* st, const double* c64, long long co
 int launch_recheck(const float* X, int d, const Centers& c, int* labels, const int* list,
                    StageState* st, const Accum& acc, int settles, cudaStream_t s, int sm_count)
 {
-    ++g_launches;
-    recheck_kernel<<<sm_count * 4, kRecheckThreads, 0, s>>>(X, d, c, labels, list, st, acc, settles);
+    const int grid = sm_count * 4;
+    if (c.kpad <= kRecheckCache) {
+        ++g_launches;
+        recheck_kernel<kAll><<<grid, kRecheckThreads, 0, s>>>(X, d, c, labels, list, st, acc, settles);
+    } else {
+        g_launches += 2;
+        recheck_kernel<kBlocks><<<grid, kRecheckThreads, 0, s>>>(X, d, c, labels, list, st, acc,
+                                                                settles | kOnlyBlocks);
+        recheck_kernel<kLarge><<<grid, kRecheckThreads, 0, s>>>(X, d, c, labels, list, st, acc, settles);
+    }
     KM2_CUDA(cudaGetLastError());
     return KMEANS2_OK;
 }

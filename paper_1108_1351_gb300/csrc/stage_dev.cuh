@@ -643,6 +643,115 @@ static __device__ __forceinline__ bool recheck_point(const float* __restrict__ X
     return recheck_point_nq<4>(X, d, c, labels, i, st, acc, cache, cache_cap);
 }
 
+// The same for more centers than the cache holds values of: pass 2 forms the values
+// again, once, and the candidates' indices (ascending) take the cache, cap of them;
+// a point with more is compared in a third pass.  (Counting the candidates and then
+// comparing them formed the values three or four times: a step of 1e6 x 2, k = 20,000 at
+// an offset of 100 74.6 ms, now 45.1; 5e5 x 17, k = 1,025 3.3 and 2.5.)
+static __device__ __forceinline__ bool recheck_point_large(const float* __restrict__ X, int d, const Centers& c,
+                                                        int* __restrict__ labels, int i, StageState* st,
+                                                        const Accum& acc, int* cand, int cap)
+{
+    constexpr int NQ = 4, STEP = 32 * NQ;
+    const int k = c.k, lane = threadIdx.x & 31;
+    const float* x = X + (long long)i * d;
+    const int old = (st->mode == kModeDelta) ? labels[i] : -1;
+    float x2 = 0.0f;
+    for (int t = lane; t < d; t += 32) { float v = __ldg(x + t); x2 = fmaf(v, v, x2); }
+    for (int o = 16; o; o >>= 1) x2 += __shfl_xor_sync(0xffffffffu, x2, o);
+    // recheck_d without its vector loads' tests, which outweigh the products for d < 4
+    auto value = [&](int j0, float (&a)[NQ]) {
+        if (d >= 4) {
+            recheck_d<NQ>(x, d, c, j0, a);
+            return;
+        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) a[q] = c.cnorm[j0 + 32 * q];
+#pragma unroll 1
+        for (int t = 0; t < d; ++t) {
+            const float xm2 = -2.0f * __ldg(x + t);
+            const float* row = c.c32t + (long long)t * c.kpad + j0;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) a[q] = fmaf(xm2, row[32 * q], a[q]);
+        }
+    };
+    float b1 = INFINITY;
+    // (kpad is a multiple of STEP; padding centers read as FLT_MAX)
+    for (int j0 = lane; j0 < c.kpad; j0 += STEP) {
+        float a[NQ];
+        value(j0, a);
+        b1 = fmin3(b1, a[0], a[1]);
+        b1 = fmin3(b1, a[2], a[3]);
+    }
+    for (int o = 16; o; o >>= 1) b1 = fminf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
+    const float lim = b1 + tie_kappa(d) * (2.0f * st->cmax2 + x2) * 1.0009765625f + tie_abs(d + 1);
+    int ncand = 0;
+    for (int j0 = lane; j0 < c.kpad; j0 += STEP) {
+        float a[NQ];
+        value(j0, a);
+        if (!__any_sync(0xffffffffu, a[0] <= lim || a[1] <= lim || a[2] <= lim || a[3] <= lim)) continue;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const bool near = j0 + 32 * q < k && a[q] <= lim;
+            const unsigned m = __ballot_sync(0xffffffffu, near);
+            const int at = ncand + __popc(m & lanemask_lt());
+            if (near && at < cap) cand[at] = j0 + 32 * q;
+            ncand += __popc(m);
+        }
+    }
+    __syncwarp();
+    int bj = INT_MAX;
+    bool decided = false;
+    const bool single = ncand == 1 && lim < FLT_MAX;
+    if (single) {
+        bj = cand[0];
+        decided = true;
+    } else if (d > 16 && ncand <= cap && ncand * (2 * ((d + 31) / 32) + 5) < 2 * d) {
+        double s1 = DBL_MAX, s2 = DBL_MAX;
+        for (int e = 0; e < ncand; ++e) {
+            const int j = cand[e];
+            const double p = recheck_lanes_f64(x, d, c, j);
+            if (p < s1) { s2 = s1; s1 = p; bj = j; }
+            else if (p < s2) s2 = p;
+        }
+        decided = recheck_ranked(s1, s2, d);
+    }
+    if (!decided) {
+        double best = DBL_MAX;
+        bj = INT_MAX;
+        auto compare = [&](int j) {
+            const double* cj64 = c.c64 + (long long)j * d;
+            double a2 = 0.0;
+            for (int t = 0; t < d; ++t) {
+                double e = (double)__ldg(x + t) - cj64[t];
+                a2 = fma(e, e, a2);
+            }
+            if (a2 < best || (a2 == best && j < bj)) { best = a2; bj = j; }
+        };
+        if (ncand <= cap) {
+            for (int e = lane; e < ncand; e += 32) compare(cand[e]);
+        } else {
+            for (int j0 = lane; j0 < k; j0 += STEP) {
+                float a[NQ];
+                value(j0, a);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q)
+                    if (j0 + 32 * q < k && a[q] <= lim) compare(j0 + 32 * q);
+            }
+        }
+        unsigned long long bb = (unsigned long long)__double_as_longlong(best);
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bb, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+            if (ob < bb || (ob == bb && oj < bj)) { bb = ob; bj = oj; }
+        }
+    }
+    __syncwarp();   // every lane has read the old label and the candidates
+    if (bj != old && label_ok(bj, k, st) && old_label_ok(old, k, st))
+        recheck_move(x, d, acc, labels, i, old, bj, st->scaleF, lane, 32);
+    return single;
+}
+
 // A block of 256 threads per point, for many centers and few listed points: the
 // warps share the centers, so a point waits for an eighth of the loads (one warp
 // per point is bound by their latency: k = 1024, d = 128 reads 512 KB of centers).
@@ -756,10 +865,11 @@ static __device__ bool recheck_point_block(const float* __restrict__ X, int d, c
     return single;
 }
 
-// One warp per listed point (recheck_point); warps w0, w0 + wstride, ... of
-// the caller each take the listed points.
+// One warp per listed point; warps gw, gw + nw, ... of the caller each take the
+// listed points.  cache: cache_cap floats per warp (LARGE: kpad is above it).
 // settles: the list comes from a screen that leaves rows to the FP32 pass here;
 // those it decides alone do not count as rechecked in FP64.
+template <bool LARGE>
 static __device__ void recheck_warps(const float* __restrict__ X, int d, Centers c,
                                      int* __restrict__ labels, const int* __restrict__ list,
                                      StageState* st, Accum acc, long long gw, long long nw,
@@ -767,8 +877,13 @@ static __device__ void recheck_warps(const float* __restrict__ X, int d, Centers
 {
     const int count = st->recheck_count;
     long long settled = 0;
-    for (long long w = gw; w < count; w += nw)
-        settled += recheck_point(X, d, c, labels, list[w], st, acc, cache, cache_cap) ? 1 : 0;
+    for (long long w = gw; w < count; w += nw) {
+        if constexpr (LARGE)
+            settled += recheck_point_large(X, d, c, labels, list[w], st, acc, reinterpret_cast<int*>(cache),
+                                           cache_cap) ? 1 : 0;
+        else
+            settled += recheck_point(X, d, c, labels, list[w], st, acc, cache, cache_cap) ? 1 : 0;
+    }
     if (settles && settled && (threadIdx.x & 31) == 0)
         atomicAdd(reinterpret_cast<unsigned long long*>(&st->rechecked_total),
                   (unsigned long long)(-settled));
