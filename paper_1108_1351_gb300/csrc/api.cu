@@ -1016,9 +1016,9 @@ int kmeans_step_noalloc(const float* X, int64_t n, int32_t d, int32_t k,
     KM2_TRY(noalloc_scratch(&arena));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DeviceScratch ws(s, arena, kNoAllocBytes);
-    // The CUDA-core form: its scratch (the near-tie list, n ints, plus O(k d)
-    // center copies and sums) fits the array over the whole stated range; the
-    // tensor-core forms would also need a per-call copy of X (about 4 n d
+    // The FP32 form, screened as under AUTO: its scratch (the near-tie list, n ints,
+    // plus O(k d) center copies and sums) fits the array over the whole stated range;
+    // the tensor-core forms would also need a per-call copy of X (about 4 n d
     // bytes for BF16), which it cannot hold.  Every form returns the same
     // labels, centers and J.
     Workspace w;
@@ -1306,7 +1306,7 @@ int kmeans2_fit_streamed(const float* X, int64_t n, int32_t d, int32_t k, double
     if (o.start_stage != 0 && o.start_stage != 1) return KMEANS2_ERR_INVALID;
     if (o.start_stage == 1 && !o.init_centers) return KMEANS2_ERR_INVALID;
     if (o.precision != KMEANS2_PRECISION_FP32 && o.precision != KMEANS2_PRECISION_AUTO) {
-        set_last_error_text("kmeans2_fit_streamed runs the CUDA-core FP32 form only");
+        set_last_error_text("kmeans2_fit_streamed runs the FP32 form only");
         return KMEANS2_ERR_UNSUPPORTED;
     }
     if (chunk_points < 0) {

@@ -9,7 +9,9 @@
 // ring of cp.async stages in shared memory (rows as they lie in X, and the old
 // labels); the centers' fragments stay in shared memory for the whole launch.
 // Warps never wait for one another except to flush the partial sums.  Shapes
-// whose centers do not fit beside the rings go to the CUDA-core kernels.
+// whose centers do not fit beside the rings go to the CUDA-core kernels, and so do the
+// later passes of a stage whose first ones leave too many rows open (review_screen):
+// data far from the origin, whose bound grows with ||x||^2.
 //
 // What bounds it: instruction issue and register ports for d <= 16 (at d = 8, k =
 // 32 it reads 3.1 TB/s), the legacy tensor rate (an MMA of 16 x 8 x 16 takes 8

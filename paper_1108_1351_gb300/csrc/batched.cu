@@ -9,12 +9,15 @@
 //   batch_recheck     FP64 re-decision of the near ties of every running job
 //                     as one flat list (a scan of the jobs' flagged counts,
 //                     then one warp per flagged point over the whole GPU)
-//   batch_finalize    one CTA per job: means, movement, J, stop test, and the
-//                     switch from the fast to the slow stage (Section 2)
+//   batch_finalize    several CTAs per job while jobs leave SMs idle: means, movement,
+//                     J, stop test, the switch from the fast to the slow stage
+//                     (Section 2), and from the screen to the CUDA cores
 //   batch_control     sets the graph's while condition: any job still running
-// and the loop is captured once as a CUDA graph with a device-side WHILE node.
-// The arithmetic of every step is the single-fit arithmetic (stage_dev.cuh,
-// the same packed-key top-2, near-tie bound and exact sums).  A tile shape in
+// and the loop is captured as a CUDA graph with a device-side WHILE node (after a
+// first iteration from the host where jobs may leave the screen).
+// The arithmetic of every step is the single-fit arithmetic (stage_dev.cuh and
+// mma_dev.cuh; batch_assign: the packed-key top-2 and near-tie bound of
+// assign_fp32.cu; the same exact sums).  A tile shape in
 // which several lanes share a point adds that point's FP32 terms in another
 // order, which the bound covers, so every decision, and with it each job's
 // result, equals kmeans2_fit on that job alone.
