@@ -1006,23 +1006,23 @@ std::mutex g_tune_mu;
 // dimension class -> (tile shape, tiles per work item)
 std::map<int, std::pair<TileShape, int>> g_tuned;
 
-// Resident CTAs per SM of the screen's kernel for a dimension class.
-int mma_ctas(int dc) { return dc <= 16 ? BMma<16>::MINB : 1; }
-
-// Tiles per work item of the screen's kernel: as many as leave each CTA four items or
-// more, at most eight.  The centers of a job are loaded per item, so long lists
-// take large items, and short ones would leave CTAs idle with them.  ms a call with
-// items of 1, 2, 4, 8 tiles: 64 instances (n 1e3 .. 1e6, d 2 .. 64) 59.0, 55.9, 54.2, 56.5
-// (by this rule 55.1); 40 jobs of 1e3 .. 1.5e6 x 64 261, 246, 236, 235; 1e6 x 8 8.07, 8.68,
-// 9.53, 10.8; 1e6 x 16 9.24, 9.87, 11.1, 12.6.  A rule on the call's own sizes: timed once per
-// process and class, the last ran with 4 tiles after a batch of many jobs.
-int mma_tiles_per_item(const std::vector<int>& members, const std::vector<long long>& n, long long ctas)
+// Tiles per work item of the screen's kernel.  The centers of a job are loaded per
+// item, so long lists take large items; short ones would leave SMs idle with them.
+// ms a call with items of 1, 2, 4, 8 tiles, the class's tiles per SM in brackets: d 64,
+// k 100 [6.4] 18.1, 19.6, 21.0, 24.5; d 8, k 100 [6.4] 8.07, 8.68, 9.53, 10.8; d 32, k 100 [6.4]
+// 11.8, 12.2, 12.8, 14.4, but 16 jobs [5.2] 6.34, 6.16, 7.08, 8.23 and in mixed batches
+// [1.8] 20.2, 19.0 and [7.2] 36.5, 34.5, 36.1, 39.5: a tile is only two steps of that
+// kernel's 16 warps; eight jobs [21] d 32 22.6, 20.9, 20.6, d 8 12.2, 11.9, 12.4; 40 jobs [135]
+// d 64 261, 246, 236, 235, d 8 58.3, 52.7, 50.4, 50.4.  A rule on the call's own sizes: timed
+// once per process and class, 1e6 x 16 ran with 4 tiles (11.1 ms, 9.2 with 1) after a
+// batch of many jobs.
+int mma_tiles_per_item(int dc, const std::vector<int>& members, const std::vector<long long>& n, int sm_count)
 {
     long long tiles = 0;
     for (int j : members) tiles += (n[j] + kTile - 1) / kTile;
-    int p = 8;
-    while (p > 1 && tiles < 4 * p * ctas) p /= 2;
-    return p;
+    const double per_sm = (double)tiles / sm_count;
+    if (dc <= 16) return per_sm >= 120.0 ? 8 : per_sm >= 30.0 ? 4 : per_sm >= 7.5 ? 2 : 1;
+    return per_sm >= 28.0 ? 8 : per_sm >= 14.0 ? 4 : per_sm >= (dc <= 32 ? 1.0 : 7.0) ? 2 : 1;
 }
 
 // Six dimension classes, each split in jobs the screen takes and others, and for the
@@ -1283,7 +1283,7 @@ extern "C" int kmeans2_fit_batched(int32_t count, const kmeans2_job* jobs, kmean
             const TileShape core_shape = shape;
             if (screened) {
                 shape = TileShape{kMmaShape, 0};
-                tpi = mma_tiles_per_item(kv.second, nvec, (long long)ws.sm_count * mma_ctas(ci.dc));
+                tpi = mma_tiles_per_item(ci.dc, kv.second, nvec, ws.sm_count);
                 settle32 = settle32 || ci.dc == 32;
                 settle64 = settle64 || ci.dc == 64;
             }
