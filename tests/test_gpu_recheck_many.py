@@ -76,7 +76,7 @@ def test_screened_rows_settle_among_many_centers():
 def test_many_ties_form_the_values_twice():
     """A point's values over all centers are formed twice, also where they are not
     kept (three or four times took 1.65 times as long here).  Against the same points
-    and centers with d = 1,024 centers, whose values are kept: per center no more than
+    with 1,024 centers, whose values are kept: per center no more than
     twice the time."""
     n = 300_000
     X = synth.iso_gaussian_mixture(n, 2, 50, 7, device="cuda") + 1000.0
